@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kSymThreads, 6) k_sym(const SymArgs a)
 
         /* ---- 1. the rank's next operation: the seeded half first, it needs nothing from anybody ---- */
         float z0[NE];
-        if (unit0 < nunits) unit_noise<DT, NW>(g, first, unit0 * NE, n, z0);
+        if (unit0 < nunits) unit_noise<DT, NW>(g, first, unit0 * NE, z0);
         if (MODE == SIFAR_BARRIER_ONESHOT || a.w.delay_max_ns != 0u) {
             if (threadIdx.x < 32) {
                 bool ok = true;
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(kSymThreads, 6) k_sym(const SymArgs a)
                 unit_combine<DT, NW>(g, first, prev_mem, u * NE, n, z0, w, n_io);
             } else {
                 float z[NE];
-                unit_noise<DT, NW>(g, first, u * NE, n, z);
+                unit_noise<DT, NW>(g, first, u * NE, z);
                 unit_combine<DT, NW>(g, first, prev_mem, u * NE, n, z, w, n_io);
             }
             if (spec) store_slot(dst, u, w[0], w[1], w[2], e);
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kSymvThreads, 4) k_symv(const SymArgs a)
 
         /* ---- 1. the rank's operation ---- */
         float z0[NE];
-        if (worker && unit0 < nunits) unit_noise<DT, NW>(g, first, unit0 * NE, n, z0);
+        if (worker && unit0 < nunits) unit_noise<DT, NW>(g, first, unit0 * NE, z0);
         if (a.w.delay_max_ns != 0u) {
             if (threadIdx.x == 0) spin_ns(gen_delay_ns(a.w, rank, t));       /* seeded skew between the ranks */
             __syncthreads();
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kSymvThreads, 4) k_symv(const SymArgs a)
                     unit_combine<DT, NW>(g, first, prev_mem, u * NE, n, z0, w, n_io);
                 } else {
                     float z[NE];
-                    unit_noise<DT, NW>(g, first, u * NE, n, z);
+                    unit_noise<DT, NW>(g, first, u * NE, z);
                     unit_combine<DT, NW>(g, first, prev_mem, u * NE, n, z, w, n_io);
                 }
                 st_slot(dst + u, make_uint4(w[0], w[1], w[2], w[3]));

@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
     {
         const Gen g0 = make_gen(a.w, a.rank, t_ahead);
         if (tid * EPU < (size_t)a.n) {
-            unit_noise<DT, NW>(g0, t_ahead == 1u, tid * EPU, (size_t)a.n, z0);
+            unit_noise<DT, NW>(g0, t_ahead == 1u, tid * EPU, z0);
 #pragma unroll
             for (int k = 0; k < EPU; ++k) asm volatile("" : "+f"(z0[k]));     /* keep it above the wait */
         }
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
                that need more units per thread than that are far beyond the decode payloads) */
             float z0[NE];
             if (unit0 < nunits) {
-                unit_noise<DT, NW>(g, first, unit0 * EPU, n, z0);
+                unit_noise<DT, NW>(g, first, unit0 * EPU, z0);
                 /* pin the values here: without this the compiler sinks the arithmetic below the wait */
 #pragma unroll
                 for (int k = 0; k < NE; ++k) asm volatile("" : "+f"(z0[k]));
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
                 const size_t u = unit0 + (size_t)k * kChainThreads;
                 if (u >= nunits) break;
                 float z[NE];
-                unit_noise<DT, NW>(g, first, u * EPU, n, z);
+                unit_noise<DT, NW>(g, first, u * EPU, z);
 #pragma unroll
                 for (int q = 0; q < NE; ++q) s_z[k - 1u][q][threadIdx.x] = z[q];
             }
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
 #pragma unroll
                     for (int q = 0; q < NE; ++q) z[q] = s_z[k - 1u][q][threadIdx.x];
                 } else {
-                    unit_noise<DT, NW>(g, first, u * EPU, n, z);
+                    unit_noise<DT, NW>(g, first, u * EPU, z);
                 }
                 if (by_flag) {
                     unit_combine<DT, NW>(g, first, prev, u * EPU, n, z, w, n_io);
