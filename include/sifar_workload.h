@@ -65,8 +65,9 @@ typedef struct sifar_chain sifar_chain;   /* opaque */
 typedef enum {
     SIFAR_CHAIN_STREAMS    = 0,  /* P producer streams + one reducer stream, events for the result dependency   */
     SIFAR_CHAIN_GRAPH      = 1,  /* the same topology captured once into a CUDA graph and replayed              */
-    SIFAR_CHAIN_PERSISTENT = 2   /* one cooperative kernel: reducer CTAs and P groups of producer CTAs that talk
-                                    only through flags / tags in memory, for all steps of a run                 */
+    SIFAR_CHAIN_PERSISTENT = 2   /* one kernel: reducer CTAs and P groups of producer CTAs that talk only through
+                                    flags / tags in memory, for all steps of a run (small grids: in the shared
+                                    memory of one thread-block cluster per chunk)                               */
 } sifar_chain_impl;
 
 /* Fourth "mode", chains only: no all-reduce at all; each rank's next operation consumes its own
@@ -133,9 +134,9 @@ int sifar_chain_chunks(sifar_chain *chain);
 
 /*
  * How a PERSISTENT chain is laid out, as the host chose it and as the kernel of the last run saw it (synchronizes
- * the device): out[0] chunks, [1] units per thread and step, [2] CTAs, [3] 1 = the CTAs of a chunk are launched as
- * one thread-block cluster, [4] 1 = results reach the next step's producers in tagged words (0 = ready flag per
- * chunk, or done flags with both barriers); from the kernel: [5] the role layout it used (1 = clustered), [6] CTAs
+ * the device): out[0] chunks, [1] units per thread and step, [2] CTAs, [3] 1 = the CTAs of a chunk are one
+ * thread-block cluster and meet in its shared memory, [4] 1 = results reach the next step's producers unit by unit,
+ * in tagged words or counted stores (0 = ready flag per chunk, or done flags with both barriers); from the kernel: [5] the role layout it used (1 = clustered), [6] CTAs
  * per cluster as the hardware reported them (1 without clusters), [7] the form of the hand-over it was built for.
  * Before the first run [5..7] are 0.
  */
@@ -172,7 +173,7 @@ int sifar_chain_destroy(sifar_chain *chain);
  * The same decode step with P readers: every emulated rank runs its own next
  * operation AND its own pull-and-reduce, as every GPU does in the paper's system
  * (Section 3.1; the oneshot pseudocode of Section 4.2), and keeps its own copy of
- * every result.  One cooperative kernel of P x C CTAs; CTA (r, c) computes chunk c
+ * every result.  One kernel of P x C CTAs; CTA (r, c) computes chunk c
  * of rank r's partial from chunk c of rank r's copy of the previous result, stores
  * it, pulls chunk c of all P partials (its own included) and reduces it.  Ranks
  * are ordered against each other by the mode's protocol alone (P x P arrival and

@@ -46,7 +46,7 @@
 #ifdef SIFAR_SLOT_S8X2
 #error "the decode-step chains are written for the default slot format; the fallback format is built for libsifar only"
 #endif
-#include "sifar_reduce.cuh"
+#include "sifar_chain.cuh"
 #include "sifar_gen.cuh"
 #include "sifar_workload.h"
 
@@ -59,45 +59,6 @@ constexpr int kSymFlagval = SIFAR_SYMCHAIN_FLAGVAL;
 constexpr int kSymFlagvalOrdered = SIFAR_SYMCHAIN_FLAGVAL_ORDERED;
 constexpr int kSymUnchecked = SIFAR_SYMCHAIN_UNCHECKED;
 constexpr int kSymvThreads = kSymThreads + 32;       /* the payload warps and one validation warp */
-
-/* Flags of one chunk: what the P CTAs that own it tell each other. */
-struct __align__(128) SymFlags {
-    uint32_t arrive[2][8];          /* [parity][rank]: chunk of the rank's partial of call e stored      */
-    uint32_t pad0[16];
-    uint32_t done[8];               /* [rank]: the rank's reader has finished reading the chunk of call e */
-    uint32_t pad1[24];
-};
-
-struct __align__(128) SymDev {
-    uint32_t exit_count;            /* CTAs that left the kernel (monotonic over runs) */
-    uint32_t pad[31];
-};
-
-struct SymArgs {
-    DevState *st;
-    int *host_status;
-    unsigned long long timeout_ns;
-    sifar_workload w;
-    unsigned long long n;
-    char *plain;                    /* [parity][rank] plain buffers */
-    unsigned long long plain_stride;
-    char *slots;                    /* [parity][rank] slot buffers  */
-    unsigned long long slot_stride;
-    char *rings;                    /* [rank][ring_len] result rows */
-    unsigned long long ring_stride;
-    uint32_t ring_len;
-    uint32_t e0;                    /* calls completed before this run */
-    uint32_t base_epoch;
-    uint32_t steps;
-    uint32_t C, K;
-    uint32_t exit_base;
-    PollShape poll;
-    SymDev *cs;
-    SymFlags *flags;                /* C */
-    unsigned long long *stamps;     /* [rank][chunk][warp][steps + 1] */
-    uint32_t *retry_marks;          /* [rank][steps]: 1 if the rank re-loaded a slot in that step */
-    unsigned long long *rank_retries; /* [P] cumulative (rank, step) pairs with a re-load */
-};
 
 template <int DT, int P, int MODE>
 __global__ void __launch_bounds__(kSymThreads, 6) k_sym(const SymArgs a)
@@ -294,29 +255,7 @@ __global__ void __launch_bounds__(kSymThreads, 6) k_sym(const SymArgs a)
         s_ok = (left == a.exit_base + gridDim.x && !no_ar && ld_relaxed_u32(&st->status) == 0u);
     }
     __syncthreads();
-    if (s_ok) {
-        if (spec) {
-            unsigned long long any_steps = 0;
-            for (uint32_t s = threadIdx.x; s < a.steps; s += kSymThreads) {
-                uint32_t any = 0;
-                for (int r = 0; r < P; ++r) {
-                    const uint32_t m = ld_relaxed_u32(&a.retry_marks[(size_t)r * a.steps + s]);
-                    if (m) {
-                        atomicAdd(&a.rank_retries[r], 1ull);
-                        st_relaxed_u32(&a.retry_marks[(size_t)r * a.steps + s], 0u);
-                    }
-                    any |= m;
-                }
-                any_steps += any ? 1ull : 0ull;
-            }
-            if (any_steps) atomicAdd(&st->stats[kStatCallsWithRetry], any_steps);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            atomicAdd(&st->stats[kStatCalls], (unsigned long long)a.steps);
-            st_release_u32(&st->epoch, a.e0 + a.steps);
-        }
-    }
+    if (s_ok) book_sym_run<P>(a, spec);
 }
 
 /*
@@ -479,27 +418,7 @@ __global__ void __launch_bounds__(kSymvThreads, 4) k_symv(const SymArgs a)
         s_ok = (left == a.exit_base + gridDim.x && ld_relaxed_u32(&st->status) == 0u);
     }
     __syncthreads();
-    if (s_ok) {
-        unsigned long long any_steps = 0;
-        for (uint32_t s = threadIdx.x; s < a.steps; s += kSymvThreads) {
-            uint32_t any = 0;
-            for (int r = 0; r < P; ++r) {
-                const uint32_t m = ld_relaxed_u32(&a.retry_marks[(size_t)r * a.steps + s]);
-                if (m) {
-                    atomicAdd(&a.rank_retries[r], 1ull);
-                    st_relaxed_u32(&a.retry_marks[(size_t)r * a.steps + s], 0u);
-                }
-                any |= m;
-            }
-            any_steps += any ? 1ull : 0ull;
-        }
-        if (any_steps) atomicAdd(&st->stats[kStatCallsWithRetry], any_steps);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            atomicAdd(&st->stats[kStatCalls], (unsigned long long)a.steps);
-            st_release_u32(&st->epoch, a.e0 + a.steps);
-        }
-    }
+    if (s_ok) book_sym_run<P>(a, true);
 }
 
 template <int DT, int P>
@@ -550,6 +469,7 @@ struct sifar_symchain {
     uint32_t C, K;
     int grid;
     bool clustered;                 /* the P CTAs of a chunk as one thread-block cluster (placement only) */
+    const void *cluster_kernel;     /* not NULL: the ranks of a chunk meet in the cluster's shared memory */
     SymDev *d_cs;
     SymFlags *d_flags;
     unsigned long long *d_stamps;
@@ -586,6 +506,8 @@ static int sym_setup(sifar_symchain *ch)
     if (!coop) { set_error("sifar_symchain_create: device lacks cooperative launch"); return SIFAR_ERR_CUDA; }
     const size_t units = (ch->mode == SIFAR_SPECULATIVE) ? slots_for(c->dtype, ch->n)
                                                          : (ch->n * elem_size(c->dtype) + 15) / 16;
+    const char *env_cluster = getenv("SIFAR_CHAIN_CLUSTER");
+    const bool clusters_allowed = !(env_cluster && atoi(env_cluster) == 0);
     int per_sm = 0;
     const int threads = sym_threads(ch->mode);
     SIFAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sym_kernel(ch), threads, 0));
@@ -599,8 +521,16 @@ static int sym_setup(sifar_symchain *ch)
     }
     ch->K = K; ch->C = (uint32_t)C; ch->grid = (int)(C * P);
     ch->clustered = false;
-    const char *env_cluster = getenv("SIFAR_CHAIN_CLUSTER");
-    if (!(env_cluster && atoi(env_cluster) == 0) && P >= 2) {
+    if (clusters_allowed) {
+        /* one unit per thread and every chunk resident: the ranks of a chunk meet in the cluster's shared memory */
+        const size_t chunks = (units + kSymThreads - 1) / kSymThreads;
+        const void *fn = sym_cluster_kernel(c->dtype, P, ch->mode);
+        if (cluster_fits(fn, P, chunks)) {
+            ch->cluster_kernel = fn;
+            ch->K = 1; ch->C = (uint32_t)chunks; ch->grid = (int)(chunks * (size_t)P);
+        }
+    }
+    if (clusters_allowed && !ch->cluster_kernel && P >= 2) {
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof cfg);
         cfg.gridDim = dim3((unsigned)ch->grid);
@@ -617,14 +547,14 @@ static int sym_setup(sifar_symchain *ch)
         if (err == cudaSuccess && (size_t)max_clusters >= C) ch->clustered = true;
         else cudaGetLastError();
     }
-    const size_t nstamps = (size_t)P * C * (kSymThreads / 32) * (ch->steps + 1);
+    const size_t nstamps = (size_t)P * ch->C * (kSymThreads / 32) * (ch->steps + 1);
     SIFAR_CUDA(cudaMalloc(&ch->d_cs, sizeof(SymDev)));
-    SIFAR_CUDA(cudaMalloc(&ch->d_flags, sizeof(SymFlags) * C));
+    SIFAR_CUDA(cudaMalloc(&ch->d_flags, sizeof(SymFlags) * ch->C));
     SIFAR_CUDA(cudaMalloc(&ch->d_stamps, sizeof(unsigned long long) * nstamps));
     SIFAR_CUDA(cudaMalloc(&ch->d_marks, sizeof(uint32_t) * P * ch->steps));
     SIFAR_CUDA(cudaMalloc(&ch->d_rank_retries, sizeof(unsigned long long) * kMaxRanks));
     SIFAR_CUDA(cudaMemset(ch->d_cs, 0, sizeof(SymDev)));
-    SIFAR_CUDA(cudaMemset(ch->d_flags, 0, sizeof(SymFlags) * C));
+    SIFAR_CUDA(cudaMemset(ch->d_flags, 0, sizeof(SymFlags) * ch->C));
     SIFAR_CUDA(cudaMemset(ch->d_stamps, 0, sizeof(unsigned long long) * nstamps));
     SIFAR_CUDA(cudaMemset(ch->d_marks, 0, sizeof(uint32_t) * P * ch->steps));
     SIFAR_CUDA(cudaMemset(ch->d_rank_retries, 0, sizeof(unsigned long long) * kMaxRanks));
@@ -693,7 +623,9 @@ extern "C" int sifar_symchain_run(sifar_symchain *ch, void *stream)
     void *params[] = {&a};
     const void *fn = sym_kernel(ch);
     cudaStream_t s = (cudaStream_t)stream;
-    if (ch->clustered) {
+    if (ch->cluster_kernel) {
+        SIFAR_CUDA(launch_clusters(ch->cluster_kernel, c->P, ch->C, s, params));
+    } else if (ch->clustered) {
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof cfg);
         cfg.gridDim = dim3((unsigned)ch->grid);

@@ -15,10 +15,12 @@
  *   SPECULATIVE     : take -> produce tagged slots -> load/validate/sum -> hand over
  *
  * where "hand over / take" is how a result reaches the next step's producers.  It
- * models ordinary same-GPU operator ordering and comes in two forms chosen by
- * size: tagged 16-byte stores polled by the thread that needs them (see
- * handoff_store), or, for grids whose polling threads would get in the way of the
- * stores they wait for, one result-ready flag per chunk.  With both barriers the
+ * models ordinary same-GPU operator ordering.  Small grids run as one thread-block
+ * cluster per chunk whose ranks meet in shared memory (sifar_chain_cluster.cu); the
+ * kernel here spreads a chunk over the machine, and there the hand-over has two
+ * forms chosen by size: tagged 16-byte stores polled by the thread that needs them
+ * (see handoff_store), or, for grids whose polling threads would get in the way of
+ * the stores they wait for, one result-ready flag per chunk.  With both barriers the
  * chunk's done flags (bottom barrier) hand the result over as well: they are
  * released after the result stores.  Every arrow is one dependent trip through the L2.
  */
@@ -31,13 +33,12 @@
 #ifdef SIFAR_SLOT_S8X2
 #error "the decode-step chains are written for the default slot format; the fallback format is built for libsifar only"
 #endif
-#include "sifar_reduce.cuh"
+#include "sifar_chain.cuh"
 #include "sifar_gen.cuh"
 #include "sifar_workload.h"
 
 namespace sifar {
 
-constexpr int kModeNoAllreduce = SIFAR_CHAIN_NO_ALLREDUCE;
 constexpr unsigned kMaxDelayNs = 1000000u;       /* producer delays are capped at 1 ms */
 constexpr size_t kConcurrentTiles = 48;          /* see sifar_chain::concurrent */
 
@@ -214,107 +215,15 @@ __global__ void k_store_blocks(const void *src, void *dst, uint32_t *flags, unsi
 /* ------------------------------------------------------------------------ */
 /* persistent chain kernel                                                   */
 /* ------------------------------------------------------------------------ */
-struct __align__(128) ChunkFlags {
-    uint32_t ready;                 /* call number whose result chunk is published (flag form of the hand-over) */
-    uint32_t pad0[7];
-    uint32_t arrive[2][8];          /* per parity, per rank: this chunk of the rank's partial stored */
-    uint32_t done[8];               /* per rank: the chunk's reducer has finished reading call e (bottom barrier) */
-};
-
-struct __align__(128) ChainDev {
-    uint32_t exit_count;            /* CTAs that left the kernel (monotonic)                        */
-    uint32_t seen[3];               /* written by CTA 0 of the last run: role layout (1 = clustered), CTAs per
-                                       cluster as the hardware reports them, form of the hand-over (1 = tagged) */
-    uint32_t pad0[28];
-};
-
-struct PersistArgs {
-    DevState *st;
-    int *host_status;
-    unsigned long long timeout_ns;
-    sifar_workload w;
-    unsigned long long n;
-    char *plain;                    /* [parity][rank] plain buffers */
-    unsigned long long plain_stride;
-    char *slots;                    /* [parity][rank] slot buffers  */
-    unsigned long long slot_stride;
-    char *ring;
-    unsigned long long ring_stride;
-    uint32_t ring_len;
-    uint32_t e0;                    /* calls completed before this run     */
-    uint32_t base_epoch;
-    uint32_t steps;
-    uint32_t C;                     /* chunks = reducer CTAs               */
-    uint32_t K;                     /* units per thread and step           */
-    uint32_t exit_base;
-    uint32_t clustered;             /* role layout, see k_chain */
-    PollShape poll;
-    ChainDev *cs;
-    ChunkFlags *chunks;
-    unsigned long long *stamps;     /* C x (steps + 1): per chunk, start of the run and every published result */
-    unsigned long long *trace;      /* NULL, or steps x kTraceSlots phase stamps of chunk 0 (see sifar_workload.h) */
-    uint32_t *retry_steps;          /* steps: 1 if any CTA re-loaded a slot in that step */
-    uint4 *handoff;                 /* [parity][unit]: the result as the next producers take it over (see
-                                       handoff_store), or NULL: one result-ready flag per chunk instead */
-    unsigned long long handoff_stride;   /* 16-byte words per parity */
-};
-
+constexpr size_t kHandoffMaxPairs = 100000;     /* (unit, rank) pairs up to which the result is handed over in tagged words */
 /*
- * Hand-over of a result unit from the chunk's reducer to the P producers of the next step.  The next operation
- * of a rank consumes the all-reduce result on the same GPU (Section 3.1: stream order there); in this one-reader
- * emulation reducer and producers are different CTAs, so the result has to cross.  It crosses the way the partials
- * do in the speculative mode: data and call number in one 16-byte store, validated by the reader, who polls the
- * unit it needs and nothing else - no CTA-wide barrier, no fence, no flag, no second round trip for the data.
- * The other form, one ready flag per chunk (barrier, release; acquire poll by thread 0, barrier, then the loads),
- * costs 0.3-1.0 us more per step at decode payloads in the two barrier-free modes; it is kept for large grids
- * (more than kHandoffMaxPairs polling threads), where eight times as many threads polling data lines as there
- * are units slowed the reducers' stores more than the flag costs (measured at P = 8: 256 KB per rank 7.8 against
- * 7.3 us, 512 KB per rank 14.2 against 11.7 us mean).  With both barriers neither form is needed: the done flags
- * of the bottom barrier follow the result stores.  The chain without all-reduce uses the words too: every rank
- * hands its partial to itself.
- * NW = 3 result words (a 12-byte unit: speculative mode, chain without all-reduce): {w0, w1, w2, tag}.  NW = 4
- * (a 16-byte vector of the dual-buffered mode): two stores {w0, tag, w1, tag}, {w2, tag, w3, tag}, each valid by
- * itself.
+ * One thread-block cluster per chunk up to this many (unit, rank) pairs (sifar_chain_cluster.cu).  Per step, cluster
+ * against spread, P = 8: 8 KB per rank 1.02 / 1.54 us speculative, 0.81 / 2.80 dual-buffered, 1.52 / 3.31 with both
+ * barriers; 64 KB 1.42 / 1.81, 1.37 / 3.01, 1.95 / 3.53; P = 4, 128 KB 1.42 / 1.66, 1.34 / 2.88, 1.47 / 3.48.
  */
-template <int NW>
-__device__ __forceinline__ void handoff_store(uint4 *base, size_t u, const uint4 &v, uint32_t tag)
-{
-    if (NW == 3) {
-        st_slot(base + u, make_uint4(v.x, v.y, v.z, tag));
-    } else {
-        st_slot(base + 2 * u, make_uint4(v.x, tag, v.y, tag));
-        st_slot(base + 2 * u + 1, make_uint4(v.z, tag, v.w, tag));
-    }
-}
-
-/* Polls until unit u carries `tag` (bounded; also gives up when the context already carries an error). */
-template <int NW>
-__device__ __forceinline__ bool handoff_wait(const uint4 *base, size_t u, uint32_t tag, uint32_t (&w)[NW], DevState *st,
-                                             int *host_status, unsigned long long timeout_ns)
-{
-    Deadline d;
-    for (;;) {
-        if (NW == 3) {
-            const uint4 a = ld_slot(base + u);
-            if (a.w == tag) { w[0] = a.x; w[1] = a.y; w[2] = a.z; return true; }
-        } else {
-            const uint4 a = ld_slot(base + 2 * u), b = ld_slot(base + 2 * u + 1);
-            if (a.y == tag && a.w == tag && b.y == tag && b.w == tag) {
-                w[0] = a.x; w[1] = a.z; w[2] = b.x; w[NW - 1] = b.z;
-                return true;
-            }
-        }
-        if (d.expired(timeout_ns)) { fail(st, host_status, SIFAR_ERR_TIMEOUT); return false; }
-        if ((d.polls % 64u) == 0u && ld_relaxed_u32(&st->status) != 0u) return false;
-    }
-}
-
-constexpr size_t kHandoffMaxPairs = 100000;
-constexpr size_t kChainClusterMaxPairs = 50000;  /* one thread-block cluster per chunk up to here, see chain_setup_persistent */
-constexpr size_t kChainWideMaxPairs = 50000;    /* speculative chain with tagged hand-over: wide polling up to here, sentinel above */      /* (unit, rank) pairs up to which the result is handed over in tagged words */
-constexpr int kChainThreads = 128;
+constexpr size_t kChainClusterMaxPairs = 50000;
+constexpr size_t kChainWideMaxPairs = 50000;    /* speculative chain with tagged hand-over: wide polling up to here, sentinel above */
 constexpr int kPreUnits = 4;            /* units per producer thread, beyond its first, whose seeded half is computed before the wait */
-constexpr int kTraceSlots = 48;         /* 0-3 reducer, 4 + 3r .. 6 + 3r rank r's producer, 28 done flags */
 
 template <int DT, int P, int MODE, bool TRACE, bool TAGGED>
 __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
@@ -322,26 +231,11 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
     DevState *st = a.st;
     const uint32_t C = a.C;
     const bool no_ar = (MODE == kModeNoAllreduce);
-    /*
-     * Roles.  Clustered layout: the CTAs that own one chunk (its reducer and its P producers) are consecutive
-     * and launched as one thread-block cluster, which the hardware places inside one GPC, so their flag
-     * and slot traffic stays on one die.  Nothing else of the cluster is used: all communication still
-     * goes through global memory.  Flat layout: reducers first, then the producers rank by rank.
-     */
-    const uint32_t roles = no_ar ? (uint32_t)P : (uint32_t)P + 1u;
-    bool is_reducer;
-    uint32_t rank, chunk;
-    if (a.clustered) {
-        const uint32_t role = blockIdx.x % roles;
-        chunk = blockIdx.x / roles;
-        is_reducer = !no_ar && role == 0u;
-        rank = no_ar ? role : (is_reducer ? 0u : role - 1u);
-    } else {
-        is_reducer = !no_ar && blockIdx.x < C;
-        const uint32_t pidx = no_ar ? blockIdx.x : blockIdx.x - C;
-        rank = is_reducer ? 0u : pidx / C;
-        chunk = is_reducer ? blockIdx.x : pidx % C;
-    }
+    /* roles: reducers first, then the producers rank by rank */
+    const bool is_reducer = !no_ar && blockIdx.x < C;
+    const uint32_t pidx = no_ar ? blockIdx.x : blockIdx.x - C;
+    const uint32_t rank = is_reducer ? 0u : pidx / C;
+    const uint32_t chunk = is_reducer ? blockIdx.x : pidx % C;
     ChunkFlags *cf = a.chunks + chunk;
     const size_t n = (size_t)a.n;
     /* 12-byte units where the unit travels with a tag in one 16-byte word (speculative slots; the chain without
@@ -362,7 +256,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
         /* what this launch really runs with, for sifar_chain_geometry */
         uint32_t cluster_ctas;
         asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cluster_ctas));
-        a.cs->seen[0] = a.clustered; a.cs->seen[1] = cluster_ctas; a.cs->seen[2] = TAGGED ? 1u : 0u;
+        a.cs->seen[0] = 0u; a.cs->seen[1] = cluster_ctas; a.cs->seen[2] = TAGGED ? 1u : 0u;
     }
     __syncthreads();
     unsigned reloads = 0;
@@ -709,7 +603,9 @@ struct sifar_chain {
     bool tagged;                    /* form of the hand-over (see handoff_store) */
     uint32_t C, K;
     int grid;
-    bool clustered;                 /* one thread-block cluster per chunk (placement only) */
+    const void *cluster_kernel;     /* not NULL: one thread-block cluster per chunk, whose ranks meet in its shared
+                                       memory (sifar_chain_cluster.cu) */
+    uint32_t stamp_pipes;           /* rows of stamps per chunk (see PersistArgs::stamps) */
 };
 
 /*
@@ -921,55 +817,45 @@ static int chain_setup_persistent(sifar_chain *ch)
     size_t max_pairs = kHandoffMaxPairs;
     if (const char *env = getenv("SIFAR_CHAIN_HANDOFF_MAX")) max_pairs = (size_t)strtoull(env, nullptr, 10);
     ch->tagged = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && units * (size_t)c->P <= max_pairs;
-    int per_sm = 0;
-    SIFAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chain_kernel(ch), kChainThreads, 0));
-    const size_t resident = (size_t)per_sm * c->sm_count;
-    /* the whole machine if need be: every unit per thread beyond the first lengthens the step by its
-       dependent load and store round trips */
-    const size_t budget = resident > (size_t)roles ? resident : (size_t)roles;
-    uint32_t K = 1;      /* units per thread and step: 1 whenever the grid fits (more only lengthens the step) */
-    size_t C = (units + kChainThreads - 1) / kChainThreads;
-    while (C * roles > budget) {
-        ++K;
-        C = (units + (size_t)kChainThreads * K - 1) / ((size_t)kChainThreads * K);
-    }
-    ch->K = K; ch->C = (uint32_t)C; ch->grid = (int)(C * roles);
-    /* One cluster per chunk if the device can hold all of them at once, for grids up to kChainClusterMaxPairs
-       (unit, rank) pairs: keeping a chunk's traffic inside one GPC takes 0.2-0.3 us off a step at decode payloads
-       (P = 8, 8 KB: 1.79 against 1.98 us speculative, 3.58 against 3.87 us with both barriers); larger grids did
-       better spread over the machine (128 KB: 3.81 against 3.34 us; 256 KB: 7.1 against 6.0 us dual-buffered mean).
-       SIFAR_CHAIN_CLUSTER=0: never. */
-    ch->clustered = false;
+    /* One cluster per chunk, its ranks meeting in the cluster's shared memory, for grids up to kChainClusterMaxPairs
+       (unit, rank) pairs that the device can hold at once with one unit per thread.  SIFAR_CHAIN_CLUSTER=0: never;
+       nor with the flag form of the hand-over asked for at such a size. */
     const char *env_cluster = getenv("SIFAR_CHAIN_CLUSTER");
-    if (!(env_cluster && atoi(env_cluster) == 0) && roles <= 16 && units * (size_t)c->P <= kChainClusterMaxPairs) {
-        const void *fn = chain_kernel(ch);
-        cudaError_t err = cudaSuccess;
-        if (roles > 8) err = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof cfg);
-        cfg.gridDim = dim3((unsigned)ch->grid);
-        cfg.blockDim = dim3(kChainThreads);
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)roles;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int max_clusters = 0;
-        if (err == cudaSuccess) err = cudaOccupancyMaxActiveClusters(&max_clusters, fn, &cfg);
-        if (err == cudaSuccess && (size_t)max_clusters >= C) ch->clustered = true;
-        else cudaGetLastError();
+    const size_t chunks = (units + kChainThreads - 1) / kChainThreads;
+    const bool flag_form = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && !ch->tagged;
+    if (!(env_cluster && atoi(env_cluster) == 0) && !flag_form && units * (size_t)c->P <= kChainClusterMaxPairs) {
+        const void *fn = chain_cluster_kernel(c->dtype, c->P, ch->mode, false);
+        if (cluster_fits(fn, roles, chunks)) ch->cluster_kernel = fn;
     }
+    ch->stamp_pipes = ch->cluster_kernel ? kChainThreads / 32 : 1;
+    if (ch->cluster_kernel) {
+        ch->K = 1; ch->C = (uint32_t)chunks;
+    } else {
+        int per_sm = 0;
+        SIFAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chain_kernel(ch), kChainThreads, 0));
+        const size_t resident = (size_t)per_sm * c->sm_count;
+        /* the whole machine if need be: every unit per thread beyond the first lengthens the step by its
+           dependent load and store round trips */
+        const size_t budget = resident > (size_t)roles ? resident : (size_t)roles;
+        uint32_t K = 1;      /* units per thread and step: 1 whenever the grid fits (more only lengthens the step) */
+        size_t C = chunks;
+        while (C * roles > budget) {
+            ++K;
+            C = (units + (size_t)kChainThreads * K - 1) / ((size_t)kChainThreads * K);
+        }
+        ch->K = K; ch->C = (uint32_t)C;
+    }
+    const size_t C = ch->C;
+    ch->grid = (int)(C * roles);
     SIFAR_CUDA(cudaMalloc(&ch->d_cs, sizeof(ChainDev)));
     SIFAR_CUDA(cudaMalloc(&ch->d_chunks, sizeof(ChunkFlags) * C));
-    SIFAR_CUDA(cudaMalloc(&ch->d_stamps, sizeof(unsigned long long) * (ch->steps + 1) * C));
+    SIFAR_CUDA(cudaMalloc(&ch->d_stamps, sizeof(unsigned long long) * (ch->steps + 1) * C * ch->stamp_pipes));
     SIFAR_CUDA(cudaMalloc(&ch->d_trace, sizeof(unsigned long long) * ch->steps * kTraceSlots));
     SIFAR_CUDA(cudaMemset(ch->d_trace, 0, sizeof(unsigned long long) * ch->steps * kTraceSlots));
     SIFAR_CUDA(cudaMalloc(&ch->d_retry_steps, sizeof(uint32_t) * ch->steps));
     SIFAR_CUDA(cudaMemset(ch->d_cs, 0, sizeof(ChainDev)));
     SIFAR_CUDA(cudaMemset(ch->d_chunks, 0, sizeof(ChunkFlags) * C));
-    SIFAR_CUDA(cudaMemset(ch->d_stamps, 0, sizeof(unsigned long long) * (ch->steps + 1) * C));
+    SIFAR_CUDA(cudaMemset(ch->d_stamps, 0, sizeof(unsigned long long) * (ch->steps + 1) * C * ch->stamp_pipes));
     SIFAR_CUDA(cudaMemset(ch->d_retry_steps, 0, sizeof(uint32_t) * ch->steps));
     /* the hand-over buffer (see handoff_store): one 16-byte word per 12-byte unit, two per 16-byte vector, whole
        warps of units, both parities; zero = tag 0 = never valid.  Large grids use the chunks' ready flags instead. */
@@ -1098,29 +984,13 @@ extern "C" int sifar_chain_run(sifar_chain *ch, void *stream)
         a.cs = ch->d_cs; a.chunks = ch->d_chunks; a.stamps = ch->d_stamps; a.retry_steps = ch->d_retry_steps;
         a.trace = ch->trace_on ? ch->d_trace : nullptr;
         a.handoff = ch->d_handoff; a.handoff_stride = ch->handoff_stride;
-        a.clustered = ch->clustered ? 1u : 0u;
         void *params[] = {&a};
-        const void *fn = chain_kernel(ch, ch->trace_on != 0);
-        if (ch->clustered) {
-            const unsigned roles = (unsigned)(no_ar ? c->P : c->P + 1);
-            if (roles > 8) SIFAR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            cudaLaunchConfig_t cfg;
-            memset(&cfg, 0, sizeof cfg);
-            cfg.gridDim = dim3((unsigned)ch->grid);
-            cfg.blockDim = dim3(kChainThreads);
-            cfg.stream = s;
-            cudaLaunchAttribute attr[2];
-            attr[0].id = cudaLaunchAttributeCooperative;
-            attr[0].val.cooperative = 1;
-            attr[1].id = cudaLaunchAttributeClusterDimension;
-            attr[1].val.clusterDim.x = roles;
-            attr[1].val.clusterDim.y = 1;
-            attr[1].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 2;
-            SIFAR_CUDA(cudaLaunchKernelExC(&cfg, fn, params));
+        if (ch->cluster_kernel) {
+            const void *fn = ch->trace_on ? chain_cluster_kernel(c->dtype, c->P, ch->mode, true) : ch->cluster_kernel;
+            SIFAR_CUDA(launch_clusters(fn, no_ar ? c->P : c->P + 1, ch->C, s, params));
         } else {
-            SIFAR_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)ch->grid), dim3(kChainThreads), params, 0, s));
+            SIFAR_CUDA(cudaLaunchCooperativeKernel(chain_kernel(ch, ch->trace_on != 0), dim3((unsigned)ch->grid),
+                                                   dim3(kChainThreads), params, 0, s));
         }
     }
     ch->runs += 1;
@@ -1132,27 +1002,33 @@ extern "C" int sifar_chain_run(sifar_chain *ch, void *stream)
     return SIFAR_OK;
 }
 
+/* Stamps of chunks [c0, c1): a result is complete when its last chunk is (and a chunk when the last of its pipes is):
+   per step the latest stamp; the run starts with the earliest CTA. */
+static int chain_stamps(sifar_chain *ch, uint32_t c0, uint32_t c1, unsigned long long *stamps)
+{
+    SIFAR_CUDA(cudaDeviceSynchronize());
+    const size_t per = (size_t)ch->steps + 1, rows = (size_t)(c1 - c0) * ch->stamp_pipes;
+    std::vector<unsigned long long> all(per * rows);
+    SIFAR_CUDA(cudaMemcpy(all.data(), ch->d_stamps + (size_t)c0 * ch->stamp_pipes * per, sizeof(unsigned long long) * all.size(),
+                          cudaMemcpyDeviceToHost));
+    for (size_t s = 0; s < per; ++s) {
+        unsigned long long v = all[s];
+        for (size_t c = 1; c < rows; ++c) {
+            const unsigned long long x = all[c * per + s];
+            v = (s == 0) ? (x < v ? x : v) : (x > v ? x : v);
+        }
+        stamps[s] = v;
+    }
+    return SIFAR_OK;
+}
+
 extern "C" int sifar_chain_stamps(sifar_chain *ch, unsigned long long *stamps)
 {
     if (!ch || !stamps || ch->impl != SIFAR_CHAIN_PERSISTENT) {
         set_error("sifar_chain_stamps: needs a persistent chain and a destination");
         return SIFAR_ERR_INVALID;
     }
-    SIFAR_CUDA(cudaDeviceSynchronize());
-    const size_t per = (size_t)ch->steps + 1;
-    std::vector<unsigned long long> all(per * ch->C);
-    SIFAR_CUDA(cudaMemcpy(all.data(), ch->d_stamps, sizeof(unsigned long long) * all.size(), cudaMemcpyDeviceToHost));
-    /* a result is complete when its last chunk is: per step the latest stamp over the chunks; the run starts
-       with the earliest CTA */
-    for (size_t s = 0; s < per; ++s) {
-        unsigned long long v = all[s];
-        for (uint32_t c = 1; c < ch->C; ++c) {
-            const unsigned long long x = all[(size_t)c * per + s];
-            v = (s == 0) ? (x < v ? x : v) : (x > v ? x : v);
-        }
-        stamps[s] = v;
-    }
-    return SIFAR_OK;
+    return chain_stamps(ch, 0u, ch->C, stamps);
 }
 
 extern "C" int sifar_chain_chunk_stamps(sifar_chain *ch, int chunk, unsigned long long *stamps)
@@ -1161,11 +1037,7 @@ extern "C" int sifar_chain_chunk_stamps(sifar_chain *ch, int chunk, unsigned lon
         set_error("sifar_chain_chunk_stamps: needs a persistent chain, a chunk below %u and a destination", ch ? ch->C : 0u);
         return SIFAR_ERR_INVALID;
     }
-    SIFAR_CUDA(cudaDeviceSynchronize());
-    const size_t per = (size_t)ch->steps + 1;
-    SIFAR_CUDA(cudaMemcpy(stamps, ch->d_stamps + (size_t)chunk * per, sizeof(unsigned long long) * per,
-                          cudaMemcpyDeviceToHost));
-    return SIFAR_OK;
+    return chain_stamps(ch, (uint32_t)chunk, (uint32_t)chunk + 1u, stamps);
 }
 
 extern "C" int sifar_chain_chunks(sifar_chain *ch) { return ch && ch->impl == SIFAR_CHAIN_PERSISTENT ? (int)ch->C : 0; }
@@ -1180,7 +1052,7 @@ extern "C" int sifar_chain_geometry(sifar_chain *ch, unsigned out[8])
     SIFAR_CUDA(cudaDeviceSynchronize());
     SIFAR_CUDA(cudaMemcpy(&h, ch->d_cs, sizeof h, cudaMemcpyDeviceToHost));
     out[0] = ch->C; out[1] = ch->K; out[2] = (unsigned)ch->grid;
-    out[3] = ch->clustered ? 1u : 0u; out[4] = ch->tagged ? 1u : 0u;
+    out[3] = ch->cluster_kernel ? 1u : 0u; out[4] = ch->tagged ? 1u : 0u;
     out[5] = h.seen[0]; out[6] = h.seen[1]; out[7] = h.seen[2];
     return SIFAR_OK;
 }
@@ -1193,6 +1065,12 @@ extern "C" int sifar_chain_trace(sifar_chain *ch, int enable, unsigned long long
     }
     if (enable && ch->ctx->P != 8 && ch->ctx->P != 2) {
         set_error("sifar_chain_trace: the traced kernel is built for P = 2 and P = 8 only");
+        return SIFAR_ERR_INVALID;
+    }
+    if (enable && ch->cluster_kernel &&
+        !cluster_fits(chain_cluster_kernel(ch->ctx->dtype, ch->ctx->P, ch->mode, true),
+                      ch->ctx->P + (ch->mode == kModeNoAllreduce ? 0 : 1), ch->C)) {
+        set_error("sifar_chain_trace: the traced kernel does not fit the device at this size");
         return SIFAR_ERR_INVALID;
     }
     ch->trace_on = enable ? 1 : 0;

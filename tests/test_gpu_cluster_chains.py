@@ -1,0 +1,67 @@
+"""The persistent chains whose ranks meet in a cluster's shared memory: edges of warps and chunks, one rank to eight,
+the hand-over from run to run, and the same results as the kernels that spread a chunk over the machine."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_08973_b200 import binding as sf
+from paper_2607_08973_b200 import synth
+
+from gpu_util import BF16, F32, MODES, Ctx, assert_bits_equal
+from test_gpu_chains import _oracle_w, _ring, _rows, run_chain
+from test_gpu_symmetric import run_sym
+
+pytestmark = pytest.mark.gpu
+
+# one element; a warp of 12-byte units and of 16-byte vectors, and one element on either side; a chunk of either
+EDGES = [1, 191, 192, 193, 255, 256, 257, 767, 768, 769, 1023, 1024, 1025, 3 * 1024 + 5]
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("P,dtype", [(1, BF16), (2, F32), (5, BF16), (8, BF16), (8, F32)])
+def test_one_reader_at_the_edges_of_warps_and_chunks(oracle, P, dtype, mode):
+    d = synth.chain_workload("moe", P)
+    steps, runs = 4, 3                                # three runs: both ways a result crosses from step to step
+    for n in EDGES:
+        got, st = run_chain(P, n, dtype, d, mode, sf.CHAIN_PERSISTENT, steps, runs=runs)
+        want = oracle.chain(_oracle_w(oracle, d), P, n, dtype, steps * runs)
+        for t in range(steps * runs):
+            assert_bits_equal(got[t], want[t], dtype, f"P={P} n={n} mode={mode} step {t + 1}")
+        assert st["calls"] == st["epoch"] == steps * runs and st["timeouts"] == 0
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("P,dtype", [(1, F32), (3, BF16), (8, BF16)])
+def test_every_reader_at_the_edges_of_warps_and_chunks(oracle, P, dtype, mode):
+    d = synth.chain_workload("sweep", P)
+    steps, runs = 4, 3
+    for n in EDGES:
+        got, _, _, _, st = run_sym(P, n, dtype, d, mode, steps, runs=runs)
+        want = oracle.chain(_oracle_w(oracle, d), P, n, dtype, steps * runs)
+        for r in range(P):
+            for t in range(steps * runs):
+                assert_bits_equal(got[r, t], want[t], dtype, f"P={P} n={n} mode={mode} rank {r} step {t + 1}")
+        assert st["calls"] == steps * runs and st["timeouts"] == 0
+
+
+@pytest.mark.parametrize("mode", MODES)
+def test_clusters_and_spread_chunks_agree_up_to_the_size_where_clusters_end(monkeypatch, mode):
+    """P = 8: the largest bf16 payload below the limit, and the first above it, in both layouts."""
+    P, steps = 8, 6
+    d = synth.chain_workload("llama", P)
+    per_unit = 6 if mode == sf.SPECULATIVE else 8
+    for n, clustered in ((50_000 // P * per_unit, 1), (50_000 // P * per_unit + 1, 0)):
+        results = []
+        for env in ("1", "0"):
+            monkeypatch.setenv("SIFAR_CHAIN_CLUSTER", env)
+            with Ctx(P, n, BF16) as ctx:
+                ring, stride = _ring(n, BF16, steps)
+                ch = sf.sifar_chain_create(ctx.h, sf.make_workload(**d), n, mode, sf.CHAIN_PERSISTENT, ring.data_ptr(),
+                                           steps, steps)
+                sf.sifar_chain_run(ch, 0)
+                torch.cuda.synchronize()
+                assert sf.sifar_status(ctx.h) == 0
+                assert sf.sifar_chain_geometry(ch)["kernel_clustered"] == (clustered if env == "1" else 0)
+                sf.sifar_chain_destroy(ch)
+                results.append(_rows(ring, stride, steps, n, BF16))
+        assert np.array_equal(results[0], results[1])
