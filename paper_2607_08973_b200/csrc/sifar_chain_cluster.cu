@@ -103,6 +103,11 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
     const bool tracer = TRACE && a.trace != nullptr && chunk == 0u;
 #define SIFAR_TRACE(slot, who) do { if (TRACE && tracer && (who)) a.trace[(size_t)s * kTraceSlots + (slot)] = globaltimer_ns(); } while (0)
 
+    /* the same shared memory in the other CTAs: a producer's partials go to the reader, results to the producers */
+    const uint32_t top_at = smem_addr(s_top) - box, hand_at = smem_addr(s_hand) - box, done_at = smem_addr(&s_done) - box;
+    uint32_t peer[P];
+#pragma unroll
+    for (uint32_t q = 0; q < (uint32_t)P; ++q) peer[q] = cluster_map(box, no_ar ? role : is_reader ? q + 1u : 0u);
     Gen g;
     float z[NE];
     if (!is_reader && active) {
@@ -131,16 +136,14 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
         const uint4 *ho_prev = a.handoff + ((size_t)(p ^ 1u) * ho_sets + ho_mine) * a.handoff_stride;
         if (last) gdc_launch_dependents();
         bool ok = true;
+        const unsigned before = reloads;
         if (is_reader) {
             /* ---------------- the pulling side ---------------- */
             SIFAR_TRACE(0, threadIdx.x == 0);
             const uint32_t in = box + (barrier ? 0u : p) * P * kBoxStride * 16u;
             uint4 x[P];
             if constexpr (spec) {
-                const unsigned before = reloads;
                 ok = take_box_slots<P>(x, in, e, a.poll.forced, st, a.host_status, a.timeout_ns, reloads);
-                if (TRACE && tracer && threadIdx.x == 0) a.trace[(size_t)s * kTraceSlots + 29] = reloads - before;
-                if (__any_sync(0xFFFFFFFFu, reloads != before) && lane == 0u) st_relaxed_u32(&a.retry_steps[s], 1u);
             } else {
                 if constexpr (barrier) {
                     if (threadIdx.x == 0) mbar_expect(smem_addr(&s_top[0][0]), P * units * 16u);
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
             if constexpr (barrier) {
                 /* bottom barrier, reader side: this warp has read its share of the single buffer */
                 __syncwarp();
-                if (!last && lane < (uint32_t)P) mbar_arrive_remote(cluster_map(smem_addr(&s_done), lane + 1u));
+                if (!last && lane < (uint32_t)P) mbar_arrive_remote(cluster_map(box, lane + 1u) + done_at);
                 SIFAR_TRACE(28, threadIdx.x == 0);
             }
             const uint4 v = sum_vec<DT, P>(x, !slot_units);
@@ -169,11 +172,11 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
             SIFAR_TRACE(3, threadIdx.x == 0);
             /* to the next producers (the critical path of the chain), then into the caller's ring */
             if (!last) {
-                const uint32_t out = box + (p * kChainThreads + threadIdx.x) * 16u;
+                const uint32_t out = (p * kChainThreads + threadIdx.x) * 16u;
 #pragma unroll
-                for (uint32_t q = 1; q <= (uint32_t)P; ++q) {
-                    if constexpr (spec) st_cluster_slot(cluster_map(out, q), make_uint4(v.x, v.y, v.z, e));
-                    else st_async_vec(cluster_map(out, q), v, cluster_map(smem_addr(&s_hand[p][warp]), q));
+                for (uint32_t q = 0; q < (uint32_t)P; ++q) {
+                    if constexpr (spec) st_cluster_slot(peer[q] + out, make_uint4(v.x, v.y, v.z, e));
+                    else st_async_vec(peer[q] + out, v, peer[q] + hand_at + (p * kWarpsPerCta + warp) * 8u);
                 }
             } else if (!barrier) {
                 handoff_store<NW>(ho_cur, u, v, e);
@@ -181,6 +184,8 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
             char *row = a.ring + (size_t)((t - 1u) % a.ring_len) * a.ring_stride;
             if constexpr (slot_units) store_slot_result<DT>(row, u, n_io, v);
             else store_vec_result<DT>(row, u, n_io, v);
+            if (spec && __any_sync(0xFFFFFFFFu, reloads != before) && lane == 0u) st_relaxed_u32(&a.retry_steps[s], 1u);
+            if (TRACE && spec && tracer && threadIdx.x == 0) a.trace[(size_t)s * kTraceSlots + 29] = reloads - before;
         } else {
             /* ---------------- rank `rank`'s next operation ---------------- */
             const bool first = (t == 1u);
@@ -224,20 +229,19 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
             unit_apply<DT, NW>(g, first, pw, u * NE, n, z, w);
             if constexpr (no_ar) {
                 /* to itself: the next step of this thread */
-                if (!last) st_cluster_slot(cluster_map(box + (p * kChainThreads + threadIdx.x) * 16u, role),
-                                           make_uint4(w[0], w[1], w[2], e));
+                if (!last) st_cluster_slot(peer[0] + (p * kChainThreads + threadIdx.x) * 16u, make_uint4(w[0], w[1], w[2], e));
                 else handoff_store<3>(ho_cur, u, make_uint4(w[0], w[1], w[2], 0u), e);
             } else {
-                const uint32_t to = cluster_map(box + (((barrier ? 0u : p) * P + rank) * kBoxStride + threadIdx.x) * 16u, 0u);
+                const uint32_t to = peer[0] + (((barrier ? 0u : p) * P + rank) * kBoxStride + threadIdx.x) * 16u;
                 if constexpr (spec) st_cluster_slot(to, make_uint4(w[0], w[1], w[2], e));
                 else st_async_vec(to, make_uint4(w[0], w[1], w[2], w[NW - 1]),
-                                  cluster_map(barrier ? smem_addr(&s_top[0][0]) : smem_addr(&s_top[p][warp]), 0u));
+                                  peer[0] + top_at + (barrier ? 0u : (p * kWarpsPerCta + warp) * 8u));
             }
             SIFAR_TRACE(5 + 3 * rank, threadIdx.x == 0);
             SIFAR_TRACE(6 + 3 * rank, !slot_units && threadIdx.x == 0);
             SIFAR_TRACE(42 + warp, rank == 0u && lane == 0u);
             if (!last) {
-                g = make_gen(a.w, rank, t + 1u);
+                gen_step(g, t + 1u);
                 unit_noise<DT, NW>(g, false, u * NE, z);
                 /* here, while the partial is on its way, not below the next wait */
 #pragma unroll
@@ -308,6 +312,10 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
     cluster_prologue(s_box, kBoxSlots, s_top, nullptr, &s_done, (uint32_t)P * (units / 32u));
     const bool stamper = lane == 0u;
     unsigned long long *my_stamps = a.stamps + (((size_t)rank * a.C + chunk) * kWarpsPerCta + warp) * (a.steps + 1u);
+    const uint32_t top_at = smem_addr(s_top) - box, done_at = smem_addr(&s_done) - box;
+    uint32_t peer[P];                                                 /* the readers, not everybody the same one first */
+#pragma unroll
+    for (uint32_t j = 0; j < (uint32_t)P; ++j) peer[j] = cluster_map(box, (rank + 1u + j) % (uint32_t)P);
     unsigned reloads = 0;
     uint32_t prevw[NW];                                               /* this thread's unit of the previous result */
 #pragma unroll
@@ -352,17 +360,16 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
             if (last) st_slot(reinterpret_cast<uint4 *>(a.plain + ((size_t)p * P + rank) * a.plain_stride) + u,
                               make_uint4(w[0], w[1], w[2], w[NW - 1]));
         } else {
-            const uint32_t to = box + (((barrier ? 0u : p) * P + rank) * kBoxStride + threadIdx.x) * 16u;
-            const uint32_t bar = barrier ? smem_addr(&s_top[0][0]) : smem_addr(&s_top[p][warp]);
+            const uint32_t to = (((barrier ? 0u : p) * P + rank) * kBoxStride + threadIdx.x) * 16u;
+            const uint32_t bar = top_at + (barrier ? 0u : (p * kWarpsPerCta + warp) * 8u);
 #pragma unroll
-            for (uint32_t j = 1; j <= (uint32_t)P; ++j) {
-                const uint32_t q = (rank + j) % (uint32_t)P;          /* not everybody to the same CTA first */
-                if constexpr (spec) st_cluster_slot(cluster_map(to, q), make_uint4(w[0], w[1], w[2], e));
-                else st_async_vec(cluster_map(to, q), make_uint4(w[0], w[1], w[2], w[NW - 1]), cluster_map(bar, q));
+            for (uint32_t j = 0; j < (uint32_t)P; ++j) {
+                if constexpr (spec) st_cluster_slot(peer[j] + to, make_uint4(w[0], w[1], w[2], e));
+                else st_async_vec(peer[j] + to, make_uint4(w[0], w[1], w[2], w[NW - 1]), peer[j] + bar);
             }
         }
         if (!last) {
-            g = make_gen(a.w, rank, t + 1u);
+            gen_step(g, t + 1u);
             unit_noise<DT, NW>(g, false, u * NE, z);
 #pragma unroll
             for (int k = 0; k < NE; ++k) asm volatile("" : "+f"(z[k]));
@@ -370,13 +377,10 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
         /* ---- pull what all P ranks have stored and reduce in rank order ---- */
         if constexpr (!no_ar) {
             const uint32_t in = box + (barrier ? 0u : p) * P * kBoxStride * 16u;
+            const unsigned before = reloads;
             uint4 x[P];
             if constexpr (spec) {
-                const unsigned before = reloads;
                 ok = take_box_slots<P>(x, in, e, a.poll.forced, st, a.host_status, a.timeout_ns, reloads);
-                /* a rank mis-speculated in this step if any of its threads had to load a slot again */
-                if (__any_sync(0xFFFFFFFFu, reloads != before) && lane == 0u)
-                    st_relaxed_u32(&a.retry_marks[(size_t)rank * a.steps + s], 1u);
             } else {
                 if constexpr (barrier) {
                     if (threadIdx.x == 0) mbar_expect(smem_addr(&s_top[0][0]), P * units * 16u);
@@ -395,7 +399,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
             if constexpr (barrier) {
                 /* bottom barrier, reader side: this warp's loads of the chunk have returned */
                 __syncwarp();
-                if (!last && lane < (uint32_t)P) mbar_arrive_remote(cluster_map(smem_addr(&s_done), lane));
+                if (!last && lane < (uint32_t)P) mbar_arrive_remote(cluster_map(box, lane) + done_at);
             }
             const uint4 o = sum_vec<DT, P>(x, !spec);
             prevw[0] = o.x; prevw[1] = o.y; prevw[2] = o.z;
@@ -403,6 +407,9 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
             char *row = my_ring + (size_t)((t - 1u) % a.ring_len) * a.ring_stride;
             if constexpr (spec) store_slot_result<DT>(row, u, n_io, o);
             else store_vec_result<DT>(row, u, n_io, o);
+            /* a rank mis-speculated in this step if any of its threads had to load a slot again */
+            if (spec && __any_sync(0xFFFFFFFFu, reloads != before) && lane == 0u)
+                st_relaxed_u32(&a.retry_marks[(size_t)rank * a.steps + s], 1u);
         }
         if (stamper) my_stamps[s + 1u] = globaltimer_ns();
     }

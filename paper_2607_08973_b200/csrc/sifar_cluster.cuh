@@ -59,6 +59,13 @@ __device__ __forceinline__ uint4 ld_shared_slot(uint32_t addr)
     return v;
 }
 
+__device__ __forceinline__ uint32_t ld_shared_tag(uint32_t slot)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(slot + 12u) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(mbar), "r"(count) : "memory");
@@ -129,11 +136,11 @@ constexpr int kBoxThreads = 128;
 constexpr uint32_t kBoxStride = kBoxThreads + 1;
 
 /*
- * Speculative read of slot threadIdx.x of every rank (all 32 lanes of the warp call): lane r < P first polls rank r's
- * copy of the warp's first slot, then every lane loads its P slots, and those whose tag is not `e` are loaded again
- * until they are (a sender's warp stores its 32 slots with one instruction, so that is rare).  Polling one slot per
- * rank instead of P per lane leaves the shared-memory ports to the arriving stores.  `reloads` counts looks that
- * found a stale slot.  False (on all lanes): time limit, or somebody has failed.
+ * Speculative read of slot threadIdx.x of every rank (all 32 lanes of the warp call): lane r < P first polls the tag of
+ * rank r's copy of the warp's last slot, then every lane loads its P slots, and those whose tag is not `e` are loaded
+ * again until they are (a sender's warp stores its 32 slots with one instruction, so that is rare).  Polling one word
+ * per rank instead of P slots per lane leaves the shared-memory ports to the arriving stores.  `reloads` counts looks
+ * that found a stale slot.  False (on all lanes): time limit, or somebody has failed.
  */
 template <int P>
 __device__ __forceinline__ bool take_box_slots(uint4 (&x)[P], uint32_t box, uint32_t e, uint32_t forced, DevState *st,
@@ -143,28 +150,32 @@ __device__ __forceinline__ bool take_box_slots(uint4 (&x)[P], uint32_t box, uint
     const uint32_t mine = box + threadIdx.x * 16u;
     bool ok = true;
     if (lane < (uint32_t)P) {
-        const uint32_t first = box + (lane * kBoxStride + (threadIdx.x - lane)) * 16u;
+        const uint32_t last = box + (lane * kBoxStride + (threadIdx.x | 31u)) * 16u;
         LocalDeadline d;
-        while (!slot_valid(ld_shared_slot(first), e)) {
-            ++reloads;
+        while (ld_shared_tag(last) != e)
             if (d.gives_up(st, host_status, timeout_ns)) { ok = false; break; }
-        }
+        reloads += d.polls;
     }
     if (!__all_sync(0xFFFFFFFFu, ok)) return false;
     for (uint32_t round = 0;; ++round) {
+        uint32_t wrong = 0;
 #pragma unroll
         for (int r = 0; r < P; ++r) x[r] = ld_shared_slot(mine + (uint32_t)r * kBoxStride * 16u);
-        LocalDeadline d;
-        for (;;) {
-            uint32_t stale = 0;
 #pragma unroll
-            for (int r = 0; r < P; ++r) stale |= (uint32_t)(!slot_valid(x[r], e)) << r;
-            if (stale == 0u) break;
-            reloads += __popc(stale);
-            if (d.gives_up(st, host_status, timeout_ns)) { ok = false; break; }
+        for (int r = 0; r < P; ++r) wrong |= x[r].w ^ e;
+        if (wrong) {
+            LocalDeadline d;
+            for (;;) {
+                uint32_t stale = 0;
 #pragma unroll
-            for (int r = 0; r < P; ++r)
-                if (stale & (1u << r)) x[r] = ld_shared_slot(mine + (uint32_t)r * kBoxStride * 16u);
+                for (int r = 0; r < P; ++r) stale |= (uint32_t)(!slot_valid(x[r], e)) << r;
+                if (stale == 0u) break;
+                reloads += __popc(stale);
+                if (d.gives_up(st, host_status, timeout_ns)) { ok = false; break; }
+#pragma unroll
+                for (int r = 0; r < P; ++r)
+                    if (stale & (1u << r)) x[r] = ld_shared_slot(mine + (uint32_t)r * kBoxStride * 16u);
+            }
         }
         ok = __all_sync(0xFFFFFFFFu, ok);
         /* forced retries (the retry-latency experiment): a read that found every slot valid is made again */

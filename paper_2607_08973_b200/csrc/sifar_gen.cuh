@@ -25,13 +25,22 @@ __host__ __device__ __forceinline__ uint32_t mix32(uint32_t x)
 
 enum { kStreamValue = 1, kStreamOutlier = 2, kStreamDelay = 3 };
 
-/* The first four of the six chained mixes depend only on (seed, stream, rank, step). */
-__host__ __device__ __forceinline__ uint32_t gen_prefix(uint32_t seed, uint32_t stream, uint32_t r, uint32_t t)
+/* The first three and four of the six chained mixes depend only on (seed, stream, rank) and on the step as well. */
+__host__ __device__ __forceinline__ uint32_t gen_rank_prefix(uint32_t seed, uint32_t stream, uint32_t r)
 {
     uint32_t h = mix32(seed);
     h = mix32(h ^ stream);
-    h = mix32(h + r);
-    return mix32(h ^ (t * 0x9E3779B9u));
+    return mix32(h + r);
+}
+
+__host__ __device__ __forceinline__ uint32_t gen_step_prefix(uint32_t rank_prefix, uint32_t t)
+{
+    return mix32(rank_prefix ^ (t * 0x9E3779B9u));
+}
+
+__host__ __device__ __forceinline__ uint32_t gen_prefix(uint32_t seed, uint32_t stream, uint32_t r, uint32_t t)
+{
+    return gen_step_prefix(gen_rank_prefix(seed, stream, r), t);
 }
 
 __host__ __device__ __forceinline__ uint32_t gen_word(uint32_t prefix, uint32_t i, uint32_t k)
@@ -40,6 +49,7 @@ __host__ __device__ __forceinline__ uint32_t gen_word(uint32_t prefix, uint32_t 
 }
 
 struct Gen {
+    uint32_t rank_prefix;      /* (seed, value stream, rank)         */
     uint32_t value_prefix;     /* (seed, value stream, rank, step)   */
     uint32_t outlier_prefix;   /* (seed, outlier stream, rank, 0)    */
     int kind;
@@ -50,11 +60,15 @@ struct Gen {
 __device__ __forceinline__ Gen make_gen(const sifar_workload &w, uint32_t r, uint32_t t)
 {
     Gen g;
-    g.value_prefix = gen_prefix(w.seed, kStreamValue, r, t);
+    g.rank_prefix = gen_rank_prefix(w.seed, kStreamValue, r);
+    g.value_prefix = gen_step_prefix(g.rank_prefix, t);
     g.outlier_prefix = gen_prefix(w.seed, kStreamOutlier, r, 0u);
     g.kind = w.kind; g.scale = w.scale; g.sigma = w.sigma; g.outlier_mod = w.outlier_mod;
     return g;
 }
+
+/* On to step t: a chain of steps computes the rank's share of the prefix once. */
+__device__ __forceinline__ void gen_step(Gen &g, uint32_t t) { g.value_prefix = gen_step_prefix(g.rank_prefix, t); }
 
 __device__ __forceinline__ float gen_uniform(const Gen &g, uint32_t i)
 {

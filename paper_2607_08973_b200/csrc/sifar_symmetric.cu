@@ -92,13 +92,15 @@ __global__ void __launch_bounds__(kSymThreads, 6) k_sym(const SymArgs a)
 #pragma unroll
     for (int j = 0; j < NW; ++j) prevw[j] = 0u;
     if (stamper) my_stamps[0] = globaltimer_ns();
+    Gen g = make_gen(a.w, rank, a.e0 + 1u - a.base_epoch);
+    float z0[NE];
+    if (unit0 < nunits) unit_noise<DT, NW>(g, a.e0 == a.base_epoch, unit0 * NE, z0);
 
     for (uint32_t s = 0; s < a.steps && alive; ++s) {
         const uint32_t e = a.e0 + 1u + s;
         const uint32_t t = e - a.base_epoch;
         const uint32_t p = e & 1u;
         const bool first = (t == 1u);
-        const Gen g = make_gen(a.w, rank, t);
         char *row = my_ring + (size_t)((t - 1u) % a.ring_len) * a.ring_stride;
         /* where the previous result (without all-reduce: the rank's previous partial) lies in memory */
         const char *prev_mem = no_ar ? a.plain + ((size_t)(p ^ 1u) * P + rank) * a.plain_stride
@@ -106,9 +108,7 @@ __global__ void __launch_bounds__(kSymThreads, 6) k_sym(const SymArgs a)
         uint4 *dst = spec ? reinterpret_cast<uint4 *>(a.slots + ((size_t)p * P + rank) * a.slot_stride)
                           : reinterpret_cast<uint4 *>(a.plain + ((size_t)(single ? 0u : p) * P + rank) * a.plain_stride);
 
-        /* ---- 1. the rank's next operation: the seeded half first, it needs nothing from anybody ---- */
-        float z0[NE];
-        if (unit0 < nunits) unit_noise<DT, NW>(g, first, unit0 * NE, z0);
+        /* ---- 1. the rank's next operation (the seeded half of its first unit is there already) ---- */
         if (MODE == SIFAR_BARRIER_ONESHOT || a.w.delay_max_ns != 0u) {
             if (threadIdx.x < 32) {
                 bool ok = true;
@@ -144,6 +144,11 @@ __global__ void __launch_bounds__(kSymThreads, 6) k_sym(const SymArgs a)
 #pragma unroll
                 for (int j = 0; j < NW; ++j) prevw[j] = w[j];
             }
+        }
+        /* the seeded half of the next operation needs nothing from anybody: while the partials are on their way */
+        if (s + 1u < a.steps) {
+            gen_step(g, t + 1u);
+            if (unit0 < nunits) unit_noise<DT, NW>(g, false, unit0 * NE, z0);
         }
         if constexpr (no_ar) {
             __syncthreads();

@@ -215,14 +215,26 @@ __global__ void k_store_blocks(const void *src, void *dst, uint32_t *flags, unsi
 /* ------------------------------------------------------------------------ */
 /* persistent chain kernel                                                   */
 /* ------------------------------------------------------------------------ */
-constexpr size_t kHandoffMaxPairs = 100000;     /* (unit, rank) pairs up to which the result is handed over in tagged words */
 /*
- * One thread-block cluster per chunk up to this many (unit, rank) pairs (sifar_chain_cluster.cu).  Per step, cluster
- * against spread, P = 8: 8 KB per rank 1.02 / 1.54 us speculative, 0.81 / 2.80 dual-buffered, 1.52 / 3.31 with both
- * barriers; 64 KB 1.42 / 1.81, 1.37 / 3.01, 1.95 / 3.53; P = 4, 128 KB 1.42 / 1.66, 1.34 / 2.88, 1.47 / 3.48.
+ * (unit, rank) pairs up to which the result is handed over in tagged words (speculative, dual-buffered), and up to
+ * which the speculative reader polls all stale ranks of its own slots (a sentinel slot per rank and warp above).
+ * us per run of 64 steps, P = 8, speculative, flag / tagged with sentinel / tagged and wide: 98 KB per rank
+ * 293 / 181 / 126, 128 KB 254 / 188 / 154, 195 KB (133 336 pairs) 309 / 215 / 212, 256 KB (174 768) 323 / 289 / 293,
+ * 512 KB 547 / 544 / 561; dual-buffered, flag / tagged: 128 KB 250 / 227, 195 KB (100 000 pairs) 265 / 256, 256 KB
+ * 335 / 318, 512 KB 529 / 567.
  */
-constexpr size_t kChainClusterMaxPairs = 50000;
-constexpr size_t kChainWideMaxPairs = 50000;    /* speculative chain with tagged hand-over: wide polling up to here, sentinel above */
+constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE ? 170000 : 130000; }
+/*
+ * One thread-block cluster per chunk up to this many (unit, rank) pairs (sifar_chain_cluster.cu).  us per run of 64
+ * steps, P = 8, cluster against spread: 8 KB per rank 66 / 107 speculative, 57 / 184 dual-buffered, 103 / 218 with both
+ * barriers; 64 KB 105 / 117, 94 / 198, 131 / 231; 78 KB 134 / 130, 105 / 215, 133 / 240; 127 KB 182 / 158, 150 / 228,
+ * 192 / 247.  Speculative is level at 50 000 pairs, where tagged slots through the L2 need no flag either; the two
+ * modes with flags gain as far as the clusters fit the machine.
+ */
+constexpr size_t cluster_max_pairs(int mode)
+{
+    return (mode == SIFAR_DUALBUF || mode == SIFAR_BARRIER_ONESHOT) ? 65000 : 50000;
+}
 constexpr int kPreUnits = 4;            /* units per producer thread, beyond its first, whose seeded half is computed before the wait */
 
 template <int DT, int P, int MODE, bool TRACE, bool TAGGED>
@@ -276,6 +288,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
         char *ring_row = a.ring + (size_t)((t - 1u) % a.ring_len) * a.ring_stride;
 
         constexpr bool tagged = TAGGED;          /* form of the hand-over, see handoff_store (the host's choice by size) */
+    Gen g = make_gen(a.w, rank, 0u);
         /* hand-over words [parity][unit]; without all-reduce [parity][rank][unit]: every rank hands its partial to itself */
         const size_t ho_sets = no_ar ? (size_t)P : 1u, ho_mine = no_ar ? (size_t)rank : 0u;
         uint4 *ho_cur = a.handoff + ((size_t)p * ho_sets + ho_mine) * a.handoff_stride;                 /* this step's result */
@@ -309,10 +322,12 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
             for (uint32_t k = 0; k < a.K; ++k) {
                 const size_t u = unit0 + (size_t)k * kChainThreads;
                 if (MODE == SIFAR_SPECULATIVE && a.poll.sentinel) {
-                    /* warp-uniform: the warp's first slot decides whether the warp has work at all */
+                    /* warp-uniform: the warp's first slot decides whether the warp has work at all.  Its later units
+                       are nearly always there when the first is done, and a look at their sentinels costs a round
+                       trip each (0.4 of 8.9 us per step at 512 KB per rank, 0.6 of 5.6 at 256 KB). */
                     const size_t w0 = u - (threadIdx.x & 31u);
                     if (w0 >= nunits) break;
-                    if (k == 0 || a.K > 1u) {
+                    if (k == 0u) {
                         const unsigned before = reloads;
                         if (!sentinel_wait<P>(src, w0, e, a.timeout_ns, reloads)) {
                             if (threadIdx.x == 0 || (threadIdx.x & 31u) == 0u) fail(st, a.host_status, SIFAR_ERR_TIMEOUT);
@@ -377,7 +392,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
             /* ---------------- rank `rank`, chunk `chunk` of the next operation ---------------- */
             constexpr int NW = kSlotUnits ? 3 : 4;
             constexpr int NE = NW * ((DT == SIFAR_BF16) ? 2 : 1);
-            const Gen g = make_gen(a.w, rank, t);
+            gen_step(g, t);
             const bool first = (t == 1u);
             /* the seeded half of a unit does not need the previous result: do it before waiting.  The first
                unit's stays in registers, those of the next kPreUnits units are parked in shared memory (grids
@@ -812,18 +827,18 @@ static int chain_setup_persistent(sifar_chain *ch)
     const int roles = (ch->mode == kModeNoAllreduce) ? c->P : c->P + 1;
     const size_t units = (ch->mode == SIFAR_SPECULATIVE || ch->mode == kModeNoAllreduce)
                              ? slots_for(c->dtype, ch->n) : (ch->n * elem_size(c->dtype) + 15) / 16;
-    /* how a result reaches the next step's producers: tagged words up to kHandoffMaxPairs polling threads, the
+    /* how a result reaches the next step's producers: tagged words up to handoff_max_pairs() polling threads, the
        chunks' ready flags above (see handoff_store); with both barriers the done flags do it */
-    size_t max_pairs = kHandoffMaxPairs;
+    size_t max_pairs = handoff_max_pairs(ch->mode);
     if (const char *env = getenv("SIFAR_CHAIN_HANDOFF_MAX")) max_pairs = (size_t)strtoull(env, nullptr, 10);
     ch->tagged = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && units * (size_t)c->P <= max_pairs;
-    /* One cluster per chunk, its ranks meeting in the cluster's shared memory, for grids up to kChainClusterMaxPairs
+    /* One cluster per chunk, its ranks meeting in the cluster's shared memory, for grids up to cluster_max_pairs()
        (unit, rank) pairs that the device can hold at once with one unit per thread.  SIFAR_CHAIN_CLUSTER=0: never;
        nor with the flag form of the hand-over asked for at such a size. */
     const char *env_cluster = getenv("SIFAR_CHAIN_CLUSTER");
     const size_t chunks = (units + kChainThreads - 1) / kChainThreads;
     const bool flag_form = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && !ch->tagged;
-    if (!(env_cluster && atoi(env_cluster) == 0) && !flag_form && units * (size_t)c->P <= kChainClusterMaxPairs) {
+    if (!(env_cluster && atoi(env_cluster) == 0) && !flag_form && units * (size_t)c->P <= cluster_max_pairs(ch->mode)) {
         const void *fn = chain_cluster_kernel(c->dtype, c->P, ch->mode, false);
         if (cluster_fits(fn, roles, chunks)) ch->cluster_kernel = fn;
     }
@@ -972,9 +987,9 @@ extern "C" int sifar_chain_run(sifar_chain *ch, void *stream)
         a.poll = poll_shape_for(c, ch->n);
         if (ch->tagged && ch->mode == SIFAR_SPECULATIVE) {
             /* with the tagged hand-over the producers store sooner after the reducer's result, and the reducer does
-               best polling all stale ranks of its own slots up to a larger grid than the discrete reducer's
-               (measured at P = 8: 2.05 / 2.24 us at 32 / 64 KB per rank against 2.98 / 3.07 us with the sentinel) */
-            size_t wide_max = kChainWideMaxPairs;
+               best polling all stale ranks of its own slots up to a larger grid than the discrete reducer's (see
+               handoff_max_pairs) */
+            size_t wide_max = handoff_max_pairs(ch->mode);
             if (const char *env = getenv("SIFAR_CHAIN_WIDE_MAX")) wide_max = (size_t)strtoull(env, nullptr, 10);
             const bool wide = slots_for(c->dtype, ch->n) * (size_t)c->P <= wide_max;
             a.poll.wide = wide ? 1u : 0u;

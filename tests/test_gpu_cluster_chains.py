@@ -49,8 +49,8 @@ def test_clusters_and_spread_chunks_agree_up_to_the_size_where_clusters_end(monk
     """P = 8: the largest bf16 payload below the limit, and the first above it, in both layouts."""
     P, steps = 8, 6
     d = synth.chain_workload("llama", P)
-    per_unit = 6 if mode == sf.SPECULATIVE else 8
-    for n, clustered in ((50_000 // P * per_unit, 1), (50_000 // P * per_unit + 1, 0)):
+    per_unit, pairs = (6, 50_000) if mode == sf.SPECULATIVE else (8, 65_000)
+    for n, clustered in ((pairs // P * per_unit, 1), (pairs // P * per_unit + 1, 0)):
         results = []
         for env in ("1", "0"):
             monkeypatch.setenv("SIFAR_CHAIN_CLUSTER", env)
