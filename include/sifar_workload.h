@@ -64,7 +64,8 @@ typedef struct sifar_chain sifar_chain;   /* opaque */
 /* How the chain runs on the device. */
 typedef enum {
     SIFAR_CHAIN_STREAMS    = 0,  /* P producer streams + one reducer stream, events for the result dependency   */
-    SIFAR_CHAIN_GRAPH      = 1,  /* the same topology captured once into a CUDA graph and replayed              */
+    SIFAR_CHAIN_GRAPH      = 1,  /* a CUDA graph, captured once and replayed: per step one launch for all ranks'
+                                    producers (a launch per rank without all-reduce) and one reducer            */
     SIFAR_CHAIN_PERSISTENT = 2   /* one kernel: reducer CTAs and P groups of producer CTAs that talk only through
                                     flags / tags in memory, for all steps of a run (small grids: in the shared
                                     memory of one thread-block cluster per chunk)                               */

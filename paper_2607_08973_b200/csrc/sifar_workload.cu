@@ -50,10 +50,12 @@ struct ProduceArgs {
     int *host_status;
     unsigned long long timeout_ns;
     sifar_workload w;
-    uint32_t rank;
+    uint32_t rank;             /* of blockIdx.y = 0; the launch covers gridDim.y ranks from here on */
     unsigned long long n;
-    const void *prev;          /* out^{t-1} (or the rank's own previous partial without all-reduce) */
-    void *dst;                 /* the rank's buffer of this step                                    */
+    const char *prev;          /* out^{t-1} (without all-reduce: rank 0's own previous partial)     */
+    unsigned long long prev_stride;   /* 0, or bytes from a rank's previous partial to the next's   */
+    char *dst;                 /* rank 0's buffer of this step                                      */
+    unsigned long long dst_stride;
     uint32_t base_epoch;       /* step t = call number - base_epoch                                 */
     uint32_t parity;
     uint32_t t_fixed;          /* no-all-reduce chains: the step, since no call number advances     */
@@ -65,6 +67,9 @@ template <int DT, int MODE>
 __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
 {
     DevState *st = a.st;
+    const uint32_t rank = a.rank + blockIdx.y;
+    const char *prev = a.prev + rank * a.prev_stride;
+    char *dst = a.dst + rank * a.dst_stride;
     __shared__ uint32_t s_e, s_t, s_guess;
     constexpr int NW = (MODE == SIFAR_SPECULATIVE) ? 3 : 4;
     constexpr int EPU = NW * ((DT == SIFAR_BF16) ? 2 : 1);
@@ -87,16 +92,28 @@ __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
     __syncthreads();
     const uint32_t t_ahead = s_guess;
     float z0[EPU];
-    {
-        const Gen g0 = make_gen(a.w, a.rank, t_ahead);
-        if (tid * EPU < (size_t)a.n) {
-            unit_noise<DT, NW>(g0, t_ahead == 1u, tid * EPU, z0);
+    Gen g = make_gen(a.w, rank, t_ahead);
+    if (tid * EPU < (size_t)a.n) {
+        unit_noise<DT, NW>(g, t_ahead == 1u, tid * EPU, z0);
 #pragma unroll
-            for (int k = 0; k < EPU; ++k) asm volatile("" : "+f"(z0[k]));     /* keep it above the wait */
-        }
+        for (int k = 0; k < EPU; ++k) asm volatile("" : "+f"(z0[k]));     /* keep it above the wait */
     }
     /* if the all-reduce before this operation released its dependents early, wait here for its completion */
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    /* The first unit of the previous result travels together with the call number (its row is known from the launch
+       and has room for whole units): one round trip less between two all-reduces. */
+    uint32_t p0[NW];
+#pragma unroll
+    for (int q = 0; q < NW; ++q) p0[q] = 0u;
+    if (t_ahead != 1u && tid * EPU < (size_t)a.n) {
+        if constexpr (NW == 4) {
+            const uint4 v = ld_slot(reinterpret_cast<const uint4 *>(prev) + tid);
+            p0[0] = v.x; p0[1] = v.y; p0[2] = v.z; p0[NW - 1] = v.w;
+        } else {
+#pragma unroll
+            for (int q = 0; q < NW; ++q) p0[q] = ld_relaxed_u32(reinterpret_cast<const uint32_t *>(prev) + tid * NW + q);
+        }
+    }
     if (threadIdx.x == 0) {
         uint32_t e = 0, t = a.t_fixed;
         bool ok = true;
@@ -111,12 +128,12 @@ __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
             }
             /* bottom barrier, producer side: the single buffer may be overwritten once its last reader is done */
             if (ok && MODE == SIFAR_BARRIER_ONESHOT && t > 1u &&
-                wait_flag_ge(&st->done[a.rank], e - 1u, a.timeout_ns) < 0) {
+                wait_flag_ge(&st->done[rank], e - 1u, a.timeout_ns) < 0) {
                 fail(st, a.host_status, SIFAR_ERR_TIMEOUT);
                 ok = false;
             }
         }
-        if (ok) spin_ns(gen_delay_ns(a.w, a.rank, t));
+        if (ok) spin_ns(gen_delay_ns(a.w, rank, t));
         s_e = ok ? (MODE == kModeNoAllreduce ? 1u : e) : 0u;
         s_t = t;
     }
@@ -124,7 +141,7 @@ __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
     const uint32_t e = s_e, t = s_t;
     if (e == 0u) return;
 
-    const Gen g = make_gen(a.w, a.rank, t);
+    gen_step(g, t);
     const bool first = (t == 1u);
     const size_t n = (size_t)a.n;
     const bool ahead_ok = (t == t_ahead);              /* always, unless the context was used against its contract */
@@ -133,21 +150,21 @@ __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
         const size_t nslots = (n + EPS - 1) / EPS;
         for (size_t s = tid; s < nslots; s += nthreads) {
             uint32_t w[3];
-            if (s == tid && ahead_ok) unit_combine<DT, 3>(g, first, a.prev, s * EPS, n, z0, w);
-            else produce_words<DT, 3>(g, first, a.prev, s * EPS, n, w);
-            store_slot(reinterpret_cast<uint4 *>(a.dst), s, w[0], w[1], w[2], e);
+            if (s == tid && ahead_ok) unit_apply<DT, 3>(g, first, p0, s * EPS, n, z0, w);
+            else produce_words<DT, 3>(g, first, prev, s * EPS, n, w);
+            store_slot(reinterpret_cast<uint4 *>(dst), s, w[0], w[1], w[2], e);
         }
     } else {
         constexpr int EPV = EPU;
         const size_t nvec = (n + EPV - 1) / EPV;       /* the last vector is zero-padded inside the context's buffer */
         for (size_t v = tid; v < nvec; v += nthreads) {
             uint32_t w[4];
-            if (v == tid && ahead_ok) unit_combine<DT, 4>(g, first, a.prev, v * EPV, n, z0, w);
-            else produce_words<DT, 4>(g, first, a.prev, v * EPV, n, w);
-            st_slot(reinterpret_cast<uint4 *>(a.dst) + v, make_uint4(w[0], w[1], w[2], w[3]));
+            if (v == tid && ahead_ok) unit_apply<DT, 4>(g, first, p0, v * EPV, n, z0, w);
+            else produce_words<DT, 4>(g, first, prev, v * EPV, n, w);
+            st_slot(reinterpret_cast<uint4 *>(dst) + v, make_uint4(w[0], w[1], w[2], w[3]));
         }
         if (MODE != kModeNoAllreduce)
-            signal_arrival(&st->pack_count[a.rank], gridDim.x, &st->arrive[e & 1u][a.rank], e);
+            signal_arrival(&st->pack_count[rank], gridDim.x, &st->arrive[e & 1u][rank], e);
     }
 }
 
@@ -271,6 +288,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
         a.cs->seen[0] = 0u; a.cs->seen[1] = cluster_ctas; a.cs->seen[2] = TAGGED ? 1u : 0u;
     }
     __syncthreads();
+    Gen g = make_gen(a.w, rank, 0u);
     unsigned reloads = 0;
     bool alive = true;
     /* the CTA that publishes chunk results stamps them: the chunk's reducer (rank 0's producer without all-reduce) */
@@ -288,7 +306,6 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
         char *ring_row = a.ring + (size_t)((t - 1u) % a.ring_len) * a.ring_stride;
 
         constexpr bool tagged = TAGGED;          /* form of the hand-over, see handoff_store (the host's choice by size) */
-    Gen g = make_gen(a.w, rank, 0u);
         /* hand-over words [parity][unit]; without all-reduce [parity][rank][unit]: every rank hands its partial to itself */
         const size_t ho_sets = no_ar ? (size_t)P : 1u, ho_mine = no_ar ? (size_t)rank : 0u;
         uint4 *ho_cur = a.handoff + ((size_t)p * ho_sets + ho_mine) * a.handoff_stride;                 /* this step's result */
@@ -677,7 +694,7 @@ extern "C" size_t sifar_chain_ring_stride(int dtype, size_t n)
 }
 
 template <int DT>
-static cudaError_t launch_produce_dt(int mode, int grid, cudaStream_t s, const ProduceArgs &a)
+static cudaError_t launch_produce_dt(int mode, dim3 grid, cudaStream_t s, const ProduceArgs &a)
 {
     switch (mode) {
     case SIFAR_BARRIER_ONESHOT: k_produce<DT, SIFAR_BARRIER_ONESHOT><<<grid, kProdThreads, 0, s>>>(a); break;
@@ -688,6 +705,12 @@ static cudaError_t launch_produce_dt(int mode, int grid, cudaStream_t s, const P
     return cudaGetLastError();
 }
 
+/* Producer streams of a stream / graph chain (see enqueue_run). */
+static int producer_streams(const sifar_chain *ch)
+{
+    return (ch->impl == SIFAR_CHAIN_GRAPH && ch->mode != kModeNoAllreduce) ? 1 : ch->ctx->P;
+}
+
 static const void *chain_rank_buffer(const sifar_ctx *c, int mode, uint32_t e, int r)
 {
     if (mode == SIFAR_BARRIER_ONESHOT) return c->plain_buf(0, r);
@@ -695,14 +718,23 @@ static const void *chain_rank_buffer(const sifar_ctx *c, int mode, uint32_t e, i
     return c->plain_buf((int)(e & 1u), r);          /* DUALBUF and the no-all-reduce floor */
 }
 
-/* Enqueue one run (steps steps starting at step first_t) as P producer streams + one reducer stream forked from `origin`. */
+/*
+ * Enqueue one run (`steps` steps starting at step first_t) as producer streams and one reducer stream forked from
+ * `origin`: a stream and a launch per rank, or, for the graph, one launch per step that covers all ranks
+ * (blockIdx.y = rank).  A graph launches its kernels one after another, and with P producers and a reducer per step
+ * that was what a step took: P = 8, 64 steps, a launch per rank against one launch: 338 / 204 us at 8 KB, 359 / 270 at
+ * 32 KB, 393 / 343 at 128 KB, 673 / 632 at 512 KB speculative; dual-buffered 386 / 299 and 736 / 720 at either end,
+ * with both barriers 398 / 342 and 775 / 767.  Without all-reduce the ranks never meet, and one launch would make
+ * them wait for one another (335 / 452 us at 512 KB): they keep a stream each.
+ */
 static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
 {
     sifar_ctx *c = ch->ctx;
     const int P = c->P;
     const bool no_ar = (ch->mode == kModeNoAllreduce);
+    const int lanes = producer_streams(ch);
     SIFAR_CUDA(cudaEventRecord(ch->ev_fork, origin));
-    for (int r = 0; r < P; ++r) SIFAR_CUDA(cudaStreamWaitEvent(ch->prod[r], ch->ev_fork, 0));
+    for (int r = 0; r < lanes; ++r) SIFAR_CUDA(cudaStreamWaitEvent(ch->prod[r], ch->ev_fork, 0));
     if (!no_ar) SIFAR_CUDA(cudaStreamWaitEvent(ch->red, ch->ev_fork, 0));
 
     const size_t units = (ch->mode == SIFAR_SPECULATIVE) ? slots_for(c->dtype, ch->n)
@@ -714,20 +746,22 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
     for (int s = 0; s < ch->steps; ++s) {
         const uint32_t t = first_t + (uint32_t)s;
         const uint32_t e = ch->base_epoch + t;
-        for (int r = 0; r < P; ++r) {
+        for (int r = 0; r < lanes; ++r) {
             if (s > 0 && !no_ar) SIFAR_CUDA(cudaStreamWaitEvent(ch->prod[r], ch->ev_step[s - 1], 0));
             ProduceArgs a;
             memset(&a, 0, sizeof a);
             a.st = c->d_state; a.host_status = c->d_status_alias; a.timeout_ns = c->timeout_ns;
             a.w = ch->w; a.rank = (uint32_t)r; a.n = ch->n;
-            a.dst = const_cast<void *>(chain_rank_buffer(c, ch->mode, e, r));
-            a.prev = no_ar ? chain_rank_buffer(c, ch->mode, e - 1u, r)
+            a.dst_stride = (ch->mode == SIFAR_SPECULATIVE) ? c->slot_stride : c->plain_stride;
+            a.dst = (char *)chain_rank_buffer(c, ch->mode, e, 0);
+            a.prev = no_ar ? (const char *)chain_rank_buffer(c, ch->mode, e - 1u, 0)
                            : ch->ring + (size_t)((t + ch->ring_len - 2u) % ch->ring_len) * ch->ring_stride;
+            a.prev_stride = no_ar ? c->plain_stride : 0u;
             a.base_epoch = ch->base_epoch; a.parity = e & 1u;
             a.t_fixed = no_ar ? t : 0u;
             cudaError_t err = (c->dtype == SIFAR_BF16)
-                ? launch_produce_dt<SIFAR_BF16>(ch->mode, (int)pgrid, ch->prod[r], a)
-                : launch_produce_dt<SIFAR_F32>(ch->mode, (int)pgrid, ch->prod[r], a);
+                ? launch_produce_dt<SIFAR_BF16>(ch->mode, dim3((unsigned)pgrid, (unsigned)(P / lanes)), ch->prod[r], a)
+                : launch_produce_dt<SIFAR_F32>(ch->mode, dim3((unsigned)pgrid, (unsigned)(P / lanes)), ch->prod[r], a);
             SIFAR_CUDA(err);
             if (!no_ar && !ch->concurrent) {
                 /* large reducer grid: order it behind the producers (see sifar_chain::concurrent) */
@@ -753,7 +787,7 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
             if (!early) SIFAR_CUDA(cudaEventRecord(ch->ev_step[s], ch->red));
         }
     }
-    for (int r = 0; r < P; ++r) {
+    for (int r = 0; r < lanes; ++r) {
         SIFAR_CUDA(cudaEventRecord(ch->ev_join[r], ch->prod[r]));
         SIFAR_CUDA(cudaStreamWaitEvent(origin, ch->ev_join[r], 0));
     }
@@ -926,7 +960,7 @@ extern "C" sifar_chain *sifar_chain_create(sifar_ctx *c, const sifar_workload *w
         ch->concurrent = reduce_tiles(c, n, mode == kModeNoAllreduce ? SIFAR_DUALBUF : mode) <= kConcurrentTiles;
         ch->ev_step.assign((size_t)ch->steps, nullptr);
         for (int s = 0; s < ch->steps; ++s) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_step[s], cudaEventDisableTiming));
-        ch->launches_per_run = ch->steps * (c->P + (mode == kModeNoAllreduce ? 0 : 1));      /* one reducer kernel per all-reduce */
+        ch->launches_per_run = ch->steps * (producer_streams(ch) + (mode == kModeNoAllreduce ? 0 : 1));      /* one reducer kernel per all-reduce */
         if (impl == SIFAR_CHAIN_GRAPH) {
             /* capture one run; every later replay finds the same parities because steps_per_run is even */
             cudaStream_t cap;
