@@ -337,25 +337,22 @@ int sifar_debug_sweep_policy(sifar_ctx *ctx, int policy);
  *              is refused with SIFAR_ERR_INVALID (use a context instead).  n = 0 is
  *              a no-op.
  *
- * The kernel's bookkeeping (the count of finished CTAs by which the last CTA
- * knows it is last, and two call counters; 256 bytes) lives in a fixed array in
- * the library's device image: every GPU that loads the library holds it until
+ * The kernel's bookkeeping (two call counters) lives in a fixed array in the
+ * library's device image: every GPU that loads the library holds it until
  * the process exits.  The first call on a device looks up the array's device
  * address (cudaGetSymbolAddress, with that device current) and caches it; make
- * that first call before any stream capture begins.  The call itself enqueues a
- * 4-byte clear of the CTA count and one kernel on `stream`; it calls no
- * cudaMalloc, cudaFree or other allocating routine and does not synchronize.
- * All calls on a device share the array, which keeps the previous call's
- * counters: calls that overlap in time on the GPU (different streams without an
- * ordering between them) race on it and are not supported.
+ * that first call before any stream capture begins.  The call itself enqueues one
+ * kernel on `stream`; it calls no cudaMalloc, cudaFree or other allocating routine
+ * and does not synchronize.  All calls on a device share the array; calls that
+ * overlap in time on the GPU are each counted, and `elements` is that of one of
+ * them.
  */
 int sifar_allreduce_noalloc(const void *const *rank_ptrs, int P, void *out, size_t n, int dtype, void *stream);
 size_t sifar_noalloc_max_elems(void);
 /*
  * The bookkeeping words of the current device's array, for tests and diagnosis (waits for the device, copies
- * to the caller's array, allocates nothing): out[0] = count of finished CTAs (0 between calls: the last CTA of
- * a call re-arms it), out[1] = calls completed on this device since the library was loaded, out[2] = n of the
- * last completed call.
+ * to the caller's array, allocates nothing): out[0] = 0 (no count of CTAs is kept between calls), out[1] = calls
+ * completed on this device since the library was loaded, out[2] = n of the last completed call.
  */
 int sifar_noalloc_counters(unsigned long long out[3]);
 
