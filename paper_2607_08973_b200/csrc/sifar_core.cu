@@ -89,6 +89,8 @@ struct ReduceArgs {
     uint32_t early;          /* 1: reads do not wait for the stream's previous kernel, writes do     */
     uint32_t e_host;         /* the call number the host expects, or 0: take it from device memory   */
     uint32_t pdl;            /* host side only: launch with programmatic stream serialization         */
+    uint32_t let_in;         /* 1: the stream's next kernel may become resident at once, 0: when this grid is done
+                                waiting for its producers (see let_dependents_in)                    */
     uint32_t sweeper;        /* 1: k_sweep follows on the stream: this grid keeps no count and no janitors */
 };
 
@@ -112,6 +114,24 @@ __device__ __forceinline__ void gdc_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void gdc_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 
 constexpr int kThreads = 256;
+
+/*
+ * When a reducer lets the next kernel of its stream in (griddepcontrol.launch_dependents; a CTA that exits does too).
+ * That kernel may be the next call's reducer, whose CTAs then sit on the SMs until this call is closed.  While this
+ * grid still waits for its producers, those may not be scheduled yet, and with the machine full of waiting CTAs they
+ * never were: calls of 8 to 30 MB per rank enqueued back to back with a stream per rank ran into the time limit.  So
+ * a CTA lets them in when its own data is there; a janitor, which may have to wait for queued tiles, when it leaves,
+ * except that one arrival flag per call (not per block) tells it that every tile's data is there.  Where nothing can
+ * be waited for (the host saw all producers done) and in the graph and stream chains, whose grids are small and whose
+ * next producers are meant to get ready beside the reducer, it happens at once.
+ */
+template <bool ONE_FLAG>
+__device__ __forceinline__ void let_dependents_in(const ReduceArgs &a)
+{
+    if (a.let_in) return;                                /* done at the start */
+    if (!ONE_FLAG && a.two_phase && blockIdx.x + a.janitors >= gridDim.x) return;
+    gdc_launch_dependents();
+}
 
 /* ------------------------------------------------------------------------ */
 /* exit of a reducer CTA                                                     */
@@ -478,11 +498,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_reduce_plain(const ReduceArgs a
     constexpr int EPV = (DT == SIFAR_BF16) ? 8 : 4;
     const size_t ntiles = tiles_for((size_t)a.n / EPV, U);
     const size_t tile = blockIdx.x;
-    /* Programmatic dependent launch: the next kernel of the stream may become resident as soon as every
-       CTA of this one has started.  Whether this kernel's own reads wait for the kernel before it is the
-       host's choice (a.early, see launch_reduce); its writes always do. */
+    /* Programmatic dependent launch: whether this kernel's own reads wait for the kernel before it is the host's
+       choice (a.early, see launch_reduce); its writes always do.  When the next kernel may become resident:
+       let_dependents_in(). */
     if (!a.early) gdc_wait();
-    gdc_launch_dependents();
+    if (a.let_in) gdc_launch_dependents();
     int give_up = 0;
     if (a.early && !a.sweeper && (threadIdx.x & 7u) == 0u) {
         /* While warp 0 makes its round trip for the flags, ask the L2 for the tile's lines (one thread per
@@ -523,6 +543,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_reduce_plain(const ReduceArgs a
         e = entry_epoch(a, ld_relaxed_u32x2(&a.st->epoch));         /* after the wait: the predecessor has published */
         alive = (e != 0u);
     } else {
+        let_dependents_in<MODE != kModeTiles>(a);
         tile_plain<DT, P>(a, tile, ntiles, a.early != 0u);             /* pull and reduce (phase 2) */
     }
     /* a sweep kernel follows on the stream: it is ordered after this whole grid, reduces what was queued
@@ -577,8 +598,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const ReduceArgs a)
     __shared__ uint32_t s_e, s_n, s_tile[K];
     __shared__ int s_ok;
     DevState *st = a.st;
-    gdc_launch_dependents();
-    gdc_wait();
+    gdc_wait();                                  /* (the next kernel comes in when this one leaves: it waits for producers) */
     if (threadIdx.x == 0) {
         uint32_t e = entry_epoch(a, ld_relaxed_u32x2(&st->epoch));
         if (e && a.e_host && e != a.e_host) { fail(st, a.host_status, SIFAR_ERR_EPOCH); e = 0u; }
@@ -682,7 +702,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_reduce_spec(const ReduceArgs a)
     /* programmatic dependent launch, as in k_reduce_plain: the slots validate themselves, so the loads
        need not wait for the kernel before this one on the stream unless the host says so */
     if (!a.early) gdc_wait();
-    gdc_launch_dependents();
+    if (a.let_in) gdc_launch_dependents();
 
     /* The call number is loaded together with the slots (no dependent round trip before the data), by one
        thread per CTA: a word that every warp of a large grid loads becomes a hot spot in its L2 slice. */
@@ -719,6 +739,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_reduce_spec(const ReduceArgs a)
             ok = validate_slot<P>(x[u], a.src, s, e, limit_ns, a.poll, reloads);
         }
     }
+    if (alive && ok) let_dependents_in<false>(a);
     if (a.early) gdc_wait();                                /* everything from here on writes */
     if (alive) {
         if (ok) {
@@ -1154,7 +1175,7 @@ int launch_reduce(sifar_ctx *ctx, const ReduceLaunch &rl, cudaStream_t stream)
             }
             const cudaError_t q = cudaStreamQuery(ctx->prod_stream[r]);
             if (q == cudaErrorNotReady) a.sweeper = 1u;
-            if (q != cudaSuccess) cudaGetLastError();          /* "not ready" is an answer, not an error */
+            if (q != cudaSuccess) { a.let_in = 0u; cudaGetLastError(); }     /* "not ready" is an answer, not an error */
         }
     }
     /* with the sweep kernel behind it the grid need not hold the machine for tiles that are not there yet */
@@ -1193,14 +1214,17 @@ static cudaError_t preload_reducers()
     cudaError_t e = preload(k_reduce_plain<DT, P, SIFAR_BARRIER_ONESHOT>);
     if (e == cudaSuccess) e = preload(k_reduce_plain<DT, P, SIFAR_DUALBUF>);
     if (e == cudaSuccess) e = preload(k_reduce_plain<DT, P, kModeTiles>);
+    a.let_in = rl.programmatic_event ? 1u : 0u;
     if (e == cudaSuccess) e = preload(k_reduce_spec<DT, P>);
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, SIFAR_BARRIER_ONESHOT>);
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, SIFAR_DUALBUF>);
+        a.let_in = 1u;                                   /* unless a producer is seen that may not be done */
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, kModeTiles>);
     return e;
 }
 
 template <int DT>
+                a.let_in = 0u;
 static cudaError_t preload_dt(int P)
 {
     cudaError_t e = cudaSuccess;
@@ -1208,6 +1232,7 @@ static cudaError_t preload_dt(int P)
     case 1: e = preload_reducers<DT, 1>(); break;
     case 2: e = preload_reducers<DT, 2>(); break;
     case 3: e = preload_reducers<DT, 3>(); break;
+    if (a.sweeper) a.let_in = 0u;
     case 4: e = preload_reducers<DT, 4>(); break;
     case 5: e = preload_reducers<DT, 5>(); break;
     case 6: e = preload_reducers<DT, 6>(); break;
