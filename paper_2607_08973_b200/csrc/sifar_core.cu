@@ -1163,14 +1163,17 @@ int launch_reduce(sifar_ctx *ctx, const ReduceLaunch &rl, cudaStream_t stream)
        the grid's janitors.  Not while capturing (a stream may not be queried then, and a graph's replays
        meet other conditions than its capture did). */
     a.sweeper = 0u;
+    a.let_in = rl.programmatic_event ? 1u : 0u;
     if (ctx->sweep_policy != SIFAR_SWEEP_NEVER && rl.early && a.e_host && !rl.programmatic_event &&
         kernel_mode != SIFAR_SPECULATIVE && ntiles >= (size_t)kSweepFromTilesPerSm * (size_t)ctx->sm_count) {
         if (ctx->sweep_policy == SIFAR_SWEEP_ALWAYS) a.sweeper = 1u;
+        a.let_in = 1u;                                   /* unless a producer is seen that may not be done */
         for (int r = 0; r < ctx->P && !a.sweeper; ++r) {
             /* a stream that is being captured may not be queried (the capture would be invalidated) */
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
             if (cudaStreamIsCapturing(ctx->prod_stream[r], &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
                 cudaGetLastError();
+                a.let_in = 0u;
                 continue;
             }
             const cudaError_t q = cudaStreamQuery(ctx->prod_stream[r]);
@@ -1178,6 +1181,7 @@ int launch_reduce(sifar_ctx *ctx, const ReduceLaunch &rl, cudaStream_t stream)
             if (q != cudaSuccess) { a.let_in = 0u; cudaGetLastError(); }     /* "not ready" is an answer, not an error */
         }
     }
+    if (a.sweeper) a.let_in = 0u;
     /* with the sweep kernel behind it the grid need not hold the machine for tiles that are not there yet */
     if (a.sweeper && a.spin_ns > kSweepSpinNs) a.spin_ns = kSweepSpinNs;
     g_programmatic_event = rl.programmatic_event;
@@ -1214,17 +1218,14 @@ static cudaError_t preload_reducers()
     cudaError_t e = preload(k_reduce_plain<DT, P, SIFAR_BARRIER_ONESHOT>);
     if (e == cudaSuccess) e = preload(k_reduce_plain<DT, P, SIFAR_DUALBUF>);
     if (e == cudaSuccess) e = preload(k_reduce_plain<DT, P, kModeTiles>);
-    a.let_in = rl.programmatic_event ? 1u : 0u;
     if (e == cudaSuccess) e = preload(k_reduce_spec<DT, P>);
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, SIFAR_BARRIER_ONESHOT>);
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, SIFAR_DUALBUF>);
-        a.let_in = 1u;                                   /* unless a producer is seen that may not be done */
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, kModeTiles>);
     return e;
 }
 
 template <int DT>
-                a.let_in = 0u;
 static cudaError_t preload_dt(int P)
 {
     cudaError_t e = cudaSuccess;
@@ -1232,7 +1233,6 @@ static cudaError_t preload_dt(int P)
     case 1: e = preload_reducers<DT, 1>(); break;
     case 2: e = preload_reducers<DT, 2>(); break;
     case 3: e = preload_reducers<DT, 3>(); break;
-    if (a.sweeper) a.let_in = 0u;
     case 4: e = preload_reducers<DT, 4>(); break;
     case 5: e = preload_reducers<DT, 5>(); break;
     case 6: e = preload_reducers<DT, 6>(); break;
