@@ -182,13 +182,13 @@ int sifar_allreduce(sifar_ctx *ctx, const void *const *rank_ptrs, void *out, siz
                     int mode, void *stream);
 
 /*
- * Same operation from HOST memory, synchronous: moves the P host partials
- * (n plain elements each) to the device, packs them, reduces, delivers the result
- * in host_out and waits.  Pinned (page-locked), 16-byte aligned buffers are read
- * and written in place by the kernels: one launch packs all ranks, one reduces.
- * Pageable buffers go through staging buffers that the context allocates on the
- * first such call (one copy per rank).  For end-to-end measurements and simple
- * clients.
+ * Same operation from HOST memory, synchronous: reduces the P host partials (n
+ * plain elements each) in one kernel, delivers the result in host_out and waits.
+ * Pinned (page-locked), 16-byte aligned buffers are read and written in place.
+ * Pageable ones go through staging that the context allocates on the first such
+ * call: a pinned buffer that the host fills, up to 32 KiB per partial, one copy to
+ * the device per rank above.  host_out may be one of the partials or overlap them.
+ * For end-to-end measurements and simple clients.
  */
 int sifar_allreduce_host(sifar_ctx *ctx, const void *const *host_rank_ptrs, void *host_out,
                          size_t n, int mode);

@@ -906,21 +906,41 @@ __global__ void __launch_bounds__(kThreads) k_pack(const PackArgs a)
     pack_body<DT, MODE>(a);
 }
 
-/* All P ranks in one launch (blockIdx.y = rank): the host-buffer entry point packs straight from pinned host memory. */
-struct PackAllArgs {
-    const void *src[kMaxRanks];
-    void *dst[kMaxRanks];
-    PackArgs common;             /* src, dst and rank are filled in per rank */
-};
-
-template <int DT, int MODE>
-__global__ void __launch_bounds__(kThreads) k_pack_all(const PackAllArgs all)
+/*
+ * The host-buffer entry point: every partial is there when the call is made and nobody stores beside it, so there is
+ * nothing to wait for and no reason to store the partials once more.  One kernel reads the P partials where they lie
+ * (pinned host memory, or staging), adds them up and writes the result; the last CTA closes the call as every
+ * reducer does.  P = 8, 8 KB per rank, pinned: 25.1 us a call with a pack kernel and a reducer, each with its own
+ * launch and trips over the bus, 17.9 us this way; below 100 KB per rank it is bound by those trips and the wait.
+ */
+template <int DT, int P, bool BARRIER>
+__global__ void __launch_bounds__(kThreads) k_reduce_ready(const ReduceArgs a)
 {
-    PackArgs a = all.common;
-    a.rank = blockIdx.y;
-    a.src = all.src[blockIdx.y];
-    a.dst = all.dst[blockIdx.y];
-    pack_body<DT, MODE>(a);
+    constexpr int EPV = (DT == SIFAR_BF16) ? 8 : 4;
+    DevState *st = a.st;
+    const size_t nvec = (size_t)a.n / EPV;
+    const size_t v = (size_t)blockIdx.x * kThreads + threadIdx.x;
+    __shared__ uint2 s_es;
+    if (threadIdx.x == 0) s_es = ld_relaxed_u32x2(&st->epoch);
+    uint4 x[P];
+    if (v < nvec) {
+#pragma unroll
+        for (int r = 0; r < P; ++r) x[r] = __ldcs(a.src[r] + v);
+    }
+    __syncthreads();
+    uint32_t e = entry_epoch(a, s_es);
+    if (e && e != a.e_host) {                          /* host and device disagree about the call number */
+        fail(st, a.host_status, SIFAR_ERR_EPOCH);
+        e = 0u;
+    }
+    if (e == 0u) return;
+    if (v < nvec) reinterpret_cast<uint4 *>(a.out)[v] = sum_vec<DT, P>(x, true);
+    if (blockIdx.x == gridDim.x - 1) ragged_tail<DT, P>(a);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint32_t arrived = atom_add_relaxed_u32(&st->cta_arrive[a.parity], 1u) + 1u;
+        if (arrived == gridDim.x) publish_call<BARRIER ? SIFAR_BARRIER_ONESHOT : SIFAR_DUALBUF>(st, e, P);
+    }
 }
 
 /* Release of one rank's arrival flag after caller-written plain partials. */
@@ -1243,10 +1263,6 @@ static cudaError_t preload_dt(int P)
     if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_DUALBUF>);
     if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_SPECULATIVE>);
     if (e == cudaSuccess) e = preload(k_pack<DT, kModeTiles>);
-    if (e == cudaSuccess) e = preload(k_pack_all<DT, SIFAR_BARRIER_ONESHOT>);
-    if (e == cudaSuccess) e = preload(k_pack_all<DT, SIFAR_DUALBUF>);
-    if (e == cudaSuccess) e = preload(k_pack_all<DT, SIFAR_SPECULATIVE>);
-    if (e == cudaSuccess) e = preload(k_pack_all<DT, kModeTiles>);
     if (e == cudaSuccess) e = preload(k_arrive);
     if (e == cudaSuccess) e = preload(k_wait_writable);
     if (e == cudaSuccess) e = preload(k_empty_call);
@@ -1259,16 +1275,27 @@ cudaError_t preload_kernels(int dtype, int P)
     return dtype == SIFAR_BF16 ? preload_dt<SIFAR_BF16>(P) : preload_dt<SIFAR_F32>(P);
 }
 
-template <int DT>
-static cudaError_t launch_pack_all_dt(int mode, dim3 grid, cudaStream_t s, const PackAllArgs &a)
+template <int DT, int P>
+static cudaError_t launch_ready_p(bool barrier, int grid, cudaStream_t s, const ReduceArgs &a)
 {
-    switch (mode) {
-    case SIFAR_BARRIER_ONESHOT: k_pack_all<DT, SIFAR_BARRIER_ONESHOT><<<grid, kThreads, 0, s>>>(a); break;
-    case SIFAR_DUALBUF:         k_pack_all<DT, SIFAR_DUALBUF><<<grid, kThreads, 0, s>>>(a); break;
-    case kModeTiles:            k_pack_all<DT, kModeTiles><<<grid, kThreads, 0, s>>>(a); break;
-    default:                    k_pack_all<DT, SIFAR_SPECULATIVE><<<grid, kThreads, 0, s>>>(a); break;
-    }
+    if (barrier) k_reduce_ready<DT, P, true><<<grid, kThreads, 0, s>>>(a);
+    else k_reduce_ready<DT, P, false><<<grid, kThreads, 0, s>>>(a);
     return cudaGetLastError();
+}
+
+template <int DT>
+static cudaError_t launch_ready_dt(int P, bool barrier, int grid, cudaStream_t s, const ReduceArgs &a)
+{
+    switch (P) {
+    case 1: return launch_ready_p<DT, 1>(barrier, grid, s, a);
+    case 2: return launch_ready_p<DT, 2>(barrier, grid, s, a);
+    case 3: return launch_ready_p<DT, 3>(barrier, grid, s, a);
+    case 4: return launch_ready_p<DT, 4>(barrier, grid, s, a);
+    case 5: return launch_ready_p<DT, 5>(barrier, grid, s, a);
+    case 6: return launch_ready_p<DT, 6>(barrier, grid, s, a);
+    case 7: return launch_ready_p<DT, 7>(barrier, grid, s, a);
+    default: return launch_ready_p<DT, 8>(barrier, grid, s, a);
+    }
 }
 
 template <int DT>
@@ -1405,6 +1432,7 @@ extern "C" int sifar_destroy(sifar_ctx *c)
     cudaFree(c->d_tflags);
     if (c->d_stage_in) cudaFree(c->d_stage_in);
     if (c->d_stage_out) cudaFree(c->d_stage_out);
+    if (c->h_bounce) cudaFreeHost(c->h_bounce);
     cudaFreeHost((void *)c->h_status);
     cudaStreamDestroy(c->host_stream);
     delete c;
@@ -1441,6 +1469,20 @@ static size_t ctx_buffer_bytes(const sifar_ctx *c, int mode, size_t n)
 {
     const bool slots = (mode == SIFAR_SPECULATIVE && spec_format(c->P, c->dtype, n) == SIFAR_FORMAT_SLOTS);
     return slots ? slots_for(c->dtype, n) * 16 : n * elem_size(c->dtype);
+}
+
+/* Identity of a stream for as long as the process lives (a handle may be used again for another stream), or 0 for one
+   that is being captured: a graph's replays need not run where it was captured. */
+static unsigned long long stream_key(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    unsigned long long id = 0;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+        cudaStreamGetId(stream, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return id + 1u;
 }
 
 /* What sifar_pack / sifar_arrive remember about the producer of `rank` for call e. */
@@ -1516,6 +1558,7 @@ extern "C" int sifar_allreduce(sifar_ctx *c, const void *const *rank_ptrs, void 
     if (rc) return rc;
     c->h_epoch = e;
     if (mode == SIFAR_BARRIER_ONESHOT) c->last_mode0_epoch = e;
+    c->last_call_stream = c->last_mode0_epoch ? stream_key((cudaStream_t)stream) : 0;
     return SIFAR_OK;
 }
 
@@ -1656,6 +1699,7 @@ extern "C" int sifar_reset(sifar_ctx *c, void *stream)
     *c->h_status = 0;
     c->h_epoch = 0;
     c->last_mode0_epoch = 0;
+    c->last_call_stream = 0;
     memset(c->prod_epoch, 0, sizeof c->prod_epoch);
     return SIFAR_OK;
 }
@@ -1669,6 +1713,7 @@ extern "C" int sifar_debug_set_epoch(sifar_ctx *c, unsigned calls_so_far)
     SIFAR_CUDA(cudaDeviceSynchronize());
     c->h_epoch = calls_so_far;
     c->last_mode0_epoch = 0;
+    c->last_call_stream = 0;
     memset(c->prod_epoch, 0, sizeof c->prod_epoch);
     return SIFAR_OK;
 }
@@ -1693,14 +1738,38 @@ extern "C" int sifar_debug_force_retries(sifar_ctx *c, unsigned rounds)
 }
 
 /* Device-usable address of a host pointer if it is pinned (or otherwise reachable from the GPU), else NULL. */
-static void *device_view(const void *p)
+static void *device_view(const void *p, bool *on_device)
 {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (at.type == cudaMemoryTypeDevice) *on_device = true;
     if (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeManaged || at.type == cudaMemoryTypeDevice)
         return at.devicePointer;
     return nullptr;
 }
+
+/* One all-reduce of partials that are ready, on the context's own stream (see k_reduce_ready). */
+static int reduce_ready(sifar_ctx *c, const void *const *src, void *out, size_t n, int mode, uint32_t e)
+{
+    ReduceArgs a;
+    memset(&a, 0, sizeof a);
+    for (int r = 0; r < c->P; ++r) a.src[r] = static_cast<const uint4 *>(src[r]);
+    a.out = out; a.n = n;
+    a.st = c->d_state; a.host_status = c->d_status_alias;
+    a.parity = e & 1u; a.check_parity = 1u; a.e_host = e;
+    const int grid = (int)tiles_for(n * elem_size(c->dtype) / 16, 1);
+    const bool barrier = (mode == SIFAR_BARRIER_ONESHOT);
+    SIFAR_CUDA(c->dtype == SIFAR_BF16 ? launch_ready_dt<SIFAR_BF16>(c->P, barrier, grid, c->host_stream, a)
+                                      : launch_ready_dt<SIFAR_F32>(c->P, barrier, grid, c->host_stream, a));
+    c->h_epoch = e;
+    if (barrier) c->last_mode0_epoch = e;
+    c->last_call_stream = c->last_mode0_epoch ? stream_key(c->host_stream) : 0;
+    return SIFAR_OK;
+}
+
+/* Pageable partials of up to this many bytes each go through a pinned buffer of the context's, filled by the host:
+   a copy engine call per rank costs more than the copy. */
+constexpr size_t kBounceBytes = (size_t)32 << 10;
 
 extern "C" int sifar_allreduce_host(sifar_ctx *c, const void *const *host_rank_ptrs, void *host_out, size_t n,
                                     int mode)
@@ -1715,76 +1784,82 @@ extern "C" int sifar_allreduce_host(sifar_ctx *c, const void *const *host_rank_p
         if (!host_rank_ptrs[r]) { set_error("sifar_allreduce_host: NULL rank pointer"); return SIFAR_ERR_INVALID; }
     cudaStream_t s = c->host_stream;
     const size_t bytes = n * elem_size(c->dtype);
-
-    /* Fast path: every partial is pinned host memory the GPU can read in place.  One kernel packs all P
-       ranks straight from host memory (the H2D transfer happens inside that kernel), one reduces. */
-    PackAllArgs all;
-    memset(&all, 0, sizeof all);
-    bool direct = (n > 0);
-    for (int r = 0; r < c->P && direct; ++r) {
-        void *d = device_view(host_rank_ptrs[r]);
-        direct = d && (((uintptr_t)d & 15u) == 0);
-        all.src[r] = d;
-    }
-    if (direct) {
-        uint32_t e;
-        if ((rc = next_epoch(c, "sifar_allreduce_host", &e))) return rc;
-        for (int r = 0; r < c->P; ++r) all.dst[r] = const_cast<void *>(ctx_buffer(c, mode, e, r));
-        all.common.tile_flags = c->tile_flags((int)(e & 1u));
-        const int kernel_mode = (mode == SIFAR_SPECULATIVE && spec_format(c->P, c->dtype, n) == SIFAR_FORMAT_TILES)
-                                    ? kModeTiles : mode;
-        all.common.n = n;
-        all.common.st = c->d_state;
-        all.common.host_status = c->d_status_alias;
-        all.common.timeout_ns = c->timeout_ns;
-        all.common.parity = e & 1u;
-        all.common.wait_delta = (mode == SIFAR_BARRIER_ONESHOT && c->last_mode0_epoch) ? e - c->last_mode0_epoch : 0u;
-        const size_t units = (kernel_mode == SIFAR_SPECULATIVE) ? slots_for(c->dtype, n) : (bytes + 15) / 16;
-        size_t gx = (kernel_mode == kModeTiles) ? flag_blocks(c->dtype, n) : (units + kThreads - 1) / kThreads;
-        const size_t cap = (size_t)c->sm_count * 2;
-        if (gx > cap) gx = cap;
-        cudaError_t err = (c->dtype == SIFAR_BF16)
-            ? launch_pack_all_dt<SIFAR_BF16>(kernel_mode, dim3((unsigned)gx, (unsigned)c->P), s, all)
-            : launch_pack_all_dt<SIFAR_F32>(kernel_mode, dim3((unsigned)gx, (unsigned)c->P), s, all);
-        SIFAR_CUDA(err);
-        for (int r = 0; r < c->P; ++r) note_producer(c, r, e, s, n);
-        void *out_dev = device_view(host_out);
-        if (out_dev && ((uintptr_t)out_dev & 15u) == 0) {
-            if ((rc = sifar_allreduce(c, nullptr, out_dev, n, mode, s))) return rc;     /* result written in place */
-        } else {
-            if (!c->d_stage_out) {
-                cudaError_t e2 = cudaMalloc(&c->d_stage_out, c->plain_stride);
-                if (e2 != cudaSuccess) { cudaGetLastError(); set_error("sifar_allreduce_host: staging allocation failed"); return SIFAR_ERR_NOMEM; }
+    uint32_t e;
+    if ((rc = next_epoch(c, "sifar_allreduce_host", &e))) return rc;
+    void *copy_back = nullptr;                              /* device staging of the result, copied to host_out */
+    const char *bounced = nullptr;                          /* pinned staging of the result                     */
+    if (n == 0) {
+        if ((rc = sifar_allreduce(c, nullptr, nullptr, 0, mode, s))) return rc;
+    } else {
+        /* In place where every partial is memory the GPU can read: the transfers happen inside the kernel. */
+        const void *src[kMaxRanks];
+        bool direct = true, crossing = false, on_device = false;
+        for (int r = 0; r < c->P; ++r) {
+            src[r] = device_view(host_rank_ptrs[r], &on_device);
+            direct &= src[r] && (((uintptr_t)src[r] & 15u) == 0);
+        }
+        /* The kernel reads a vector of every partial and then writes it: the result may take the place of a partial,
+           but not straddle one. */
+        for (int r = 0; r < c->P; ++r)
+            crossing |= (host_rank_ptrs[r] != host_out && overlaps(host_rank_ptrs[r], bytes, host_out, bytes));
+        void *out_dev = device_view(host_out, &on_device);
+        if (!direct || crossing) out_dev = nullptr;
+        if (out_dev && ((uintptr_t)out_dev & 15u)) out_dev = nullptr;
+        const size_t slice = (bytes + 255) / 256 * 256;
+        if (!direct && !on_device && bytes <= kBounceBytes) {
+            if (!c->h_bounce) {
+                const cudaError_t err = cudaHostAlloc((void **)&c->h_bounce, kBounceBytes * (c->P + 1), cudaHostAllocMapped);
+                if (err != cudaSuccess) {
+                    cudaGetLastError();
+                    c->h_bounce = nullptr;
+                    set_error("sifar_allreduce_host: staging allocation failed: %s", cudaGetErrorString(err));
+                    return SIFAR_ERR_NOMEM;
+                }
             }
-            if ((rc = sifar_allreduce(c, nullptr, c->d_stage_out, n, mode, s))) return rc;
-            SIFAR_CUDA(cudaMemcpyAsync(host_out, c->d_stage_out, bytes, cudaMemcpyDeviceToHost, s));
+            char *dev = nullptr;
+            SIFAR_CUDA(cudaHostGetDevicePointer((void **)&dev, c->h_bounce, 0));
+            for (int r = 0; r < c->P; ++r) {
+                memcpy(c->h_bounce + r * slice, host_rank_ptrs[r], bytes);
+                src[r] = dev + r * slice;
+            }
+            out_dev = dev + c->P * slice;
+            bounced = c->h_bounce + c->P * slice;
+        } else {
+            if (!out_dev) {
+                if (!c->d_stage_out) {
+                    const cudaError_t err = cudaMalloc(&c->d_stage_out, c->plain_stride);
+                    if (err != cudaSuccess) {
+                        cudaGetLastError();
+                        c->d_stage_out = nullptr;
+                        set_error("sifar_allreduce_host: staging allocation failed: %s", cudaGetErrorString(err));
+                        return SIFAR_ERR_NOMEM;
+                    }
+                }
+                out_dev = copy_back = c->d_stage_out;
+            }
+            if (!direct) {
+                /* large pageable (or unaligned) partials: through device buffers allocated on first use */
+                if (!c->d_stage_in) {
+                    const cudaError_t err = cudaMalloc(&c->d_stage_in, c->plain_stride * c->P);
+                    if (err != cudaSuccess) {
+                        cudaGetLastError();
+                        c->d_stage_in = nullptr;
+                        set_error("sifar_allreduce_host: staging allocation failed: %s", cudaGetErrorString(err));
+                        return SIFAR_ERR_NOMEM;
+                    }
+                }
+                for (int r = 0; r < c->P; ++r) {
+                    src[r] = c->d_stage_in + r * c->plain_stride;
+                    SIFAR_CUDA(cudaMemcpyAsync(const_cast<void *>(src[r]), host_rank_ptrs[r], bytes, cudaMemcpyHostToDevice, s));
+                }
+            }
         }
-        SIFAR_CUDA(cudaStreamSynchronize(s));
-        rc = *c->h_status;
-        if (rc) set_error("sifar_allreduce_host: device status %d", rc);
-        return rc;
+        if ((rc = reduce_ready(c, src, out_dev, n, mode, e))) return rc;
+        if (copy_back) SIFAR_CUDA(cudaMemcpyAsync(host_out, copy_back, bytes, cudaMemcpyDeviceToHost, s));
     }
-
-    /* General path: pageable host memory goes through staging buffers allocated on first use. */
-    const size_t stride = c->plain_stride;
-    if (!c->d_stage_in) {
-        cudaError_t e = cudaMalloc(&c->d_stage_in, stride * c->P);
-        if (e == cudaSuccess && !c->d_stage_out) e = cudaMalloc(&c->d_stage_out, stride);
-        if (e != cudaSuccess) {
-            if (c->d_stage_in) { cudaFree(c->d_stage_in); c->d_stage_in = nullptr; }
-            cudaGetLastError();
-            set_error("sifar_allreduce_host: staging allocation failed: %s", cudaGetErrorString(e));
-            return SIFAR_ERR_NOMEM;
-        }
-    }
-    for (int r = 0; r < c->P; ++r) {
-        if (bytes) SIFAR_CUDA(cudaMemcpyAsync(c->d_stage_in + r * stride, host_rank_ptrs[r], bytes, cudaMemcpyHostToDevice, s));
-        if ((rc = sifar_pack(c, r, c->d_stage_in + r * stride, n, mode, s))) return rc;
-    }
-    if ((rc = sifar_allreduce(c, nullptr, c->d_stage_out, n, mode, s))) return rc;
-    if (bytes) SIFAR_CUDA(cudaMemcpyAsync(host_out, c->d_stage_out, bytes, cudaMemcpyDeviceToHost, s));
     SIFAR_CUDA(cudaStreamSynchronize(s));
     rc = *c->h_status;
     if (rc) set_error("sifar_allreduce_host: device status %d", rc);
+    else if (bounced) memcpy(host_out, bounced, bytes);
     return rc;
 }

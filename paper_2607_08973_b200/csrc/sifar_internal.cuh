@@ -89,6 +89,7 @@ struct sifar_ctx {
     int *d_status_alias;             /* device alias of h_status                         */
     uint32_t h_epoch;                /* calls enqueued so far                            */
     uint32_t last_mode0_epoch;       /* last BARRIER_ONESHOT call (0: none): whose done flags a producer waits for */
+    unsigned long long last_call_stream;   /* stream (stream_key) of the previous call's reducer, 0: not known       */
     unsigned long long timeout_ns;
     unsigned long long spin_ns;      /* deferring reducer: how long a CTA waits before it queues its tile     */
     size_t poll_wide_max;            /* speculative: wide polling up to this many (slot, rank) pairs per call */
@@ -104,6 +105,7 @@ struct sifar_ctx {
     /* staging for sifar_allreduce_host, allocated on first use */
     char *d_stage_in;
     char *d_stage_out;
+    char *h_bounce;                  /* pinned: small pageable partials and their result                          */
     cudaStream_t host_stream;
 
     char *plain_buf(int parity, int r) const { return d_plain + ((size_t)parity * P + r) * plain_stride; }

@@ -651,6 +651,7 @@ extern "C" int sifar_symchain_run(sifar_symchain *ch, void *stream)
     }
     ch->runs += 1;
     if (!no_ar) c->h_epoch += (uint32_t)ch->steps;
+    c->last_call_stream = 0;
     c->last_mode0_epoch = 0;        /* the chain keeps its own done flags; when it has run, nothing reads the buffers */
     return SIFAR_OK;
 }

@@ -1048,6 +1048,7 @@ extern "C" int sifar_chain_run(sifar_chain *ch, void *stream)
        persistent kernel keeps done flags of its own, and once it has run nothing reads the rank buffers any more. */
     if (ch->mode == SIFAR_BARRIER_ONESHOT)
         c->last_mode0_epoch = (ch->impl == SIFAR_CHAIN_PERSISTENT) ? 0u : c->h_epoch;
+    c->last_call_stream = 0;
     return SIFAR_OK;
 }
 

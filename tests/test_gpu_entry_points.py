@@ -1,0 +1,139 @@
+"""Calls that need no protocol between streams: partials in host memory, caller buffers and packs on one stream, and
+the allocation-free call on two streams at once."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_08973_b200 import binding as sf
+from paper_2607_08973_b200 import synth
+
+from gpu_util import BF16, F32, MODES, Ctx, assert_bits_equal, canary_ok, empty_out, out_to_numpy, to_device
+
+pytestmark = pytest.mark.gpu
+
+# elements around one 16-byte vector, one CTA (256 vectors) and the 32 KiB up to which pageable partials are bounced
+EDGES = {BF16: [1, 7, 8, 9, 2047, 2048, 2049, 16383, 16384, 16385, 50_001],
+         F32: [1, 3, 4, 5, 1023, 1024, 1025, 8191, 8192, 8193, 50_001]}
+
+
+
+@pytest.mark.parametrize("memory", ["pinned", "pageable", "mixed"])
+@pytest.mark.parametrize("P,dtype", [(1, F32), (3, BF16), (8, BF16), (8, F32)])
+def test_host_partials_at_the_edges(oracle, P, dtype, memory):
+    with Ctx(P, 50_001, dtype) as ctx:
+        calls = 0
+        for n in EDGES[dtype]:
+            for mode in MODES:
+                xs = synth.rank_inputs(P, n, dtype, 31 + n + mode, "gauss")
+                hx = [torch.from_numpy(x.view(np.int16) if dtype == BF16 else x) for x in xs]
+                if memory != "pageable":
+                    hx = [t.pin_memory() if memory == "pinned" or r % 2 else t for r, t in enumerate(hx)]
+                out = torch.zeros(n + 8, dtype=hx[0].dtype)
+                out = out.pin_memory() if memory == "pinned" else out
+                sf.sifar_allreduce_host(ctx.h, [t.data_ptr() for t in hx], out.data_ptr(), n, mode)
+                calls += 1
+                got = out.numpy().view(np.uint16) if dtype == BF16 else out.numpy()
+                assert not got[n:].any(), "wrote past n"
+                assert_bits_equal(got[:n], oracle.allreduce(xs, dtype), dtype, f"P={P} n={n} mode={mode} {memory}")
+        st = sf.sifar_get_stats(ctx.h)
+        assert st["calls"] == st["epoch"] == calls and st["timeouts"] == 0
+
+
+@pytest.mark.parametrize("pinned", [False, True])
+@pytest.mark.parametrize("shift", [0, 8, -8])
+def test_a_host_result_may_lie_on_a_partial(oracle, pinned, shift):
+    """In place of rank 1's partial, and straddling it by 16 bytes: the result is that of the values before the call."""
+    P, n = 4, 20_011
+    with Ctx(P, n, BF16) as ctx:
+        xs = synth.rank_inputs(P, n, BF16, 5, "gauss")
+        flat = torch.zeros(P * (n + 5) + 64, dtype=torch.int16)
+        flat = flat.pin_memory() if pinned else flat
+        base = [32 + r * 20_016 for r in range(P)]                       # 16-byte aligned rows
+        for r in range(P):
+            flat[base[r]: base[r] + n] = torch.from_numpy(xs[r].view(np.int16))
+        at = base[1] + shift
+        sf.sifar_allreduce_host(ctx.h, [flat.data_ptr() + 2 * b for b in base], flat.data_ptr() + 2 * at, n, sf.SPECULATIVE)
+        assert_bits_equal(flat.numpy()[at: at + n].view(np.uint16), oracle.allreduce(xs, BF16), BF16, f"shift {shift}")
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("P,dtype", [(1, BF16), (8, BF16), (5, F32)])
+def test_packs_and_reducer_on_one_stream(oracle, P, dtype, mode):
+    """Each small pack may become resident while the one before it runs; its inputs come from the stream as well."""
+    sizes = [1, 5, 6, 7, 8, 9, 1535, 1536, 1537, 2048, 2049, 65_549, 300_007]
+    with Ctx(P, max(sizes), dtype) as ctx:
+        s = torch.cuda.Stream()
+        for n in sizes:
+            for rep in range(3):                                          # calls back to back, without waiting
+                xs = synth.rank_inputs(P, n, dtype, 7 * rep + n, "gauss")
+                hx = [torch.from_numpy(x.view(np.int16) if dtype == BF16 else x).pin_memory() for x in xs]
+                out = empty_out(n, dtype)
+                torch.cuda.synchronize()
+                with torch.cuda.stream(s):
+                    for r in range(P):
+                        xd = hx[r].to("cuda", non_blocking=True)
+                        sf.sifar_pack(ctx.h, r, xd.data_ptr(), n, mode, s.cuda_stream)
+                    sf.sifar_allreduce(ctx.h, None, out.data_ptr(), n, mode, s.cuda_stream)
+                    again = empty_out(n, dtype)
+                    for r in range(P):
+                        sf.sifar_pack(ctx.h, r, out.data_ptr(), n, mode, s.cuda_stream)
+                    sf.sifar_allreduce(ctx.h, None, again.data_ptr(), n, mode, s.cuda_stream)
+                torch.cuda.synchronize()
+                assert sf.sifar_status(ctx.h) == 0
+                got, tail = out_to_numpy(out, n, dtype)
+                want = oracle.allreduce(xs, dtype)
+                assert canary_ok(tail, dtype)
+                assert_bits_equal(got, want, dtype, f"P={P} n={n} mode={mode}")
+                assert_bits_equal(out_to_numpy(again, n, dtype)[0], oracle.allreduce([want] * P, dtype), dtype, "second call")
+
+
+@pytest.mark.parametrize("other_stream", [False, True])
+def test_caller_buffers_on_one_stream_and_across_streams(oracle, other_stream):
+    """sifar_wait_writable behind a reducer of the same stream, and on a stream that has to wait for it."""
+    P, n = 8, 40_003
+    with Ctx(P, n, BF16) as ctx:
+        s, q = torch.cuda.Stream(), torch.cuda.Stream()
+        bufs = [torch.zeros(n + 8, dtype=torch.int16, device="cuda") for _ in range(P)]
+        outs, wants = [], []
+        done = torch.cuda.Event()
+        torch.cuda.synchronize()
+        for call in range(4):
+            xs = synth.rank_inputs(P, n, BF16, 60 + call, "gauss")
+            w = q if (other_stream and call % 2) else s
+            w.wait_event(done)
+            xd = [torch.from_numpy(x.view(np.int16)).pin_memory() for x in xs]
+            with torch.cuda.stream(w):
+                for r in range(P):
+                    sf.sifar_wait_writable(ctx.h, r, w.cuda_stream)
+                    bufs[r][:n].copy_(xd[r], non_blocking=True)
+                    sf.sifar_arrive(ctx.h, r, sf.BARRIER_ONESHOT, w.cuda_stream)
+            out = empty_out(n, BF16)
+            s.wait_stream(torch.cuda.current_stream())
+            sf.sifar_allreduce(ctx.h, [b.data_ptr() for b in bufs], out.data_ptr(), n, sf.BARRIER_ONESHOT, s.cuda_stream)
+            done.record(s)
+            outs.append(out)
+            wants.append((xd, oracle.allreduce(xs, BF16)))
+        torch.cuda.synchronize()
+        assert sf.sifar_status(ctx.h) == 0
+        for call in range(4):
+            got, tail = out_to_numpy(outs[call], n, BF16)
+            assert canary_ok(tail, BF16)
+            assert_bits_equal(got, wants[call][1], BF16, f"call {call}")
+
+
+def test_noalloc_calls_on_two_streams_are_both_booked(oracle):
+    P, n = 8, 1 << 20
+    xs = synth.rank_inputs(P, n, BF16, 3, "gauss")
+    xd = [to_device(x) for x in xs]
+    want = oracle.allreduce(xs, BF16)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    outs = [empty_out(n, BF16) for _ in range(2)]
+    torch.cuda.synchronize()
+    before = sf.sifar_noalloc_counters()["calls"]
+    for _ in range(20):
+        for s, out in zip(streams, outs):
+            sf.sifar_allreduce_noalloc([x.data_ptr() for x in xd], out.data_ptr(), n, BF16, s.cuda_stream)
+    torch.cuda.synchronize()
+    assert sf.sifar_noalloc_counters() == {"cta_arrive": 0, "calls": before + 40, "elements": n}
+    for out in outs:
+        assert_bits_equal(out_to_numpy(out, n, BF16)[0], want, BF16, "two streams")
