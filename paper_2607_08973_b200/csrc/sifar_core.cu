@@ -778,8 +778,26 @@ __device__ __forceinline__ void pack_body(const PackArgs &a)
 {
     DevState *st = a.st;
     __shared__ uint32_t s_epoch;
-    /* a reducer that follows on the same stream may become resident now; it waits for this grid's completion */
-    asm volatile("griddepcontrol.launch_dependents;");
+    /* What follows on the same stream may become resident now; it waits for this grid's completion.  This grid may
+       have become resident early too (small grids, see sifar_pack): the kernel before it may have written src. */
+    gdc_launch_dependents();
+    gdc_wait();
+    const size_t tid = (size_t)blockIdx.x * kThreads + threadIdx.x;
+    const size_t nthreads = (size_t)gridDim.x * kThreads;
+    /* Where a thread has one whole unit at most, its words travel together with the call number: a small pack is two
+       round trips and a launch, and this is one of the two. */
+    constexpr int EPU = (MODE == SIFAR_SPECULATIVE) ? kSlotDataWords * ((DT == SIFAR_BF16) ? 2 : 1) : ((DT == SIFAR_BF16) ? 8 : 4);
+    const bool ahead = MODE != kModeTiles && a.n <= nthreads * EPU && (tid + 1) * EPU <= a.n;
+    uint4 first = make_uint4(0u, 0u, 0u, 0u);
+    if (ahead) {
+        if (MODE == SIFAR_SPECULATIVE) {
+            const uint32_t *p = reinterpret_cast<const uint32_t *>(a.src) + tid * kSlotDataWords;
+            first.x = __ldcs(p); first.y = __ldcs(p + 1);
+            if (kSlotDataWords == 3) first.z = __ldcs(p + 2);
+        } else {
+            first = __ldcs(reinterpret_cast<const uint4 *>(a.src) + tid);
+        }
+    }
     if (threadIdx.x == 0) {
         const uint2 es = ld_relaxed_u32x2(&st->epoch);
         uint32_t e = es.x + 1u;
@@ -804,8 +822,6 @@ __device__ __forceinline__ void pack_body(const PackArgs &a)
     const uint32_t e = s_epoch;
     if (e == 0u) return;
 
-    const size_t tid = (size_t)blockIdx.x * kThreads + threadIdx.x;
-    const size_t nthreads = (size_t)gridDim.x * kThreads;
     if (MODE == kModeTiles) {
         /* Flagged tiles: plain data, and one arrival flag per block of kFlagBlockVecs vectors, released as soon
            as the block is stored, so that the reducer can start on it while the rest is still being written.
@@ -844,6 +860,7 @@ __device__ __forceinline__ void pack_body(const PackArgs &a)
         uint4 *dst = reinterpret_cast<uint4 *>(a.dst);
         /* kPackUnroll independent loads in flight per thread, then their stores */
         size_t v = tid;
+        if (ahead) { st_slot(dst + v, first); v += nthreads; }
         for (; v + (kPackUnroll - 1) * nthreads < nvec; v += kPackUnroll * nthreads) {
             uint4 x[kPackUnroll];
 #pragma unroll
@@ -869,6 +886,13 @@ __device__ __forceinline__ void pack_body(const PackArgs &a)
         /* whole slots first, kPackUnroll of them in flight per thread; the loop below takes the rest */
         const size_t nfull = (size_t)a.n / EPS;
         size_t s = tid;
+        if (ahead) {
+            uint32_t w[NW];
+            w[0] = first.x; w[1] = first.y;
+            if (NW == 3) w[NW - 1] = first.z;
+            store_slot_words(slots, s, w, e);
+            s += nthreads;
+        }
         for (; s + (kPackUnroll - 1) * nthreads < nfull; s += kPackUnroll * nthreads) {
             uint32_t w[kPackUnroll][NW];
 #pragma unroll
@@ -943,14 +967,22 @@ __global__ void __launch_bounds__(kThreads) k_reduce_ready(const ReduceArgs a)
     }
 }
 
+/*
+ * The two one-thread kernels of callers that store partials themselves.  They come in rows, one per rank, and a row
+ * on one stream is as long as its launches: programmatic launch lets the next one get ready while this one runs.  P = 8,
+ * 64 MiB per rank, waits, arrivals and reducer on one stream: 143 us a call, 99 us this way and with the waits left out
+ * where the stream makes them redundant (sifar_wait_writable); the reducer alone takes 87.  Both wait for the kernel
+ * before them on the stream before they do anything.
+ */
 /* Release of one rank's arrival flag after caller-written plain partials. */
 __global__ void k_arrive(DevState *st, int *host_status, uint32_t rank, uint32_t parity)
 {
+    gdc_launch_dependents();
+    gdc_wait();
     const uint2 es = ld_relaxed_u32x2(&st->epoch);
     if (es.y != 0u) return;
     const uint32_t e = es.x + 1u;
     if ((e & 1u) != parity) { fail(st, host_status, SIFAR_ERR_EPOCH); return; }   /* not ordered after the previous call */
-    __threadfence();
     st_release_u32(&st->arrive[e & 1u][rank], e);
 }
 
@@ -958,6 +990,8 @@ __global__ void k_arrive(DevState *st, int *host_status, uint32_t rank, uint32_t
 __global__ void k_wait_writable(DevState *st, int *host_status, uint32_t rank, uint32_t wait_delta, uint32_t parity,
                                 unsigned long long timeout_ns)
 {
+    gdc_launch_dependents();
+    gdc_wait();
     const uint2 es = ld_relaxed_u32x2(&st->epoch);
     if (es.y != 0u) return;
     const uint32_t e = es.x + 1u;
@@ -1176,8 +1210,8 @@ int launch_reduce(sifar_ctx *ctx, const ReduceLaunch &rl, cudaStream_t stream)
         else cudaGetLastError();
     }
     /* Early reads need programmatic launch to mean anything, and the baseline keeps the plain stream order. */
-    a.pdl = (rl.early && g_pdl && !rl.programmatic_event) ? 1u : 0u;
-    a.early = (a.pdl && (rl.mode != SIFAR_BARRIER_ONESHOT || g_barrier_early)) ? 1u : 0u;
+    a.pdl = ((rl.early || rl.behind) && g_pdl && !rl.programmatic_event) ? 1u : 0u;
+    a.early = (a.pdl && rl.early && (rl.mode != SIFAR_BARRIER_ONESHOT || g_barrier_early)) ? 1u : 0u;
     /* Large plain-format call whose producers run on other streams and have not all finished: their data
        may be late, and what the grid then queues is swept by a kernel of its own (see k_sweep) instead of
        the grid's janitors.  Not while capturing (a stream may not be queried then, and a graph's replays
@@ -1298,16 +1332,37 @@ static cudaError_t launch_ready_dt(int P, bool barrier, int grid, cudaStream_t s
     }
 }
 
+/* Launch with programmatic stream serialization: the kernel may become resident before the one ahead of it on the
+   stream is complete, and waits for that inside (griddepcontrol.wait). */
+template <typename... Params, typename... Args>
+static cudaError_t launch_dependent(void (*kernel)(Params...), int grid, int threads, cudaStream_t s, Args... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads); cfg.stream = s;
+    cfg.attrs = at; cfg.numAttrs = g_pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
+template <int DT, int MODE>
+static cudaError_t launch_pack_mode(int grid, bool dependent, cudaStream_t s, const PackArgs &a)
+{
+    if (dependent) return launch_dependent(k_pack<DT, MODE>, grid, kThreads, s, a);
+    k_pack<DT, MODE><<<grid, kThreads, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <int DT>
-static cudaError_t launch_pack_dt(int mode, int grid, cudaStream_t s, const PackArgs &a)
+static cudaError_t launch_pack_dt(int mode, int grid, bool dependent, cudaStream_t s, const PackArgs &a)
 {
     switch (mode) {
-    case SIFAR_BARRIER_ONESHOT: k_pack<DT, SIFAR_BARRIER_ONESHOT><<<grid, kThreads, 0, s>>>(a); break;
-    case SIFAR_DUALBUF:         k_pack<DT, SIFAR_DUALBUF><<<grid, kThreads, 0, s>>>(a); break;
-    case kModeTiles:            k_pack<DT, kModeTiles><<<grid, kThreads, 0, s>>>(a); break;
-    default:                    k_pack<DT, SIFAR_SPECULATIVE><<<grid, kThreads, 0, s>>>(a); break;
+    case SIFAR_BARRIER_ONESHOT: return launch_pack_mode<DT, SIFAR_BARRIER_ONESHOT>(grid, dependent, s, a);
+    case SIFAR_DUALBUF:         return launch_pack_mode<DT, SIFAR_DUALBUF>(grid, dependent, s, a);
+    case kModeTiles:            return launch_pack_mode<DT, kModeTiles>(grid, dependent, s, a);
+    default:                    return launch_pack_mode<DT, SIFAR_SPECULATIVE>(grid, dependent, s, a);
     }
-    return cudaGetLastError();
 }
 
 }  /* namespace sifar */
@@ -1543,8 +1598,10 @@ extern "C" int sifar_allreduce(sifar_ctx *c, const void *const *rank_ptrs, void 
        while that kernel drains (its writes still wait).  Unknown producers (partials stored by the
        caller's own kernels without sifar_arrive) or the same stream: the plain stream order. */
     rl.early = (stream != nullptr);
+    rl.behind = true;
     for (int r = 0; r < c->P; ++r) {
-        if (c->prod_epoch[r] != e) { rl.early = false; continue; }
+        if (c->prod_epoch[r] != e) { rl.early = rl.behind = false; continue; }
+        if (c->prod_stream[r] != (cudaStream_t)stream) rl.behind = false;
         if (c->prod_stream[r] == (cudaStream_t)stream || c->prod_stream[r] == nullptr) rl.early = false;
         if (c->prod_n[r] != (size_t)-1 && c->prod_n[r] != n && mode == SIFAR_SPECULATIVE &&
             spec_format(c->P, c->dtype, c->prod_n[r]) != rl.format) {
@@ -1625,9 +1682,13 @@ extern "C" int sifar_pack(sifar_ctx *c, int rank, const void *src, size_t n, int
     const size_t cap = (size_t)c->sm_count * 2;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
+    /* A grid of at most one CTA per SM may get ready while the kernel before it on the stream still runs (a client
+       that packs its ranks one after another on one stream).  Larger grids would hold room that kernels of other
+       streams, the ranks that a reducer waits for among them, need meanwhile. */
+    const bool dependent = grid <= (size_t)c->sm_count;
     cudaError_t err = (c->dtype == SIFAR_BF16)
-        ? launch_pack_dt<SIFAR_BF16>(kernel_mode, (int)grid, (cudaStream_t)stream, a)
-        : launch_pack_dt<SIFAR_F32>(kernel_mode, (int)grid, (cudaStream_t)stream, a);
+        ? launch_pack_dt<SIFAR_BF16>(kernel_mode, (int)grid, dependent, (cudaStream_t)stream, a)
+        : launch_pack_dt<SIFAR_F32>(kernel_mode, (int)grid, dependent, (cudaStream_t)stream, a);
     SIFAR_CUDA(err);
     note_producer(c, rank, e, (cudaStream_t)stream, n);
     return SIFAR_OK;
@@ -1643,8 +1704,7 @@ extern "C" int sifar_arrive(sifar_ctx *c, int rank, int mode, void *stream)
     }
     uint32_t e;
     if ((rc = next_epoch(c, "sifar_arrive", &e))) return rc;
-    k_arrive<<<1, 1, 0, (cudaStream_t)stream>>>(c->d_state, c->d_status_alias, (uint32_t)rank, e & 1u);
-    SIFAR_CUDA(cudaGetLastError());
+    SIFAR_CUDA(launch_dependent(k_arrive, 1, 1, (cudaStream_t)stream, c->d_state, c->d_status_alias, (uint32_t)rank, e & 1u));
     note_producer(c, rank, e, (cudaStream_t)stream, (size_t)-1);
     return SIFAR_OK;
 }
@@ -1655,10 +1715,12 @@ extern "C" int sifar_wait_writable(sifar_ctx *c, int rank, void *stream)
     if (rc) return rc;
     if (rank < 0 || rank >= c->P) { set_error("sifar_wait_writable: bad rank"); return SIFAR_ERR_INVALID; }
     if (!c->last_mode0_epoch) return SIFAR_OK;      /* nothing has read the buffer yet */
+    /* The previous call's reducer went onto this very stream: what follows here is behind it, and it sets the done
+       flags and the call number that the kernel would look for. */
+    if (c->last_call_stream && c->last_call_stream == stream_key((cudaStream_t)stream)) return SIFAR_OK;
     const uint32_t delta = c->h_epoch + 1u - c->last_mode0_epoch;
-    k_wait_writable<<<1, 1, 0, (cudaStream_t)stream>>>(c->d_state, c->d_status_alias, (uint32_t)rank, delta,
-                                                       (c->h_epoch + 1u) & 1u, c->timeout_ns);
-    SIFAR_CUDA(cudaGetLastError());
+    SIFAR_CUDA(launch_dependent(k_wait_writable, 1, 1, (cudaStream_t)stream, c->d_state, c->d_status_alias, (uint32_t)rank,
+                                delta, (c->h_epoch + 1u) & 1u, c->timeout_ns));
     return SIFAR_OK;
 }
 

@@ -137,6 +137,7 @@ struct ReduceLaunch {
     cudaEvent_t programmatic_event;  /* NULL, or an event the kernel fires as soon as all its CTAs have started */
     int format;                      /* SPECULATIVE: SIFAR_FORMAT_SLOTS or SIFAR_FORMAT_TILES                   */
     const uint32_t *tile_flags;      /* SIFAR_FORMAT_TILES: the flag array of this call's parity                */
+    bool behind;                     /* all producers were enqueued on the reducer's own stream                  */
     bool early;                      /* the producers are known to run on other streams: reads need not wait for
                                         the kernel before this one on the stream (see the reducer kernels)       */
 };
