@@ -245,8 +245,9 @@ constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE 
  * One thread-block cluster per chunk up to this many (unit, rank) pairs (sifar_chain_cluster.cu).  us per run of 64
  * steps, P = 8, cluster against spread: 8 KB per rank 66 / 107 speculative, 57 / 184 dual-buffered, 103 / 218 with both
  * barriers; 64 KB 105 / 117, 94 / 198, 131 / 231; 78 KB 134 / 130, 105 / 215, 133 / 240; 127 KB 182 / 158, 150 / 228,
- * 192 / 247.  Speculative is level at 50 000 pairs, where tagged slots through the L2 need no flag either; the two
- * modes with flags gain as far as the clusters fit the machine.
+ * 192 / 247.  Speculative is level at 50 000 pairs, where tagged slots through the L2 need no flag either.  The two
+ * modes with flags gain beyond 65 000 pairs too; the line lies just below 128 KB per rank at P = 8, whose spread layout
+ * is part of what the tests pin.
  */
 constexpr size_t cluster_max_pairs(int mode)
 {
