@@ -5,7 +5,7 @@
 
 One "step" is one decode step of the Llama-3.1-8B-shaped workload: 64 dependent
 {8 producers -> all-reduce} iterations on P=8 ranks of 4096 bf16 (8 KB per rank),
-run as ONE persistent cooperative kernel in speculative mode (the paper measures
+run as ONE persistent kernel in speculative mode (the paper measures
 all-reduce latency back to back inside a fused forward-pass kernel).  The line
 printed on stdout is one JSON object; `value` is the p50 time between two
 consecutive all-reduce results in microseconds.
@@ -563,8 +563,21 @@ def measure_symmetric(sf, torch, synth, ranks, n, name="llama", steps=ARS_PER_ST
 def verification_overhead(sf, torch, synth, shapes=((8, 4096), (8, 16384), (2, 4096)), forced=(1, 2, 3)):
     """Section 6.3, "Mis-Speculation and Verification Overhead" and "Retry Overhead", in the chain with P readers:
     p50 per all-reduce of the two validation schemes (the paper's per-threadblock flags, tags inside the slots)
-    over the same pull without any validation, and what each forced retry adds to either."""
+    over the same pull without any validation, and what each forced retry adds to either.  The paper's scheme and
+    the unchecked pull exist through the L2 only, so the others are held to the same layout here (the chains run as
+    clusters by default)."""
     out = {}
+    saved = os.environ.get("SIFAR_CHAIN_CLUSTER")
+    os.environ["SIFAR_CHAIN_CLUSTER"] = "0"
+    try:
+        return _verification_rows(sf, torch, synth, shapes, forced, out)
+    finally:
+        os.environ.pop("SIFAR_CHAIN_CLUSTER")
+        if saved is not None:
+            os.environ["SIFAR_CHAIN_CLUSTER"] = saved
+
+
+def _verification_rows(sf, torch, synth, shapes, forced, out):
     for P_, n in shapes:
         run = lambda mode, k=0: _sym_run(sf, torch, synth, P_, n, mode, "llama", ARS_PER_STEP, 3, 6, forced=k)["p50_us"]
         base = run(sf.SYMCHAIN_UNCHECKED)
@@ -740,8 +753,8 @@ def run_gpu(args) -> None:
         windows.append((w0, time.time()))
         e2e = {"value": round(pct(per_call, 50), 2), "unit": "us", "p99": round(pct(per_call, 99), 2),
                "h2d_bytes_per_step": ARS_PER_STEP * P * n * 2, "d2h_bytes_per_step": ARS_PER_STEP * n * 2,
-               "what": "sifar_allreduce_host on pinned host buffers: one kernel packs the 8 partials straight from "
-                       "host memory (H2D inside the kernel), one reduces and writes the result to host memory, then "
+               "what": "sifar_allreduce_host on pinned host buffers: one kernel reads the 8 partials straight from "
+                       "host memory (H2D inside the kernel), sums them and writes the result to host memory, then "
                        "a stream synchronisation; per call"}
         # -- 5. CPU oracle ---------------------------------------------------------------------------
         from oracle import oracle
