@@ -1263,8 +1263,8 @@ int launch_reduce(sifar_ctx *ctx, const ReduceLaunch &rl, cudaStream_t stream)
 /*
  * With lazy module loading (the CUDA default) the first launch of a kernel loads its code, and that load
  * can wait for the device to become idle.  Producers are routinely launched for the first time while a
- * reducer is already polling for them, so such a launch would block on the host until the reducer gave
- * up.  Every kernel of a context's shape is therefore loaded when the context is created.
+ * reducer is already polling for them (and a host call on one context while another context's reducer
+ * waits for its packs), so such a launch would block on the host until the reducer gave up.  Every kernel of a context's shape is therefore loaded when the context is created.
  */
 template <typename K>
 static cudaError_t preload(K kernel)
@@ -1283,6 +1283,8 @@ static cudaError_t preload_reducers()
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, SIFAR_BARRIER_ONESHOT>);
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, SIFAR_DUALBUF>);
     if (e == cudaSuccess) e = preload(k_sweep<DT, P, kModeTiles>);
+    if (e == cudaSuccess) e = preload(k_reduce_ready<DT, P, false>);
+    if (e == cudaSuccess) e = preload(k_reduce_ready<DT, P, true>);
     return e;
 }
 

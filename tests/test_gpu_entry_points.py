@@ -1,5 +1,10 @@
 """Calls that need no protocol between streams: partials in host memory, caller buffers and packs on one stream, and
 the allocation-free call on two streams at once."""
+import os
+import subprocess
+import sys
+import textwrap
+
 import numpy as np
 import pytest
 import torch
@@ -54,6 +59,42 @@ def test_a_host_result_may_lie_on_a_partial(oracle, pinned, shift):
         at = base[1] + shift
         sf.sifar_allreduce_host(ctx.h, [flat.data_ptr() + 2 * b for b in base], flat.data_ptr() + 2 * at, n, sf.SPECULATIVE)
         assert_bits_equal(flat.numpy()[at: at + n].view(np.uint16), oracle.allreduce(xs, BF16), BF16, f"shift {shift}")
+
+
+def _in_a_process_of_its_own(code, **env):
+    """Loaded kernels and the switches that are read at load time belong to a process."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    out = subprocess.run([sys.executable, "-c", textwrap.dedent(code)], capture_output=True, text=True, timeout=300,
+                         cwd=os.path.dirname(here),
+                         env=dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(here), here]), **env))
+    assert out.returncode == 0, out.stdout + out.stderr
+    return out.stdout
+
+
+@pytest.mark.parametrize("mode", MODES)
+def test_the_first_host_call_beside_a_reducer_that_waits_for_a_late_pack(mode):
+    """The process's first host call is made while another context's reducer polls for a pack that the same thread
+    enqueues afterwards: it may not wait for the device to become idle (its kernel is loaded with the context)."""
+    _in_a_process_of_its_own(f"""
+        import torch
+        from paper_2607_08973_b200 import binding as sf
+        n, mode = 4096, {mode}
+        waiting, host = sf.sifar_create(2, n, sf.BF16), sf.sifar_create(3, n, sf.F32)
+        sf.sifar_set_timeout_us(waiting, 2_000_000)
+        x = [torch.ones(n, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        out = torch.zeros(n, dtype=torch.bfloat16, device="cuda")
+        hx = [torch.full((n,), float(r + 1)).pin_memory() for r in range(3)]
+        hout = torch.zeros(n).pin_memory()
+        packs, red = [torch.cuda.Stream() for _ in range(2)], torch.cuda.Stream()
+        torch.cuda.synchronize()
+        sf.sifar_pack(waiting, 0, x[0].data_ptr(), n, mode, packs[0].cuda_stream)
+        sf.sifar_allreduce(waiting, None, out.data_ptr(), n, mode, red.cuda_stream)
+        sf.sifar_allreduce_host(host, [t.data_ptr() for t in hx], hout.data_ptr(), n, mode)
+        sf.sifar_pack(waiting, 1, x[1].data_ptr(), n, mode, packs[1].cuda_stream)
+        torch.cuda.synchronize()
+        assert sf.sifar_status(waiting) == 0 and sf.sifar_get_stats(waiting)["timeouts"] == 0
+        assert bool((out == 2).all()) and bool((hout == 6).all())
+        """)
 
 
 @pytest.mark.parametrize("mode", MODES)
