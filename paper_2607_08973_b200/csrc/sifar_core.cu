@@ -1212,35 +1212,30 @@ int launch_reduce(sifar_ctx *ctx, const ReduceLaunch &rl, cudaStream_t stream)
     /* Early reads need programmatic launch to mean anything, and the baseline keeps the plain stream order. */
     a.pdl = ((rl.early || rl.behind) && g_pdl && !rl.programmatic_event) ? 1u : 0u;
     a.early = (a.pdl && rl.early && (rl.mode != SIFAR_BARRIER_ONESHOT || g_barrier_early)) ? 1u : 0u;
-    /* Are the producers done?  Asked where the answer changes the launch, until one is seen that is not: a large
-       plain-format call whose producers run on other streams and have not all finished leaves what its grid queues to
-       a sweep kernel of its own (see k_sweep) instead of the grid's janitors; and the formats whose janitors cannot
-       know that every tile's data is there let the next kernel in at once where all are done (back to back on ready
-       data, P = 8, speculative: 3.2 against 4.7 us per call at 512 KB per rank, 4.4 against 7.6 at 2 MiB).  Not
-       while capturing (a stream may not be queried then, and a graph's replays meet other conditions than its capture
-       did). */
-    const bool other_streams = rl.early && a.e_host && !rl.programmatic_event;
-    const bool large_plain = other_streams && kernel_mode != SIFAR_SPECULATIVE &&
+    /* Are the producers done?  A large plain-format call whose producers run on other streams and have not all
+       finished leaves what its grid queues to a sweep kernel of its own (see k_sweep) instead of the grid's janitors;
+       where all are done the next kernel is let in at once.  No other call asks, whatever it could gain (back to back
+       on ready data, P = 8, speculative, 3.2 against 4.7 us per call at 512 KB per rank and 4.4 against 7.6 at 2 MiB):
+       a producer's stream has to outlive sifar_pack only where sifar.h says so.  Not while capturing (a stream may not
+       be queried then, and a graph's replays meet other conditions than its capture did). */
+    const bool large_plain = rl.early && a.e_host && !rl.programmatic_event && kernel_mode != SIFAR_SPECULATIVE &&
                              ntiles >= (size_t)kSweepFromTilesPerSm * (size_t)ctx->sm_count;
-    const bool per_tile = kernel_mode == SIFAR_SPECULATIVE || kernel_mode == kModeTiles;
-    bool busy = large_plain && ctx->sweep_policy == SIFAR_SWEEP_ALWAYS, done = !busy;
-    if (large_plain || (other_streams && per_tile && a.two_phase)) {
-        for (int r = 0; r < ctx->P && !busy; ++r) {
-            /* a stream that is being captured may not be queried (the capture would be invalidated) */
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-            if (cudaStreamIsCapturing(ctx->prod_stream[r], &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-                cudaGetLastError();
-                done = false;
-                continue;
-            }
-            const cudaError_t q = cudaStreamQuery(ctx->prod_stream[r]);
-            if (q == cudaErrorNotReady) busy = true;
-            if (q != cudaSuccess) { done = false; cudaGetLastError(); }      /* "not ready" is an answer, not an error */
+    bool busy = large_plain && ctx->sweep_policy == SIFAR_SWEEP_ALWAYS;
+    const bool ask = large_plain && ctx->sweep_policy == SIFAR_SWEEP_AUTO;
+    bool done = ask;
+    for (int r = 0; ask && r < ctx->P && !busy; ++r) {
+        /* a stream that is being captured may not be queried (the capture would be invalidated) */
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+        if (cudaStreamIsCapturing(ctx->prod_stream[r], &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            done = false;
+            continue;
         }
-    } else {
-        done = false;
+        const cudaError_t q = cudaStreamQuery(ctx->prod_stream[r]);
+        if (q == cudaErrorNotReady) busy = true;
+        if (q != cudaSuccess) { done = false; cudaGetLastError(); }      /* "not ready" is an answer, not an error */
     }
-    a.sweeper = (large_plain && busy && ctx->sweep_policy != SIFAR_SWEEP_NEVER) ? 1u : 0u;
+    a.sweeper = busy ? 1u : 0u;
     /* producers on the reducer's own stream are complete before it reads anything */
     a.let_in = (rl.programmatic_event || rl.behind || done) ? 1u : 0u;
     /* with the sweep kernel behind it the grid need not hold the machine for tiles that are not there yet */

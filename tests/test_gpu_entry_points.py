@@ -178,3 +178,30 @@ def test_noalloc_calls_on_two_streams_are_both_booked(oracle):
     assert sf.sifar_noalloc_counters() == {"cta_arrive": 0, "calls": before + 40, "elements": n}
     for out in outs:
         assert_bits_equal(out_to_numpy(out, n, BF16)[0], want, BF16, "two streams")
+
+
+@pytest.mark.parametrize("n,mode,policy", [(4096, sf.SPECULATIVE, None), (262_144, sf.SPECULATIVE, None),
+                                           (1 << 20, sf.SPECULATIVE, None), (1 << 20, sf.DUALBUF, None)] +
+                         [(4 << 20, mode, sf.SWEEP_NEVER) for mode in MODES] +
+                         [(4 << 20, mode, sf.SWEEP_ALWAYS) for mode in MODES])
+def test_producer_streams_may_go_once_their_packs_are_enqueued(oracle, n, mode, policy):
+    """Slots, block flags below 8 tiles per SM, and any size where the policy says that the streams are not asked."""
+    from cuda.bindings import runtime as rt
+    P = 8
+    xs = synth.rank_inputs(P, n, BF16, 77, "gauss")
+    xd, out = [to_device(x) for x in xs], empty_out(n, BF16)
+    red = torch.cuda.Stream()
+    with Ctx(P, n, BF16) as ctx:
+        if policy is not None:
+            sf.sifar_debug_sweep_policy(ctx.h, policy)
+        torch.cuda.synchronize()
+        for _ in range(2):
+            for r in range(P):
+                err, s = rt.cudaStreamCreateWithFlags(rt.cudaStreamNonBlocking)
+                assert err == rt.cudaError_t.cudaSuccess
+                sf.sifar_pack(ctx.h, r, xd[r].data_ptr(), n, mode, int(s))
+                assert rt.cudaStreamDestroy(s)[0] == rt.cudaError_t.cudaSuccess       # its work goes on
+            sf.sifar_allreduce(ctx.h, None, out.data_ptr(), n, mode, red.cuda_stream)
+            torch.cuda.synchronize()
+            assert sf.sifar_status(ctx.h) == 0
+            assert_bits_equal(out_to_numpy(out, n, BF16)[0], oracle.allreduce(xs, BF16), BF16, f"n={n} mode={mode}")
