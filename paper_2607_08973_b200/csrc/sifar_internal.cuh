@@ -120,10 +120,15 @@ namespace sifar {
 void set_error(const char *fmt, ...);
 int cuda_fail(cudaError_t e, const char *what);
 
+/* An error that has been reported is not left for the next cudaGetLastError() to find (each library has a CUDA
+   runtime of its own, so this is done where the call was made). */
 #define SIFAR_CUDA(call)                                                   \
     do {                                                                   \
         cudaError_t e__ = (call);                                          \
-        if (e__ != cudaSuccess) return ::sifar::cuda_fail(e__, #call);     \
+        if (e__ != cudaSuccess) {                                          \
+            cudaGetLastError();                                            \
+            return ::sifar::cuda_fail(e__, #call);                         \
+        }                                                                  \
     } while (0)
 
 /* Internal launchers, implemented in sifar_core.cu, used by the chains too. */

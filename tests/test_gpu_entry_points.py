@@ -205,3 +205,37 @@ def test_producer_streams_may_go_once_their_packs_are_enqueued(oracle, n, mode, 
             torch.cuda.synchronize()
             assert sf.sifar_status(ctx.h) == 0
             assert_bits_equal(out_to_numpy(out, n, BF16)[0], oracle.allreduce(xs, BF16), BF16, f"n={n} mode={mode}")
+
+
+@pytest.mark.parametrize("entry", ["noalloc", "pack", "arrive"])
+def test_a_launch_that_cuda_refuses_leaves_no_error_for_the_next_call(oracle, entry):
+    """The legacy stream may not be used while a blocking stream is being captured.  The call reports that, once."""
+    from cuda.bindings import runtime as rt
+    n = 4096
+    xs = synth.rank_inputs(1, n, BF16, 3, "gauss")
+    x, out = to_device(xs[0]), empty_out(n, BF16)
+    sf.sifar_allreduce_noalloc([x.data_ptr()], out.data_ptr(), n, BF16, 0)            # resolves its array
+    s = torch.cuda.Stream()
+    err, capturing = rt.cudaStreamCreate()
+    assert err == rt.cudaError_t.cudaSuccess
+    with Ctx(1, n, BF16) as ctx:
+        torch.cuda.synchronize()
+        assert rt.cudaStreamBeginCapture(capturing, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)[0] == 0
+        try:
+            with pytest.raises(sf.SifarError) as ei:
+                if entry == "noalloc":
+                    sf.sifar_allreduce_noalloc([x.data_ptr()], out.data_ptr(), n, BF16, 0)
+                elif entry == "pack":
+                    sf.sifar_pack(ctx.h, 0, x.data_ptr(), n, sf.SPECULATIVE, 0)
+                else:
+                    sf.sifar_arrive(ctx.h, 0, sf.DUALBUF, 0)
+            assert ei.value.code == sf.ERR_CUDA
+        finally:
+            rt.cudaStreamEndCapture(capturing)                                        # invalidated by then
+            rt.cudaStreamDestroy(capturing)
+        sf.sifar_allreduce(ctx.h, None, out.data_ptr(), 0, sf.SPECULATIVE, s.cuda_stream)      # nothing to add: a plain launch
+        sf.sifar_pack(ctx.h, 0, x.data_ptr(), n, sf.SPECULATIVE, s.cuda_stream)
+        sf.sifar_allreduce(ctx.h, None, out.data_ptr(), n, sf.SPECULATIVE, s.cuda_stream)
+        torch.cuda.synchronize()
+        assert sf.sifar_status(ctx.h) == 0
+        assert_bits_equal(out_to_numpy(out, n, BF16)[0], xs[0], BF16, entry)
