@@ -36,13 +36,19 @@
  *                           this many (slot, rank) pairs, wait on a sentinel slot above (170000)
  *   SIFAR_CHAIN_PDL         0 = stream / graph chains record the step events the plain way (by default the
  *                           all-reduce of a step fires its event as soon as all its CTAs have started, and the
- *                           next step's producers wait inside the kernel for its completion)
- *   SIFAR_PDL               0 = reducers are launched without programmatic dependent launch (read when the
- *                           library is loaded).  By default a reducer with more CTAs than the GPU has SMs,
- *                           or one whose producers were all enqueued on other streams, may become resident
- *                           while the kernel before it on its stream drains.  In the two barrier-free modes
- *                           its loads then start at once (they are ordered by flags or tags, not by the
- *                           stream); everything it writes waits until that kernel is complete.
+ *                           next step's producers wait inside the kernel for its completion), and a run of a
+ *                           persistent chain in clusters starts when the kernel before it on its stream is over (by
+ *                           default its prologue overlaps that kernel's end); read at the first such launch of the
+ *                           process
+ *   SIFAR_PDL               0 = every kernel of libsifar.so is launched without programmatic dependent launch (read
+ *                           when the library is loaded).  By default a kernel of one of these kinds may become
+ *                           resident while the kernel before it on its stream drains: a reducer with more CTAs than
+ *                           the GPU has SMs, one whose producers were all enqueued on other streams or all on its
+ *                           own (sifar_pack, sifar_arrive), the sweep kernel, a pack of at most one CTA per SM,
+ *                           sifar_arrive, sifar_wait_writable and sifar_allreduce_noalloc.  In the two barrier-free
+ *                           modes the loads of a reducer whose producers are on other streams then start at once
+ *                           (they are ordered by flags or tags, not by the stream); everything else that such a
+ *                           kernel reads or writes waits until the kernel before it is complete.
  *   SIFAR_BARRIER_EARLY     1 = the loads of a BARRIER_ONESHOT reducer may start early as well (they are ordered by
  *                           its arrival flags); off by default, the baseline keeps the conventional stream order
  *                           (read when the library is loaded)
@@ -228,6 +234,9 @@ int sifar_arrive(sifar_ctx *ctx, int rank, int mode, void *stream);
  * barrier, a bounded wait until the reducer of the previous call has released
  * `rank`'s done flag.  Enqueue it before the kernel that overwrites the buffer,
  * and after the previous call's reducer in stream or event order (ordering contract).
+ * Nothing is enqueued where there is nothing to wait for: before the first
+ * BARRIER_ONESHOT call, and on the stream that the previous call's reducer went onto
+ * (outside stream capture), where whatever follows is behind that reducer anyway.
  */
 int sifar_wait_writable(sifar_ctx *ctx, int rank, void *stream);
 

@@ -1020,13 +1020,15 @@ __global__ void k_set_epoch(DevState *st, uint32_t e) { st->epoch = e; st->cta_a
 /* launch geometry                                                           */
 /* ------------------------------------------------------------------------ */
 /*
- * Programmatic dependent launch: a reducer may become resident while the kernel before it on its stream
- * is still draining.  Its CTAs then sit in griddepcontrol.wait until that kernel has completed and its
- * writes are visible, so what they read is unchanged; what is saved is the launch gap and the ramp-up
- * between back-to-back kernels (about 2 us per pair).  Used for reducer grids above the SM count, where
- * bandwidth is what counts.  SIFAR_PDL=0 launches the plain way.
+ * Programmatic dependent launch: a kernel may become resident while the kernel before it on its stream is still
+ * draining.  Its CTAs then sit in griddepcontrol.wait until that kernel has completed and its writes are visible, so
+ * what they read is unchanged; what is saved is the launch gap and the ramp-up between back-to-back kernels (about
+ * 2 us per pair).  Used for reducers above the SM count or whose producers were all enqueued with the library (see
+ * launch_k), their sweep kernel, packs of at most one CTA per SM, the one-thread kernels of callers that store for
+ * themselves, and the allocation-free call.  SIFAR_PDL=0 launches all of them the plain way.
  */
 static bool g_pdl = !(getenv("SIFAR_PDL") && atoi(getenv("SIFAR_PDL")) == 0);
+bool dependent_launches() { return g_pdl; }
 /* SIFAR_BARRIER_EARLY=1: the baseline's reads may start early too (they are ordered by its arrival flags just as
    well); off by default: the baseline stands for the conventional design, which orders everything by the stream. */
 static bool g_barrier_early = getenv("SIFAR_BARRIER_EARLY") && atoi(getenv("SIFAR_BARRIER_EARLY")) != 0;

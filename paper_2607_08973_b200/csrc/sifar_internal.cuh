@@ -119,6 +119,7 @@ namespace sifar {
 /* Error text of the calling thread. */
 void set_error(const char *fmt, ...);
 int cuda_fail(cudaError_t e, const char *what);
+bool dependent_launches();               /* false: SIFAR_PDL=0 when the library was loaded */
 
 /* An error that has been reported is not left for the next cudaGetLastError() to find (each library has a CUDA
    runtime of its own, so this is done where the call was made). */

@@ -45,7 +45,7 @@ struct NoallocArgs {
  * for the kernel).  The memset that cleared it was the greater part of a row of small
  * calls: 6.1 us a call before, 3.6 us after (2 KB per rank; 5.1 us at 128 KB).
  * The launch may overlap the end of the kernel before it on the stream
- * (programmatic launch); nothing is read before that kernel is complete.
+ * (programmatic launch, unless SIFAR_PDL=0); nothing is read before that kernel is complete.
  */
 template <int DT, int P>
 __global__ void __launch_bounds__(kNoallocThreads) k_reduce_noalloc(const NoallocArgs a)
@@ -198,7 +198,7 @@ extern "C" int sifar_allreduce_noalloc(const void *const *rank_ptrs, int P, void
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kNoallocThreads); cfg.stream = (cudaStream_t)stream;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    cfg.attrs = at; cfg.numAttrs = dependent_launches() ? 1 : 0;
     cudaError_t err = (dtype == SIFAR_BF16) ? launch_noalloc_dt<SIFAR_BF16>(P, cfg, a) : launch_noalloc_dt<SIFAR_F32>(P, cfg, a);
     SIFAR_CUDA(err);
     return SIFAR_OK;

@@ -239,3 +239,54 @@ def test_a_launch_that_cuda_refuses_leaves_no_error_for_the_next_call(oracle, en
         torch.cuda.synchronize()
         assert sf.sifar_status(ctx.h) == 0
         assert_bits_equal(out_to_numpy(out, n, BF16)[0], xs[0], BF16, entry)
+
+
+@pytest.mark.parametrize("pdl", ["1", "0"])
+@pytest.mark.parametrize("entry", ["noalloc", "packs", "arrivals"])
+def test_dependent_launches_follow_the_switch(entry, pdl):
+    """A captured row of launches shows how each was launched: a programmatic edge to the kernel before it, or a full
+    one.  With SIFAR_PDL=0 the plain stream order is back in all of them."""
+    out = _in_a_process_of_its_own(f"""
+        import torch
+        from cuda.bindings import runtime as rt
+        from paper_2607_08973_b200 import binding as sf
+        P, n, entry = 4, 4096, "{entry}"
+        x = [torch.ones(n, dtype=torch.bfloat16, device="cuda") for _ in range(P)]
+        out = torch.zeros(n, dtype=torch.bfloat16, device="cuda")
+        ptrs, s = [t.data_ptr() for t in x], torch.cuda.Stream().cuda_stream
+        ctx = sf.sifar_create(P, n, sf.BF16)
+        sf.sifar_allreduce_noalloc(ptrs, out.data_ptr(), n, sf.BF16, s)
+        torch.cuda.synchronize()
+        assert rt.cudaStreamBeginCapture(s, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)[0] == 0
+        if entry == "noalloc":
+            for _ in range(3):
+                sf.sifar_allreduce_noalloc(ptrs, out.data_ptr(), n, sf.BF16, s)
+        else:
+            for call in range(2):
+                for r in range(P):
+                    if entry == "packs":
+                        sf.sifar_pack(ctx, r, ptrs[r], n, sf.SPECULATIVE, s)
+                    else:
+                        sf.sifar_wait_writable(ctx, r, s)
+                        sf.sifar_arrive(ctx, r, sf.BARRIER_ONESHOT, s)
+                sf.sifar_allreduce(ctx, ptrs if entry == "arrivals" else None, out.data_ptr(), n,
+                                   sf.BARRIER_ONESHOT if entry == "arrivals" else sf.SPECULATIVE, s)
+        err, graph = rt.cudaStreamEndCapture(s)
+        assert err == 0
+        err, _, _, _, k = rt.cudaGraphGetEdges_v2(graph)
+        err, _, _, data, k = rt.cudaGraphGetEdges_v2(graph, k)
+        assert err == 0 and k > 0
+        kinds = [int(d.type) for d in data[:k]]
+        err, ex = rt.cudaGraphInstantiate(graph, 0)
+        assert err == 0
+        for _ in range(3):                                        # the call number advances on the device
+            out.zero_()
+            torch.cuda.synchronize()
+            assert rt.cudaGraphLaunch(ex, s)[0] == 0
+            torch.cuda.synchronize()
+            assert bool((out == P).all()) and sf.sifar_status(ctx) == 0
+        rt.cudaGraphExecDestroy(ex)
+        print(len(kinds), sum(k == int(rt.cudaGraphDependencyType.cudaGraphDependencyTypeProgrammatic) for k in kinds))
+        """, SIFAR_PDL=pdl)
+    edges, programmatic = map(int, out.split()[-2:])
+    assert edges > 0 and programmatic == (edges if pdl == "1" else 0)
