@@ -7,8 +7,9 @@ One "step" is one decode step of the Llama-3.1-8B-shaped workload: 64 dependent
 {8 producers -> all-reduce} iterations on P=8 ranks of 4096 bf16 (8 KB per rank),
 run as ONE persistent kernel in speculative mode (the paper measures
 all-reduce latency back to back inside a fused forward-pass kernel).  The line
-printed on stdout is one JSON object; `value` is the p50 time between two
-consecutive all-reduce results in microseconds.
+printed on stdout is one short JSON object (see headline()); `value` is the p50 time
+between two consecutive all-reduce results in microseconds.  The whole record, with
+every section below, goes to stderr as one JSON line, or to the file of --record.
 
 Sections measured by the default run (all on the device, CUDA events on the
 launching stream; per-all-reduce percentiles from %globaltimer stamps written by
@@ -21,7 +22,7 @@ the kernel):
      64 MiB per rank                                         -> by_payload
   4. the two validation schemes over an unchecked pull        -> detail.verification_overhead
   5. large-payload reducer kernel, inputs larger than L2     -> roofline
-  6. host-buffer entry point (H2D + pack + reduce + D2H)      -> e2e
+  6. host-buffer entry point (H2D + reduce + D2H)             -> e2e
   7. the CPU oracle on the host cores (bounded sample)        -> cpu_baseline
 --sweep adds every batch size, the stream chains, the whole payload sweep, the
 retry-overhead table, the late-producer section at three sizes and the two forms of
@@ -50,9 +51,9 @@ P, HIDDEN, ARS_PER_STEP = 8, 4096, 64
 LARGE_N = 8 << 20                      # 16 MiB of bf16 per rank
 NOMINAL_GBS = 8000.0                   # the HBM3e figure the metric names
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the roofline kernel at LARGE_N, from the
-# ncu capture summarised in the file named below; refreshed whenever the reducer kernels change
+# ncu capture summarised in profiles/ under the kernel's name; refreshed whenever the reducer kernels change
 NCU_TRAFFIC = {"bytes": 147_380_224, "captured_at_commit": "6a27414",
-               "summary": "profiles/k_reduce_plain_bf16_P8_16MiB.md (134.28 MB read + 13.10 MB written, flagged tiles, the median of three captured launches)"}
+               "summary": "134.28 MB read + 13.10 MB written, flagged tiles, the median of three captured launches"}
 
 
 def read_peaks() -> tuple[float, str]:
@@ -618,6 +619,21 @@ def retry_overhead(sf, torch, synth, ranks=(2, 4, 8), kbytes=(8, 16, 32), forced
     return res
 
 
+def headline(record: dict) -> dict:
+    """The line for stdout: the keys a reader of the result needs, without the sections' tables.  Kept under 3000
+    characters, so that the end of a log holds all of it."""
+    def keep(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else d
+    line = {k: v for k, v in record.items() if not isinstance(v, dict) and k != "paper_context"}
+    line["config"] = keep(record["config"], "workload", "l2", "replicas")
+    line["clocks"] = record["clocks"]
+    line["e2e"] = keep(record["e2e"], "value", "unit", "p99", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    line["roofline"] = keep(record["roofline"], "bound", "kernel", "achieved", "peak", "unit", "frac", "peak_kind",
+                            "frac_of_8TBs_nominal", "kernel_us", "algorithmic_bytes", "traffic")
+    line["cpu_baseline"] = keep(record["cpu_baseline"], "value", "unit", "cores", "kind")
+    return line
+
+
 def run_gpu(args) -> None:
     import torch
     from paper_2607_08973_b200 import binding as sf
@@ -742,7 +758,7 @@ def run_gpu(args) -> None:
                                   "frac": round(pk_bytes / pk_s / 1e9 / peak_gbs, 4)}
         alg_d = sf.sifar_algorithmic_bytes(P, sf.BF16, n, sf.SPECULATIVE) * ARS_PER_STEP
         step_s = secs / args.steps if secs else float("inf")
-        roof_decode = {"bound": "latency", "kernel": "k_chain<bf16,P=8,speculative>", "achieved": round(alg_d / step_s / 1e9, 1),
+        roof_decode = {"bound": "latency", "kernel": "k_chain_cluster<bf16,P=8,speculative>", "achieved": round(alg_d / step_s / 1e9, 1),
                        "peak": peak_gbs, "unit": "GB/s", "frac": round(alg_d / step_s / 1e9 / peak_gbs, 5),
                        "note": "decode payloads are L2-resident and latency-bound; see detail.modes"}
         windows.append((w0, time.time()))
@@ -788,7 +804,7 @@ def run_gpu(args) -> None:
 
     clocks = sampler.stop(windows)
     if rank == 0:
-        line = {
+        record = {
             "metric": METRIC, "value": round(p50, 3), "unit": "us", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": round(secs / args.steps * 1e3, 5), "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "accumulator": "f32", "data": "synthetic",
@@ -811,7 +827,12 @@ def run_gpu(args) -> None:
             "paper_context": "8xH200: oneshot 8 KB TP8 transfer 4.01 us; best baseline 5.11 us -> SiFAR 2.44 us "
                              "(with in-switch redundant pull, not built here)",
         }
-        print(json.dumps(line))
+        if args.record:
+            with open(args.record, "w") as fh:
+                json.dump(record, fh)
+        else:
+            print(json.dumps(record), file=sys.stderr, flush=True)
+        print(json.dumps(headline(record)))
     dist.finalize()
 
 
@@ -822,6 +843,7 @@ def main() -> None:
     ap.add_argument("--warmup", type=int, default=None)
     ap.add_argument("--impl", default="sifar", choices=["sifar", "reference"])
     ap.add_argument("--sweep", action="store_true", help="also batch sizes 2..16 and the stream chain")
+    ap.add_argument("--record", metavar="FILE", help="write the whole record there instead of to stderr")
     ap.add_argument("--only", default="all", choices=["all", "decode", "roofline", "p_readers", "late", "late16"],
                     help="profiling aid: run the timed decode region only, the roofline section only, or the "
                          "P-reader chain only")
