@@ -290,3 +290,28 @@ def test_dependent_launches_follow_the_switch(entry, pdl):
         """, SIFAR_PDL=pdl)
     edges, programmatic = map(int, out.split()[-2:])
     assert edges > 0 and programmatic == (edges if pdl == "1" else 0)
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("dtype", [BF16, F32])
+def test_packs_around_the_size_from_which_threads_take_several_units(oracle, dtype, mode):
+    """Two CTAs of 256 threads per SM: up to there a thread has one unit, whose words travel ahead of the call number."""
+    P, threads = 2, 2 * 256 * torch.cuda.get_device_properties(0).multi_processor_count
+    per_unit = (3 if mode == sf.SPECULATIVE else 4) * (2 if dtype == BF16 else 1)
+    edge = threads * per_unit
+    sizes = [edge - per_unit, edge - 1, edge, edge + 1, edge + per_unit, edge + per_unit * 256 + 1]
+    assert sf.sifar_spec_format(P, dtype, max(sizes)) == sf.FORMAT_SLOTS
+    s = torch.cuda.Stream()
+    with Ctx(P, max(sizes), dtype) as ctx:
+        for n in sizes:
+            xs = synth.rank_inputs(P, n, dtype, 11 + n % 97, "gauss")
+            xd, out = [to_device(x) for x in xs], empty_out(n, dtype)
+            torch.cuda.synchronize()
+            for r in range(P):
+                sf.sifar_pack(ctx.h, r, xd[r].data_ptr(), n, mode, s.cuda_stream)
+            sf.sifar_allreduce(ctx.h, None, out.data_ptr(), n, mode, s.cuda_stream)
+            torch.cuda.synchronize()
+            assert sf.sifar_status(ctx.h) == 0
+            got, tail = out_to_numpy(out, n, dtype)
+            assert canary_ok(tail, dtype)
+            assert_bits_equal(got, oracle.allreduce(xs, dtype), dtype, f"n={n} mode={mode}")
