@@ -194,6 +194,10 @@ int sifar_allreduce(sifar_ctx *ctx, const void *const *rank_ptrs, void *out, siz
  * Pageable ones go through staging that the context allocates on the first such
  * call: a pinned buffer that the host fills, up to 32 KiB per partial, one copy to
  * the device per rank above.  host_out may be one of the partials or overlap them.
+ * All partials are there when the call is made, so nothing is packed, waited for or
+ * validated, whatever the mode: it decides only whether the done flags of the bottom
+ * barrier are released.  Forced retries (sifar_debug_force_retries) do not apply, and
+ * the call leaves the counters of re-loads and flag polls alone.
  * For end-to-end measurements and simple clients.
  */
 int sifar_allreduce_host(sifar_ctx *ctx, const void *const *host_rank_ptrs, void *host_out,
@@ -246,7 +250,9 @@ int sifar_status(sifar_ctx *ctx);
 /*
  * Copies eight counters (synchronizes the device):
  *   [0] calls completed        [1] calls in which at least one slot was re-loaded
- *   [2] slot re-loads          [3] arrival-flag polls that found the flag not yet set
+ *   [2] slot re-loads: loads of a slot that was not yet valid.  Where one lane waits for a whole warp on the last
+ *       slot of each rank (persistent chains on large grids and in clusters), the loads by that lane
+ *   [3] arrival-flag polls that found the flag not yet set
  *   [4] waits that timed out   [5] current call number on the device   [6],[7] reserved
  */
 int sifar_get_stats(sifar_ctx *ctx, unsigned long long out[8]);

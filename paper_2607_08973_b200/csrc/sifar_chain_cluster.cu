@@ -38,12 +38,21 @@ static_assert(kChainThreads == kBoxThreads, "one slot per thread");
 __device__ __forceinline__ void gdc_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void gdc_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 
+/*
+ * How many steps of this run the warps of every CTA of the cluster have made counted stores for, in the receiver's shared
+ * memory: as many as a whole run has, unless a warp gave up and said otherwise before it came to the cluster's last barrier.
+ */
+template <uint32_t SENDERS>
+struct Stored { uint32_t steps[SENDERS][kWarpsPerCta]; };
+
 /* Zero tags in `slots` slots of shared memory, mbarriers ready, every CTA of the cluster past this point. */
+template <uint32_t SENDERS>
 __device__ __forceinline__ void cluster_prologue(uint4 *box, uint32_t slots, unsigned long long (*top)[kWarpsPerCta],
                                                  unsigned long long (*hand)[kWarpsPerCta], unsigned long long *done,
-                                                 uint32_t done_count)
+                                                 uint32_t done_count, Stored<SENDERS> &stored, uint32_t steps)
 {
     for (uint32_t i = threadIdx.x; i < slots; i += kChainThreads) box[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x < SENDERS * kWarpsPerCta) (&stored.steps[0][0])[threadIdx.x] = steps;
     if (threadIdx.x < 2 * kWarpsPerCta) {
         mbar_init(smem_addr(&top[0][0] + threadIdx.x), 1u);
         if (hand) mbar_init(smem_addr(&hand[0][0] + threadIdx.x), 1u);
@@ -54,13 +63,50 @@ __device__ __forceinline__ void cluster_prologue(uint4 *box, uint32_t slots, uns
     cluster_sync();
 }
 
-/* After the last step.  A store into a CTA that has left would be an error, so nobody leaves before all are done; and
-   where somebody gave up, nobody waited for what was still on its way to this CTA, which 20 us more let land. */
-__device__ __forceinline__ void cluster_epilogue(DevState *st)
+/*
+ * After the last step.  A store into a CTA that has left would be an error, so nobody leaves before all are done.  Plain
+ * remote stores and arrivals have been performed by then; counted ones need not have been.  Where every wait came to
+ * its end they have all been waited for; true: somebody gave up, and what is still on its way to this CTA is to be
+ * waited for (mbar_drain).  (Whoever gave up has seen the context's status set before it came to the barrier.)
+ */
+__device__ __forceinline__ bool cluster_epilogue(DevState *st)
 {
     __syncwarp();
     cluster_sync();
-    if (ld_relaxed_u32(&st->status) != 0u) spin_ns(20000u);
+    return ld_relaxed_u32(&st->status) != 0u;
+}
+
+/* Bytes that the warps [w0, w1) of the senders [r0, r1) have stored for step d (512 per warp). */
+template <uint32_t SENDERS>
+__device__ __forceinline__ uint32_t stored_bytes(const Stored<SENDERS> &stored, uint32_t r0, uint32_t r1, uint32_t w0,
+                                                 uint32_t w1, uint32_t d)
+{
+    uint32_t bytes = 0;
+    for (uint32_t r = r0; r < r1; ++r)
+        for (uint32_t w = w0; w < w1; ++w) bytes += (stored.steps[r][w] > d) ? 512u : 0u;
+    return bytes;
+}
+
+/*
+ * The partials that may still be on their way to a reader after a failure (one lane of a warp calls).  The warp has armed
+ * `armed` phases: the last of them may be incomplete, and stores of the step after it may have been made (its writers
+ * wait for this reader's result or for one of the barriers before they go further).  Both barriers: one mbarrier for the
+ * whole chunk, which warp 0 arms.
+ */
+template <bool BARRIER, uint32_t SENDERS>
+__device__ __forceinline__ void drain_partials(unsigned long long (*top)[kWarpsPerCta], const Stored<SENDERS> &stored,
+                                               uint32_t r0, uint32_t r1, uint32_t warp, uint32_t warps, uint32_t armed,
+                                               uint32_t e0, uint32_t steps, DevState *st)
+{
+    if (BARRIER && warp != 0u) return;
+    for (uint32_t d = armed ? armed - 1u : 0u; d <= armed && d < steps; ++d) {
+        if constexpr (BARRIER)
+            mbar_drain(smem_addr(&top[0][0]), d & 1u, d < armed, (r1 - r0) * warps * 512u,
+                       stored_bytes(stored, r0, r1, 0u, warps, d), st);
+        else
+            mbar_drain(smem_addr(&top[(e0 + 1u + d) & 1u][warp]), (d >> 1) & 1u, d < armed, (r1 - r0) * 512u,
+                       stored_bytes(stored, r0, r1, warp, warp + 1u, d), st);
+    }
 }
 
 template <int DT, int P, int MODE, bool TRACE>
@@ -77,6 +123,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
     /* the reader's box: [parity][rank][kBoxStride] partials; a producer's box: [parity][thread] results */
     __shared__ __align__(16) uint4 s_box[kBoxSlots];
     __shared__ unsigned long long s_top[2][kWarpsPerCta], s_hand[2][kWarpsPerCta], s_done;
+    __shared__ Stored<kRoles> s_stored;                               /* by role: results of the reader, partials of the ranks */
     __shared__ int s_last;
 
     DevState *st = a.st;
@@ -94,7 +141,9 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
     const bool active = threadIdx.x < units;                          /* warp-uniform */
     const size_t u = unit0 + threadIdx.x;
     const uint32_t box = smem_addr(s_box);
-    cluster_prologue(s_box, kBoxSlots, s_top, s_hand, &s_done, units / 32u);
+    cluster_prologue(s_box, kBoxSlots, s_top, s_hand, &s_done, units / 32u, s_stored, a.steps);
+    constexpr bool counted = !slot_units;                             /* stores counted on mbarriers */
+    uint32_t gave_up = a.steps;                                       /* the step this warp did not get through */
     unsigned reloads = 0;
     /* results are stamped by the warps that publish them (rank 0's without all-reduce): the warps of a chunk are
        pipelines of their own, a chunk is complete with the last of them */
@@ -158,7 +207,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
                     for (int r = 0; r < P; ++r) x[r] = ld_shared_slot(in + (r * kBoxStride + threadIdx.x) * 16u);
                 }
             }
-            if (!ok) break;
+            if (!ok) { gave_up = s; break; }
             SIFAR_TRACE(1, threadIdx.x == 0);
             SIFAR_TRACE(38 + warp, spec && lane == 0u);
             if constexpr (barrier) {
@@ -223,7 +272,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
                 }
             }
             ok = __all_sync(0xFFFFFFFFu, ok);
-            if (!ok) break;
+            if (!ok) { gave_up = s; break; }
             SIFAR_TRACE(4 + 3 * rank, threadIdx.x == 0);
             if (a.w.delay_max_ns != 0u) spin_ns(gen_delay_ns(a.w, rank, t));      /* seeded skew */
             unit_apply<DT, NW>(g, first, pw, u * NE, n, z, w);
@@ -251,7 +300,22 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_cluster(const Persis
         if (stamper) my_stamps[s + 1u] = globaltimer_ns();
     }
 #undef SIFAR_TRACE
-    cluster_epilogue(st);
+    /* A warp that gave up in step s has stored for the s steps before it; the reader has armed step s as well, a
+       producer the results of the s steps before it.  A whole run hands over all results but the last. */
+    if (counted && gave_up != a.steps && lane < (is_reader ? (uint32_t)P : 1u))
+        st_cluster_u32(cluster_map(smem_addr(&s_stored.steps[role][warp]), is_reader ? lane + 1u : 0u), gave_up);
+    const bool failed = cluster_epilogue(st);
+    if (counted && failed && active && lane == 0u) {
+        if (is_reader) {
+            drain_partials<barrier>(s_top, s_stored, 1u, kRoles, warp, units / 32u, gave_up == a.steps ? gave_up : gave_up + 1u,
+                                    a.e0, a.steps, st);
+        } else {
+            const uint32_t armed = gave_up == a.steps ? a.steps - 1u : gave_up;
+            for (uint32_t d = armed ? armed - 1u : 0u; d <= armed && d + 1u < a.steps; ++d)
+                mbar_drain(smem_addr(&s_hand[(a.e0 + 1u + d) & 1u][warp]), (d >> 1) & 1u, d < armed, 512u,
+                           stored_bytes(s_stored, 0u, 1u, warp, warp + 1u, d), st);
+        }
+    }
     /* leave: mis-speculation counters, then the last CTA out publishes the call number */
     const unsigned warp_reloads = __reduce_add_sync(0xFFFFFFFFu, reloads);
     if (warp_reloads && lane == 0u) atomicAdd(&st->stats[kStatSlotReloads], (unsigned long long)warp_reloads);
@@ -294,6 +358,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
     constexpr uint32_t kBoxSlots = (barrier ? 1 : 2) * P * kBoxStride;
     __shared__ __align__(16) uint4 s_box[kBoxSlots];                  /* [parity][rank][kBoxStride] */
     __shared__ unsigned long long s_top[2][kWarpsPerCta], s_done;
+    __shared__ Stored<P> s_stored;
     __shared__ int s_last;
 
     DevState *st = a.st;
@@ -309,7 +374,9 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
     const size_t u = unit0 + threadIdx.x;
     const uint32_t box = smem_addr(s_box);
     char *my_ring = a.rings + (size_t)rank * a.ring_len * a.ring_stride;
-    cluster_prologue(s_box, kBoxSlots, s_top, nullptr, &s_done, (uint32_t)P * (units / 32u));
+    cluster_prologue(s_box, kBoxSlots, s_top, nullptr, &s_done, (uint32_t)P * (units / 32u), s_stored, a.steps);
+    constexpr bool counted = !spec && !no_ar;                         /* stores counted on mbarriers */
+    uint32_t stored = a.steps, armed = a.steps;                       /* steps that this warp has stored, waited for */
     const bool stamper = lane == 0u;
     unsigned long long *my_stamps = a.stamps + (((size_t)rank * a.C + chunk) * kWarpsPerCta + warp) * (a.steps + 1u);
     const uint32_t top_at = smem_addr(s_top) - box, done_at = smem_addr(&s_done) - box;
@@ -348,7 +415,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
         if constexpr (barrier) {
             /* bottom barrier, writer side: all P readers are done with the single buffer (Section 3.1, phase 3) */
             if (s > 0u) ok = mbar_wait_or_fail(smem_addr(&s_done), (s - 1u) & 1u, st, a.host_status, a.timeout_ns);
-            if (!__all_sync(0xFFFFFFFFu, ok)) break;
+            if (!__all_sync(0xFFFFFFFFu, ok)) { stored = armed = s; break; }
         }
         if (a.w.delay_max_ns != 0u) spin_ns(gen_delay_ns(a.w, rank, t));          /* seeded skew between the ranks */
         /* ---- the rank's operation, stored for every reader ---- */
@@ -395,7 +462,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
                     for (int r = 0; r < P; ++r) x[r] = ld_shared_slot(in + (r * kBoxStride + threadIdx.x) * 16u);
                 }
             }
-            if (!ok) break;
+            if (!ok) { stored = armed = s + 1u; break; }
             if constexpr (barrier) {
                 /* bottom barrier, reader side: this warp's loads of the chunk have returned */
                 __syncwarp();
@@ -413,7 +480,11 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_sym_cluster(const SymArgs 
         }
         if (stamper) my_stamps[s + 1u] = globaltimer_ns();
     }
-    cluster_epilogue(st);
+    if (counted && stored != a.steps && lane < (uint32_t)P)
+        st_cluster_u32(cluster_map(smem_addr(&s_stored.steps[rank][warp]), lane), stored);
+    const bool failed = cluster_epilogue(st);
+    if (counted && failed && active && lane == 0u)
+        drain_partials<barrier>(s_top, s_stored, 0u, (uint32_t)P, warp, units / 32u, armed, a.e0, a.steps, st);
     /* leave: statistics, then the last CTA out books the run and publishes the call number */
     const unsigned warp_reloads = __reduce_add_sync(0xFFFFFFFFu, reloads);
     if (warp_reloads && lane == 0u) atomicAdd(&st->stats[kStatSlotReloads], (unsigned long long)warp_reloads);

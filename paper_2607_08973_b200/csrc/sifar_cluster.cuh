@@ -113,6 +113,41 @@ __device__ __forceinline__ bool mbar_wait_or_fail(uint32_t mbar, uint32_t parity
     }
 }
 
+/* Takes `bytes` off what the current phase waits for, as if they had been stored. */
+__device__ __forceinline__ void mbar_complete_tx(uint32_t mbar, uint32_t bytes)
+{
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" :: "r"(mbar), "r"(bytes) : "memory");
+}
+
+/*
+ * After a failure: waits until counted stores that are still on their way have landed, so that the CTA may leave.
+ * `coming` bytes of the phase have been or will be stored, `expected` were armed (or, `armed` false, none yet).  The
+ * phase is brought to exactly what is coming and then completes with the last of it; with everything that was expected
+ * coming, or the phase complete already, nothing is changed.  A store takes well below a microsecond, so the limit is
+ * there for the loop alone; running into it is counted as one more wait that timed out.
+ */
+constexpr unsigned long long kDrainLimitNs = 1000000ull;
+
+__device__ __forceinline__ void mbar_drain(uint32_t mbar, uint32_t parity, bool armed, uint32_t expected, uint32_t coming,
+                                           DevState *st)
+{
+    if (armed) {
+        if (coming < expected) mbar_complete_tx(mbar, expected - coming);
+    } else if (coming) {
+        mbar_expect(mbar, coming);
+    } else {
+        return;
+    }
+    Deadline d;
+    while (!mbar_try(mbar, parity))
+        if (d.expired(kDrainLimitNs)) { atomicAdd(&st->stats[kStatTimeouts], 1ull); return; }
+}
+
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v)
+{
+    asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
+}
+
 /* Time limit of a loop that polls shared memory: a poll takes some 30 cycles, so the clock is read on every 64th and
    the context's status looked at on every 1024th. */
 struct LocalDeadline {

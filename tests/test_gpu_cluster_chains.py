@@ -65,3 +65,40 @@ def test_clusters_and_spread_chunks_agree_up_to_the_size_where_clusters_end(monk
                 sf.sifar_chain_destroy(ch)
                 results.append(_rows(ring, stride, steps, n, BF16))
         assert np.array_equal(results[0], results[1])
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("readers", ["one", "all"])
+@pytest.mark.parametrize("P,n", [(8, 4096), (8, 1025), (3, 2049), (2, 70)])
+def test_a_cluster_that_gives_up_waits_for_the_stores_on_their_way(oracle, P, n, mode, readers):
+    """Ranks delayed by up to 1 ms against a 50 us limit, so warps give up with stores of others still to come.  Every
+    CTA waits for what comes to it and for no more: had one of those waits run out it would be counted as a second
+    time-out.  The context then runs the same chain without delays."""
+    steps = 8
+    create, run, destroy = ((sf.sifar_chain_create, sf.sifar_chain_run, sf.sifar_chain_destroy) if readers == "one" else
+                            (sf.sifar_symchain_create, sf.sifar_symchain_run, sf.sifar_symchain_destroy))
+    impl = (sf.CHAIN_PERSISTENT,) if readers == "one" else ()
+    d = synth.chain_workload("llama", P)
+    copies = 1 if readers == "one" else P
+    with Ctx(P, n, BF16) as ctx:
+        for seed in range(4):
+            late = dict(d, seed=100 + seed, delay_max_ns=1_000_000)
+            sf.sifar_set_timeout_us(ctx.h, 50)
+            rings, stride = _ring(n, BF16, copies * steps)
+            ch = create(ctx.h, sf.make_workload(**late), n, mode, *impl, rings.data_ptr(), steps, steps)
+            run(ch, 0)
+            torch.cuda.synchronize()
+            assert sf.sifar_status(ctx.h) == sf.ERR_TIMEOUT
+            assert sf.sifar_get_stats(ctx.h)["timeouts"] == 1
+            destroy(ch)
+            sf.sifar_reset(ctx.h, 0)
+        sf.sifar_set_timeout_us(ctx.h, 2_000_000)
+        ch = create(ctx.h, sf.make_workload(**d), n, mode, *impl, rings.data_ptr(), steps, steps)
+        run(ch, 0)
+        torch.cuda.synchronize()
+        assert sf.sifar_status(ctx.h) == 0
+        destroy(ch)
+        want = oracle.chain(_oracle_w(oracle, d), P, n, BF16, steps)
+        got = _rows(rings, stride, copies * steps, n, BF16)
+        for i in range(copies * steps):
+            assert_bits_equal(got[i], want[i % steps], BF16, f"row {i}")
