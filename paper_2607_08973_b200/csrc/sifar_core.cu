@@ -773,8 +773,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_reduce_spec(const ReduceArgs a)
 /* ------------------------------------------------------------------------ */
 constexpr int kPackUnroll = 4;
 
-/* AHEAD: no thread has more than one unit (see launch_pack_mode). */
-template <int DT, int MODE, bool AHEAD>
+template <int DT, int MODE>
 __device__ __forceinline__ void pack_body(const PackArgs &a)
 {
     DevState *st = a.st;
@@ -786,11 +785,9 @@ __device__ __forceinline__ void pack_body(const PackArgs &a)
     const size_t tid = (size_t)blockIdx.x * kThreads + threadIdx.x;
     const size_t nthreads = (size_t)gridDim.x * kThreads;
     /* Where a thread has one whole unit at most, its words travel together with the call number: a small pack is two
-       round trips and a launch, and this is one of the two.  A kernel of its own: in the same one the loops of the large
-       packs came out with fewer loads in flight (40-48 registers instead of 64; eight ranks of 2 MiB on one stream,
-       dual-buffered, 48.7 us a call, 51.0 that way). */
+       round trips and a launch, and this is one of the two. */
     constexpr int EPU = (MODE == SIFAR_SPECULATIVE) ? kSlotDataWords * ((DT == SIFAR_BF16) ? 2 : 1) : ((DT == SIFAR_BF16) ? 8 : 4);
-    const bool ahead = AHEAD && (tid + 1) * EPU <= a.n;
+    const bool ahead = MODE != kModeTiles && a.n <= nthreads * EPU && (tid + 1) * EPU <= a.n;
     uint4 first = make_uint4(0u, 0u, 0u, 0u);
     if (ahead) {
         if (MODE == SIFAR_SPECULATIVE) {
@@ -927,10 +924,10 @@ __device__ __forceinline__ void pack_body(const PackArgs &a)
     }
 }
 
-template <int DT, int MODE, bool AHEAD>
+template <int DT, int MODE>
 __global__ void __launch_bounds__(kThreads) k_pack(const PackArgs a)
 {
-    pack_body<DT, MODE, AHEAD>(a);
+    pack_body<DT, MODE>(a);
 }
 
 /*
@@ -1302,13 +1299,10 @@ static cudaError_t preload_dt(int P)
     case 7: e = preload_reducers<DT, 7>(); break;
     default: e = preload_reducers<DT, 8>(); break;
     }
-    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_BARRIER_ONESHOT, false>);
-    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_BARRIER_ONESHOT, true>);
-    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_DUALBUF, false>);
-    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_DUALBUF, true>);
-    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_SPECULATIVE, false>);
-    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_SPECULATIVE, true>);
-    if (e == cudaSuccess) e = preload(k_pack<DT, kModeTiles, false>);
+    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_BARRIER_ONESHOT>);
+    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_DUALBUF>);
+    if (e == cudaSuccess) e = preload(k_pack<DT, SIFAR_SPECULATIVE>);
+    if (e == cudaSuccess) e = preload(k_pack<DT, kModeTiles>);
     if (e == cudaSuccess) e = preload(k_arrive);
     if (e == cudaSuccess) e = preload(k_wait_writable);
     if (e == cudaSuccess) e = preload(k_empty_call);
@@ -1359,25 +1353,21 @@ static cudaError_t launch_dependent(void (*kernel)(Params...), int grid, int thr
 }
 
 template <int DT, int MODE>
-static cudaError_t launch_pack_mode(int grid, bool ahead, bool dependent, cudaStream_t s, const PackArgs &a)
+static cudaError_t launch_pack_mode(int grid, bool dependent, cudaStream_t s, const PackArgs &a)
 {
-    void (*kernel)(PackArgs) = k_pack<DT, MODE, false>;
-    if constexpr (MODE != kModeTiles) {
-        if (ahead) kernel = k_pack<DT, MODE, true>;
-    }
-    if (dependent) return launch_dependent(kernel, grid, kThreads, s, a);
-    kernel<<<grid, kThreads, 0, s>>>(a);
+    if (dependent) return launch_dependent(k_pack<DT, MODE>, grid, kThreads, s, a);
+    k_pack<DT, MODE><<<grid, kThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int DT>
-static cudaError_t launch_pack_dt(int mode, int grid, bool ahead, bool dependent, cudaStream_t s, const PackArgs &a)
+static cudaError_t launch_pack_dt(int mode, int grid, bool dependent, cudaStream_t s, const PackArgs &a)
 {
     switch (mode) {
-    case SIFAR_BARRIER_ONESHOT: return launch_pack_mode<DT, SIFAR_BARRIER_ONESHOT>(grid, ahead, dependent, s, a);
-    case SIFAR_DUALBUF:         return launch_pack_mode<DT, SIFAR_DUALBUF>(grid, ahead, dependent, s, a);
-    case kModeTiles:            return launch_pack_mode<DT, kModeTiles>(grid, ahead, dependent, s, a);
-    default:                    return launch_pack_mode<DT, SIFAR_SPECULATIVE>(grid, ahead, dependent, s, a);
+    case SIFAR_BARRIER_ONESHOT: return launch_pack_mode<DT, SIFAR_BARRIER_ONESHOT>(grid, dependent, s, a);
+    case SIFAR_DUALBUF:         return launch_pack_mode<DT, SIFAR_DUALBUF>(grid, dependent, s, a);
+    case kModeTiles:            return launch_pack_mode<DT, kModeTiles>(grid, dependent, s, a);
+    default:                    return launch_pack_mode<DT, SIFAR_SPECULATIVE>(grid, dependent, s, a);
     }
 }
 
@@ -1702,10 +1692,9 @@ extern "C" int sifar_pack(sifar_ctx *c, int rank, const void *src, size_t n, int
        that packs its ranks one after another on one stream).  Larger grids would hold room that kernels of other
        streams, the ranks that a reducer waits for among them, need meanwhile. */
     const bool dependent = grid <= (size_t)c->sm_count;
-    const bool ahead = units <= grid * kThreads;
     cudaError_t err = (c->dtype == SIFAR_BF16)
-        ? launch_pack_dt<SIFAR_BF16>(kernel_mode, (int)grid, ahead, dependent, (cudaStream_t)stream, a)
-        : launch_pack_dt<SIFAR_F32>(kernel_mode, (int)grid, ahead, dependent, (cudaStream_t)stream, a);
+        ? launch_pack_dt<SIFAR_BF16>(kernel_mode, (int)grid, dependent, (cudaStream_t)stream, a)
+        : launch_pack_dt<SIFAR_F32>(kernel_mode, (int)grid, dependent, (cudaStream_t)stream, a);
     SIFAR_CUDA(err);
     note_producer(c, rank, e, (cudaStream_t)stream, n);
     return SIFAR_OK;
