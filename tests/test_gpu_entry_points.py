@@ -72,29 +72,34 @@ def _in_a_process_of_its_own(code, **env):
 
 
 @pytest.mark.parametrize("mode", MODES)
-def test_the_first_host_call_beside_a_reducer_that_waits_for_a_late_pack(mode):
-    """The process's first host call is made while another context's reducer polls for a pack that the same thread
-    enqueues afterwards: it may not wait for the device to become idle (its kernel is loaded with the context)."""
+def test_the_first_host_call_beside_a_reducer_that_waits_for_a_late_rank(mode):
+    """The process's first host call is made while another context's reducer polls for a rank whose store the same thread
+    launches afterwards: it may not wait for the device to become idle (its kernel is loaded with the context)."""
     _in_a_process_of_its_own(f"""
+        import time
         import torch
         from paper_2607_08973_b200 import binding as sf
-        n, mode = 4096, {mode}
+        n = 4096
+        sf.sifar_workload_preload()
         waiting, host = sf.sifar_create(2, n, sf.BF16), sf.sifar_create(3, n, sf.F32)
         sf.sifar_set_timeout_us(waiting, 2_000_000)
         x = [torch.ones(n, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
         out = torch.zeros(n, dtype=torch.bfloat16, device="cuda")
         hx = [torch.full((n,), float(r + 1)).pin_memory() for r in range(3)]
         hout = torch.zeros(n).pin_memory()
-        packs, red = [torch.cuda.Stream() for _ in range(2)], torch.cuda.Stream()
+        ranks, red = [torch.cuda.Stream() for _ in range(2)], torch.cuda.Stream()
         torch.cuda.synchronize()
-        sf.sifar_pack(waiting, 0, x[0].data_ptr(), n, mode, packs[0].cuda_stream)
-        sf.sifar_allreduce(waiting, None, out.data_ptr(), n, mode, red.cuda_stream)
-        sf.sifar_allreduce_host(host, [t.data_ptr() for t in hx], hout.data_ptr(), n, mode)
-        sf.sifar_pack(waiting, 1, x[1].data_ptr(), n, mode, packs[1].cuda_stream)
+        sf.sifar_pack(waiting, 0, x[0].data_ptr(), n, sf.SPECULATIVE, ranks[0].cuda_stream)
+        late, epoch = sf.sifar_rank_buffer(waiting, 1, sf.SPECULATIVE)
+        sf.sifar_allreduce(waiting, None, out.data_ptr(), n, sf.SPECULATIVE, red.cuda_stream)
+        t0 = time.perf_counter()
+        sf.sifar_allreduce_host(host, [t.data_ptr() for t in hx], hout.data_ptr(), n, {mode})
+        assert time.perf_counter() - t0 < 1.0, "the call waited for the reducer's time limit"
+        sf.sifar_store_slots(x[1].data_ptr(), late, 0, sf.sifar_slot_count(sf.BF16, n), n, sf.BF16, epoch, ranks[1].cuda_stream)
         torch.cuda.synchronize()
         assert sf.sifar_status(waiting) == 0 and sf.sifar_get_stats(waiting)["timeouts"] == 0
         assert bool((out == 2).all()) and bool((hout == 6).all())
-        """)
+        """, CUDA_DEVICE_MAX_CONNECTIONS="32")                    # no two of the streams in one hardware queue
 
 
 @pytest.mark.parametrize("mode", MODES)
@@ -247,6 +252,7 @@ def test_dependent_launches_follow_the_switch(entry, pdl):
     """A captured row of launches shows how each was launched: a programmatic edge to the kernel before it, or a full
     one.  With SIFAR_PDL=0 the plain stream order is back in all of them."""
     out = _in_a_process_of_its_own(f"""
+        import ctypes
         import torch
         from cuda.bindings import runtime as rt
         from paper_2607_08973_b200 import binding as sf
@@ -273,10 +279,10 @@ def test_dependent_launches_follow_the_switch(entry, pdl):
                                    sf.BARRIER_ONESHOT if entry == "arrivals" else sf.SPECULATIVE, s)
         err, graph = rt.cudaStreamEndCapture(s)
         assert err == 0
-        err, _, _, _, k = rt.cudaGraphGetEdges_v2(graph)
-        err, _, _, data, k = rt.cudaGraphGetEdges_v2(graph, k)
-        assert err == 0 and k > 0
-        kinds = [int(d.type) for d in data[:k]]
+        k = ctypes.c_size_t(64)
+        ends, data = [(ctypes.c_void_p * 64)() for _ in range(2)], (ctypes.c_uint8 * 8 * 64)()
+        assert ctypes.CDLL("libcudart.so.12").cudaGraphGetEdges_v2(ctypes.c_void_p(int(graph)), *ends, data, ctypes.byref(k)) == 0
+        kinds = [d[2] for d in data[:k.value]]                    # from port, to port, type
         err, ex = rt.cudaGraphInstantiate(graph, 0)
         assert err == 0
         for _ in range(3):                                        # the call number advances on the device
