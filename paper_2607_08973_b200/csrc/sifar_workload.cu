@@ -255,8 +255,19 @@ constexpr size_t cluster_max_pairs(int mode)
 }
 constexpr int kPreUnits = 4;            /* units per producer thread, beyond its first, whose seeded half is computed before the wait */
 
-template <int DT, int P, int MODE, bool TRACE, bool TAGGED>
-__global__ void __launch_bounds__(kChainThreads, 6) k_chain(const PersistArgs a)
+/*
+ * CTAs per SM that the kernel is compiled for.  Six leaves 80 registers, which the generator's loops use; where that
+ * makes a thread of the modes with flags take one unit more per step than a denser grid would, the kernel compiled for
+ * eight (tagged hand-over, 64 registers) or nine CTAs (56) is used: no spills, and the same instructions in another
+ * order cost 1-2 % at the sizes where both take one unit.  us per run of 64 steps, six / eight or nine: P = 8 bf16 with
+ * both barriers 224 KB per rank 332 / 289, 448 KB 461 / 423, 512 KB 530 / 464; dual-buffered 224 KB 304 / 278, 512 KB 533 /
+ * 458; P = 8 fp32 448 KB 379 / 338; P = 4 fp32 448 KB 298 / 258; P = 3 bf16 448 KB 308 / 258.  The speculative kernel
+ * holds P slots and polls them: it spills at that bound.
+ */
+constexpr int chain_ctas(bool dense, bool tagged) { return !dense ? 6 : tagged ? 8 : 9; }
+
+template <int DT, int P, int MODE, bool TRACE, bool TAGGED, bool DENSE>
+__global__ void __launch_bounds__(kChainThreads, chain_ctas(DENSE, TAGGED)) k_chain(const PersistArgs a)
 {
     DevState *st = a.st;
     const uint32_t C = a.C;
@@ -634,6 +645,7 @@ struct sifar_chain {
     uint4 *d_handoff;
     size_t handoff_stride;
     bool tagged;                    /* form of the hand-over (see handoff_store) */
+    bool dense;                     /* the kernel compiled for more CTAs per SM (see chain_ctas) */
     uint32_t C, K;
     int grid;
     const void *cluster_kernel;     /* not NULL: one thread-block cluster per chunk, whose ranks meet in its shared
@@ -799,41 +811,63 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
     return SIFAR_OK;
 }
 
-template <int DT, int P, bool TRACE>
+template <int DT, int P, bool TRACE, bool DENSE>
 static const void *chain_kernel_p(int mode, bool tagged)
 {
     switch (mode) {
-    case SIFAR_BARRIER_ONESHOT: return (const void *)k_chain<DT, P, SIFAR_BARRIER_ONESHOT, TRACE, false>;
-    case SIFAR_DUALBUF:         return tagged ? (const void *)k_chain<DT, P, SIFAR_DUALBUF, TRACE, true>
-                                              : (const void *)k_chain<DT, P, SIFAR_DUALBUF, TRACE, false>;
-    case SIFAR_SPECULATIVE:     return tagged ? (const void *)k_chain<DT, P, SIFAR_SPECULATIVE, TRACE, true>
-                                              : (const void *)k_chain<DT, P, SIFAR_SPECULATIVE, TRACE, false>;
-    default:                    return (const void *)k_chain<DT, P, kModeNoAllreduce, false, false>;
+    case SIFAR_BARRIER_ONESHOT: return (const void *)k_chain<DT, P, SIFAR_BARRIER_ONESHOT, TRACE, false, DENSE>;
+    case SIFAR_DUALBUF:         return tagged ? (const void *)k_chain<DT, P, SIFAR_DUALBUF, TRACE, true, DENSE>
+                                              : (const void *)k_chain<DT, P, SIFAR_DUALBUF, TRACE, false, DENSE>;
+    case SIFAR_SPECULATIVE:     return tagged ? (const void *)k_chain<DT, P, SIFAR_SPECULATIVE, TRACE, true, false>
+                                              : (const void *)k_chain<DT, P, SIFAR_SPECULATIVE, TRACE, false, false>;
+    default:                    return (const void *)k_chain<DT, P, kModeNoAllreduce, false, false, false>;
     }
 }
 
-template <int DT>
+template <int DT, bool DENSE>
 static const void *chain_kernel_dt(int P, int mode, bool trace, bool tagged)
 {
     /* the traced build exists for the shapes of the workload list only */
-    if (trace && P == 8) return chain_kernel_p<DT, 8, true>(mode, tagged);
-    if (trace && P == 2) return chain_kernel_p<DT, 2, true>(mode, tagged);
+    if (trace && P == 8) return chain_kernel_p<DT, 8, true, DENSE>(mode, tagged);
+    if (trace && P == 2) return chain_kernel_p<DT, 2, true, DENSE>(mode, tagged);
     switch (P) {
-    case 1: return chain_kernel_p<DT, 1, false>(mode, tagged);
-    case 2: return chain_kernel_p<DT, 2, false>(mode, tagged);
-    case 3: return chain_kernel_p<DT, 3, false>(mode, tagged);
-    case 4: return chain_kernel_p<DT, 4, false>(mode, tagged);
-    case 5: return chain_kernel_p<DT, 5, false>(mode, tagged);
-    case 6: return chain_kernel_p<DT, 6, false>(mode, tagged);
-    case 7: return chain_kernel_p<DT, 7, false>(mode, tagged);
-    default: return chain_kernel_p<DT, 8, false>(mode, tagged);
+    case 1: return chain_kernel_p<DT, 1, false, DENSE>(mode, tagged);
+    case 2: return chain_kernel_p<DT, 2, false, DENSE>(mode, tagged);
+    case 3: return chain_kernel_p<DT, 3, false, DENSE>(mode, tagged);
+    case 4: return chain_kernel_p<DT, 4, false, DENSE>(mode, tagged);
+    case 5: return chain_kernel_p<DT, 5, false, DENSE>(mode, tagged);
+    case 6: return chain_kernel_p<DT, 6, false, DENSE>(mode, tagged);
+    case 7: return chain_kernel_p<DT, 7, false, DENSE>(mode, tagged);
+    default: return chain_kernel_p<DT, 8, false, DENSE>(mode, tagged);
     }
 }
 
 static const void *chain_kernel(const sifar_chain *ch, bool trace = false)
 {
-    return ch->ctx->dtype == SIFAR_BF16 ? chain_kernel_dt<SIFAR_BF16>(ch->ctx->P, ch->mode, trace, ch->tagged)
-                                        : chain_kernel_dt<SIFAR_F32>(ch->ctx->P, ch->mode, trace, ch->tagged);
+    const int P = ch->ctx->P;
+    if (ch->ctx->dtype == SIFAR_BF16)
+        return ch->dense ? chain_kernel_dt<SIFAR_BF16, true>(P, ch->mode, trace, ch->tagged)
+                         : chain_kernel_dt<SIFAR_BF16, false>(P, ch->mode, trace, ch->tagged);
+    return ch->dense ? chain_kernel_dt<SIFAR_F32, true>(P, ch->mode, trace, ch->tagged)
+                     : chain_kernel_dt<SIFAR_F32, false>(P, ch->mode, trace, ch->tagged);
+}
+
+/* Units per thread and chunks of the grid that spreads over the whole machine if need be: every unit per thread beyond
+   the first lengthens the step by its dependent load and store round trips. */
+static int chain_spread(const sifar_chain *ch, size_t units, int roles, uint32_t *K, uint32_t *C)
+{
+    int per_sm = 0;
+    SIFAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chain_kernel(ch), kChainThreads, 0));
+    const size_t resident = (size_t)per_sm * ch->ctx->sm_count;
+    const size_t budget = resident > (size_t)roles ? resident : (size_t)roles;
+    *K = 1;
+    size_t chunks = (units + kChainThreads - 1) / kChainThreads;
+    while (chunks * roles > budget) {
+        ++*K;
+        chunks = (units + (size_t)kChainThreads * *K - 1) / ((size_t)kChainThreads * *K);
+    }
+    *C = (uint32_t)chunks;
+    return SIFAR_OK;
 }
 
 static void chain_free(sifar_chain *ch)
@@ -881,19 +915,15 @@ static int chain_setup_persistent(sifar_chain *ch)
     if (ch->cluster_kernel) {
         ch->K = 1; ch->C = (uint32_t)chunks;
     } else {
-        int per_sm = 0;
-        SIFAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chain_kernel(ch), kChainThreads, 0));
-        const size_t resident = (size_t)per_sm * c->sm_count;
-        /* the whole machine if need be: every unit per thread beyond the first lengthens the step by its
-           dependent load and store round trips */
-        const size_t budget = resident > (size_t)roles ? resident : (size_t)roles;
-        uint32_t K = 1;      /* units per thread and step: 1 whenever the grid fits (more only lengthens the step) */
-        size_t C = chunks;
-        while (C * roles > budget) {
-            ++K;
-            C = (units + (size_t)kChainThreads * K - 1) / ((size_t)kChainThreads * K);
+        int rc = chain_spread(ch, units, roles, &ch->K, &ch->C);
+        if (rc) return rc;
+        if (ch->K > 1 && (ch->mode == SIFAR_BARRIER_ONESHOT || ch->mode == SIFAR_DUALBUF)) {
+            uint32_t K, C;
+            ch->dense = true;
+            if ((rc = chain_spread(ch, units, roles, &K, &C))) return rc;
+            ch->dense = K < ch->K;                       /* see chain_ctas() */
+            if (ch->dense) { ch->K = K; ch->C = C; }
         }
-        ch->K = K; ch->C = (uint32_t)C;
     }
     const size_t C = ch->C;
     ch->grid = (int)(C * roles);

@@ -211,6 +211,34 @@ def test_the_kernel_runs_with_the_layout_the_host_chose(mode, n, clustered, tagg
     assert g["ctas"] == g["chunks"] * (P + 1)
 
 
+@pytest.mark.parametrize("P,n,dtype,mode", [
+    (8, 114_688, BF16, sf.BARRIER_ONESHOT), (8, 114_688, BF16, sf.DUALBUF), (8, 262_144, BF16, sf.DUALBUF),
+    (8, 114_688, F32, sf.DUALBUF), (4, 114_691, F32, sf.BARRIER_ONESHOT), (3, 229_381, BF16, sf.BARRIER_ONESHOT)])
+def test_grids_denser_than_six_ctas_per_sm(oracle, P, n, dtype, mode):
+    """Where six CTAs per SM would give a thread one unit more, the kernel compiled for more of them runs: tagged words,
+    ready flags and done flags, one unit per thread and two, whole and ragged last chunks."""
+    steps = 4
+    _, d = _workloads("llama", P)
+    with Ctx(P, n, dtype) as ctx:
+        ring, stride = _ring(n, dtype, 2 * steps)
+        ch = sf.sifar_chain_create(ctx.h, sf.make_workload(**d), n, mode, sf.CHAIN_PERSISTENT, ring.data_ptr(), 2 * steps, steps)
+        try:
+            for _ in range(2):
+                sf.sifar_chain_run(ch, 0)
+            g = sf.sifar_chain_geometry(ch)
+        finally:
+            sf.sifar_chain_destroy(ch)
+        assert sf.sifar_status(ctx.h) == 0
+        assert g["clustered"] == 0
+        sparse = 6 * torch.cuda.get_device_properties(0).multi_processor_count
+        units = -(-n * (2 if dtype == BF16 else 4) // 16)
+        assert g["ctas"] > sparse or g["units_per_thread"] < -(-units // (128 * (sparse // (P + 1))))
+        got = _rows(ring, stride, 2 * steps, n, dtype)
+    want = oracle.chain(_oracle_w(oracle, d), P, n, dtype, 2 * steps)
+    for t in range(2 * steps):
+        assert_bits_equal(got[t], want[t], dtype, f"step {t + 1}")
+
+
 @pytest.mark.parametrize("handoff_max", ["100000", "0"])
 @pytest.mark.parametrize("mode", MODES)
 def test_a_wait_that_runs_out_ends_the_persistent_chain_and_the_context_recovers(oracle, monkeypatch, mode, handoff_max):
