@@ -258,16 +258,20 @@ constexpr int kPreUnits = 4;            /* units per producer thread, beyond its
 /*
  * CTAs per SM that the kernel is compiled for.  Six leaves 80 registers, which the generator's loops use; where that
  * makes a thread of the modes with flags take one unit more per step than a denser grid would, the kernel compiled for
- * eight (tagged hand-over, 64 registers) or nine CTAs (56) is used: no spills, and the same instructions in another
+ * nine CTAs (56 registers) is used, with the tagged hand-over eight (64; fp32 seven: P = 6, 320 KB, 262 us at two units
+ * per thread and seven, 273 at one and eight): no spills, and the same instructions in another
  * order cost 1-2 % at the sizes where both take one unit.  us per run of 64 steps, six / eight or nine: P = 8 bf16 with
  * both barriers 224 KB per rank 332 / 289, 448 KB 461 / 423, 512 KB 530 / 464; dual-buffered 224 KB 304 / 278, 512 KB 533 /
  * 458; P = 8 fp32 448 KB 379 / 338; P = 4 fp32 448 KB 298 / 258; P = 3 bf16 448 KB 308 / 258.  The speculative kernel
  * holds P slots and polls them: it spills at that bound.
  */
-constexpr int chain_ctas(bool dense, bool tagged) { return !dense ? 6 : tagged ? 8 : 9; }
+constexpr int chain_ctas(bool dense, bool tagged, int dtype)
+{
+    return !dense ? 6 : !tagged ? 9 : dtype == SIFAR_BF16 ? 8 : 7;
+}
 
 template <int DT, int P, int MODE, bool TRACE, bool TAGGED, bool DENSE>
-__global__ void __launch_bounds__(kChainThreads, chain_ctas(DENSE, TAGGED)) k_chain(const PersistArgs a)
+__global__ void __launch_bounds__(kChainThreads, chain_ctas(DENSE, TAGGED, DT)) k_chain(const PersistArgs a)
 {
     DevState *st = a.st;
     const uint32_t C = a.C;

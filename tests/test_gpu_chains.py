@@ -220,11 +220,14 @@ def test_grids_denser_than_six_ctas_per_sm(oracle, P, n, dtype, mode):
     steps = 4
     _, d = _workloads("llama", P)
     with Ctx(P, n, dtype) as ctx:
-        ring, stride = _ring(n, dtype, 2 * steps)
-        ch = sf.sifar_chain_create(ctx.h, sf.make_workload(**d), n, mode, sf.CHAIN_PERSISTENT, ring.data_ptr(), 2 * steps, steps)
+        ring, stride = _ring(n, dtype, steps)
+        ch = sf.sifar_chain_create(ctx.h, sf.make_workload(**d), n, mode, sf.CHAIN_PERSISTENT, ring.data_ptr(), steps, steps)
+        got = []
         try:
             for _ in range(2):
                 sf.sifar_chain_run(ch, 0)
+                torch.cuda.synchronize()
+                got.append(_rows(ring, stride, steps, n, dtype))
             g = sf.sifar_chain_geometry(ch)
         finally:
             sf.sifar_chain_destroy(ch)
@@ -233,10 +236,9 @@ def test_grids_denser_than_six_ctas_per_sm(oracle, P, n, dtype, mode):
         sparse = 6 * torch.cuda.get_device_properties(0).multi_processor_count
         units = -(-n * (2 if dtype == BF16 else 4) // 16)
         assert g["ctas"] > sparse or g["units_per_thread"] < -(-units // (128 * (sparse // (P + 1))))
-        got = _rows(ring, stride, 2 * steps, n, dtype)
     want = oracle.chain(_oracle_w(oracle, d), P, n, dtype, 2 * steps)
     for t in range(2 * steps):
-        assert_bits_equal(got[t], want[t], dtype, f"step {t + 1}")
+        assert_bits_equal(got[t // steps][t % steps], want[t], dtype, f"step {t + 1}")
 
 
 @pytest.mark.parametrize("handoff_max", ["100000", "0"])
