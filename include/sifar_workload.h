@@ -136,7 +136,7 @@ int sifar_chain_chunks(sifar_chain *chain);
 /*
  * How a PERSISTENT chain is laid out, as the host chose it and as the kernel of the last run saw it (synchronizes
  * the device): out[0] chunks, [1] units per thread and step, [2] CTAs, [3] 1 = the CTAs of a chunk are one
- * thread-block cluster and meet in its shared memory, [4] 1 = results reach the next step's producers unit by unit,
+ * thread-block cluster (sifar.h, SIFAR_CHAIN_CLUSTER), [4] 1 = results reach the next step's producers unit by unit,
  * in tagged words or counted stores (0 = ready flag per chunk, or done flags with both barriers); from the kernel: [5] the role layout it used (1 = clustered), [6] CTAs
  * per cluster as the hardware reported them (1 without clusters), [7] the form of the hand-over it was built for.
  * Before the first run [5..7] are 0.

@@ -48,6 +48,7 @@ struct PersistArgs {
     uint32_t C;                     /* chunks = reducer CTAs               */
     uint32_t K;                     /* units per thread and step           */
     uint32_t exit_base;
+    uint32_t placed;                /* k_chain: one cluster per chunk, for placement only */
     PollShape poll;
     ChainDev *cs;
     ChunkFlags *chunks;
@@ -186,7 +187,8 @@ const void *chain_cluster_kernel(int dtype, int P, int mode, bool trace);
 const void *sym_cluster_kernel(int dtype, int P, int mode);
 /* Can the device hold `clusters` clusters of `cluster` CTAs of the kernel at once? */
 bool cluster_fits(const void *kernel, int cluster, size_t clusters);
-cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params);
+/* `dependent`: the kernel does a prologue of its own and then waits for what precedes it on the stream. */
+cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params, bool dependent);
 
 }  /* namespace sifar */
 #endif

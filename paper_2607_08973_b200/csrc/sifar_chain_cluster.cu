@@ -595,13 +595,12 @@ bool cluster_fits(const void *kernel, int cluster, size_t clusters)
     return (size_t)most >= clusters;
 }
 
-cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params)
+cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params, bool dependent)
 {
-    /* as a dependent launch, unless switched off: the kernel does its prologue and then waits for what precedes it */
     static const bool early = !(getenv("SIFAR_CHAIN_PDL") && atoi(getenv("SIFAR_CHAIN_PDL")) == 0);
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = cluster_config(attr, cluster, clusters, kChainThreads, stream);
-    if (early) {
+    if (dependent && early) {
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.numAttrs = 2;

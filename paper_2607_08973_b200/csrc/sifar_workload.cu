@@ -242,17 +242,23 @@ __global__ void k_store_blocks(const void *src, void *dst, uint32_t *flags, unsi
  */
 constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE ? 170000 : 130000; }
 /*
- * One thread-block cluster per chunk up to this many (unit, rank) pairs (sifar_chain_cluster.cu).  us per run of 64
- * steps, P = 8, cluster against spread: 8 KB per rank 66 / 107 speculative, 57 / 184 dual-buffered, 103 / 218 with both
- * barriers; 64 KB 105 / 117, 94 / 198, 131 / 231; 78 KB 134 / 130, 105 / 215, 133 / 240; 127 KB 182 / 158, 150 / 228,
- * 192 / 247.  Speculative is level at 50 000 pairs, where tagged slots through the L2 need no flag either.  The two
- * modes with flags gain beyond 65 000 pairs too; the line lies just below 128 KB per rank at P = 8, whose spread layout
- * is part of what the tests pin.
+ * One thread-block cluster per chunk, its ranks meeting in shared memory, up to this many (unit, rank) pairs
+ * (sifar_chain_cluster.cu); above that, speculative, one cluster per chunk for placement (see k_chain) up to
+ * kPlacedMaxPairs, as far as cluster_max_pairs() ends before.  us per run of 64 steps, P = 8, bf16, shared memory against
+ * spread over the machine: dual-buffered 8 KB per rank 58 / 170, 64 KB 94 / 203, 96 KB 123 / 213; both barriers
+ * 104 / 220, 132 / 232, 156 / 241.  The modes with flags gain beyond 65 000 pairs, too (127 KB 150 / 228 and 192 / 247);
+ * nothing above is taken, because where the two layouts cross has not been measured.
+ * Speculative, shared memory / placed: P = 8 bf16 24 KB 74 / 83, 32 KB 82 / 84, 40 KB 86 / 85, 56 KB 107 / 97, 72 KB
+ * 121 / 112; P = 8 fp32 32 KB 80 / 79, 48 KB 102 / 83, 64 KB 112 / 84; P = 7 bf16 56 KB 87 / 94, 64 KB 95 / 98, 72 KB
+ * 104 / 98; P = 6 72 KB 81 / 95; P = 4 128 KB 89 / 110.  A chunk's one reader CTA takes and sends P vectors per thread
+ * through its SM's ports; with eight ranks and more than about 30 clusters that costs more than the hop saves.
  */
-constexpr size_t cluster_max_pairs(int mode)
+constexpr size_t cluster_max_pairs(int mode, int P)
 {
-    return (mode == SIFAR_DUALBUF || mode == SIFAR_BARRIER_ONESHOT) ? 65000 : 50000;
+    if (mode == SIFAR_DUALBUF || mode == SIFAR_BARRIER_ONESHOT) return 65000;
+    return mode != SIFAR_SPECULATIVE ? 50000 : P == 8 ? 25000 : P == 7 ? 40000 : 50000;
 }
+constexpr size_t kPlacedMaxPairs = 50000;
 constexpr int kPreUnits = 4;            /* units per producer thread, beyond its first, whose seeded half is computed before the wait */
 
 /*
@@ -276,11 +282,25 @@ __global__ void __launch_bounds__(kChainThreads, chain_ctas(DENSE, TAGGED, DT)) 
     DevState *st = a.st;
     const uint32_t C = a.C;
     const bool no_ar = (MODE == kModeNoAllreduce);
-    /* roles: reducers first, then the producers rank by rank */
-    const bool is_reducer = !no_ar && blockIdx.x < C;
-    const uint32_t pidx = no_ar ? blockIdx.x : blockIdx.x - C;
-    const uint32_t rank = is_reducer ? 0u : pidx / C;
-    const uint32_t chunk = is_reducer ? blockIdx.x : pidx % C;
+    /*
+     * Roles.  Placed: the CTAs that own one chunk (its reducer and its P producers) are consecutive and launched as one
+     * thread-block cluster, which the hardware places inside one GPC, so their flag and slot traffic stays on one die;
+     * nothing else of the cluster is used.  Otherwise reducers first, then the producers rank by rank.
+     */
+    bool is_reducer;
+    uint32_t rank, chunk;
+    if (a.placed) {
+        const uint32_t roles = no_ar ? (uint32_t)P : (uint32_t)P + 1u;
+        const uint32_t role = blockIdx.x % roles;
+        chunk = blockIdx.x / roles;
+        is_reducer = !no_ar && role == 0u;
+        rank = no_ar ? role : (is_reducer ? 0u : role - 1u);
+    } else {
+        is_reducer = !no_ar && blockIdx.x < C;
+        const uint32_t pidx = no_ar ? blockIdx.x : blockIdx.x - C;
+        rank = is_reducer ? 0u : pidx / C;
+        chunk = is_reducer ? blockIdx.x : pidx % C;
+    }
     ChunkFlags *cf = a.chunks + chunk;
     const size_t n = (size_t)a.n;
     /* 12-byte units where the unit travels with a tag in one 16-byte word (speculative slots; the chain without
@@ -301,7 +321,7 @@ __global__ void __launch_bounds__(kChainThreads, chain_ctas(DENSE, TAGGED, DT)) 
         /* what this launch really runs with, for sifar_chain_geometry */
         uint32_t cluster_ctas;
         asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cluster_ctas));
-        a.cs->seen[0] = 0u; a.cs->seen[1] = cluster_ctas; a.cs->seen[2] = TAGGED ? 1u : 0u;
+        a.cs->seen[0] = a.placed; a.cs->seen[1] = cluster_ctas; a.cs->seen[2] = TAGGED ? 1u : 0u;
     }
     __syncthreads();
     Gen g = make_gen(a.w, rank, 0u);
@@ -654,6 +674,7 @@ struct sifar_chain {
     int grid;
     const void *cluster_kernel;     /* not NULL: one thread-block cluster per chunk, whose ranks meet in its shared
                                        memory (sifar_chain_cluster.cu) */
+    bool placed;                    /* k_chain in one cluster per chunk, for placement */
     uint32_t stamp_pipes;           /* rows of stamps per chunk (see PersistArgs::stamps) */
 };
 
@@ -911,7 +932,8 @@ static int chain_setup_persistent(sifar_chain *ch)
     const char *env_cluster = getenv("SIFAR_CHAIN_CLUSTER");
     const size_t chunks = (units + kChainThreads - 1) / kChainThreads;
     const bool flag_form = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && !ch->tagged;
-    if (!(env_cluster && atoi(env_cluster) == 0) && !flag_form && units * (size_t)c->P <= cluster_max_pairs(ch->mode)) {
+    const bool clusters_allowed = !(env_cluster && atoi(env_cluster) == 0) && !flag_form;
+    if (clusters_allowed && units * (size_t)c->P <= cluster_max_pairs(ch->mode, c->P)) {
         const void *fn = chain_cluster_kernel(c->dtype, c->P, ch->mode, false);
         if (cluster_fits(fn, roles, chunks)) ch->cluster_kernel = fn;
     }
@@ -928,6 +950,8 @@ static int chain_setup_persistent(sifar_chain *ch)
             ch->dense = K < ch->K;                       /* see chain_ctas() */
             if (ch->dense) { ch->K = K; ch->C = C; }
         }
+        ch->placed = clusters_allowed && ch->mode == SIFAR_SPECULATIVE && ch->K == 1 &&
+                     units * (size_t)c->P <= kPlacedMaxPairs && cluster_fits(chain_kernel(ch), roles, chunks);
     }
     const size_t C = ch->C;
     ch->grid = (int)(C * roles);
@@ -1071,7 +1095,10 @@ extern "C" int sifar_chain_run(sifar_chain *ch, void *stream)
         void *params[] = {&a};
         if (ch->cluster_kernel) {
             const void *fn = ch->trace_on ? chain_cluster_kernel(c->dtype, c->P, ch->mode, true) : ch->cluster_kernel;
-            SIFAR_CUDA(launch_clusters(fn, no_ar ? c->P : c->P + 1, ch->C, s, params));
+            SIFAR_CUDA(launch_clusters(fn, no_ar ? c->P : c->P + 1, ch->C, s, params, true));
+        } else if (ch->placed) {
+            a.placed = 1u;
+            SIFAR_CUDA(launch_clusters(chain_kernel(ch, ch->trace_on != 0), c->P + 1, ch->C, s, params, false));
         } else {
             SIFAR_CUDA(cudaLaunchCooperativeKernel(chain_kernel(ch, ch->trace_on != 0), dim3((unsigned)ch->grid),
                                                    dim3(kChainThreads), params, 0, s));
@@ -1137,7 +1164,7 @@ extern "C" int sifar_chain_geometry(sifar_chain *ch, unsigned out[8])
     SIFAR_CUDA(cudaDeviceSynchronize());
     SIFAR_CUDA(cudaMemcpy(&h, ch->d_cs, sizeof h, cudaMemcpyDeviceToHost));
     out[0] = ch->C; out[1] = ch->K; out[2] = (unsigned)ch->grid;
-    out[3] = ch->cluster_kernel ? 1u : 0u; out[4] = ch->tagged ? 1u : 0u;
+    out[3] = (ch->cluster_kernel || ch->placed) ? 1u : 0u; out[4] = ch->tagged ? 1u : 0u;
     out[5] = h.seen[0]; out[6] = h.seen[1]; out[7] = h.seen[2];
     return SIFAR_OK;
 }
@@ -1152,8 +1179,8 @@ extern "C" int sifar_chain_trace(sifar_chain *ch, int enable, unsigned long long
         set_error("sifar_chain_trace: the traced kernel is built for P = 2 and P = 8 only");
         return SIFAR_ERR_INVALID;
     }
-    if (enable && ch->cluster_kernel &&
-        !cluster_fits(chain_cluster_kernel(ch->ctx->dtype, ch->ctx->P, ch->mode, true),
+    if (enable && (ch->cluster_kernel || ch->placed) &&
+        !cluster_fits(ch->placed ? chain_kernel(ch, true) : chain_cluster_kernel(ch->ctx->dtype, ch->ctx->P, ch->mode, true),
                       ch->ctx->P + (ch->mode == kModeNoAllreduce ? 0 : 1), ch->C)) {
         set_error("sifar_chain_trace: the traced kernel does not fit the device at this size");
         return SIFAR_ERR_INVALID;

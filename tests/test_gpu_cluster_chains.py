@@ -102,3 +102,29 @@ def test_a_cluster_that_gives_up_waits_for_the_stores_on_their_way(oracle, P, n,
         got = _rows(rings, stride, copies * steps, n, BF16)
         for i in range(copies * steps):
             assert_bits_equal(got[i], want[i % steps], BF16, f"row {i}")
+
+
+@pytest.mark.parametrize("P,dtype,pairs", [(8, BF16, 25_000), (8, F32, 25_000), (7, BF16, 40_000), (7, F32, 40_000), (8, F32, 49_000)])
+def test_speculative_chunks_meet_in_shared_memory_or_through_the_l2(monkeypatch, P, dtype, pairs):
+    """Seven and eight ranks: the largest payload whose chunks meet in shared memory and the first whose clusters are there
+    for placement only, against chunks spread over the machine; the results of two runs, the second from the first."""
+    steps = 6
+    d = synth.chain_workload("moe", P)
+    per_unit = 6 if dtype == BF16 else 3
+    for n in (pairs // P * per_unit, pairs // P * per_unit + 1):
+        results = []
+        for env in ("1", "0"):
+            monkeypatch.setenv("SIFAR_CHAIN_CLUSTER", env)
+            with Ctx(P, n, dtype) as ctx:
+                ring, stride = _ring(n, dtype, steps)
+                ch = sf.sifar_chain_create(ctx.h, sf.make_workload(**d), n, sf.SPECULATIVE, sf.CHAIN_PERSISTENT,
+                                           ring.data_ptr(), steps, steps)
+                for _ in range(2):
+                    sf.sifar_chain_run(ch, 0)
+                torch.cuda.synchronize()
+                assert sf.sifar_status(ctx.h) == 0
+                g = sf.sifar_chain_geometry(ch)
+                assert (g["clustered"], g["kernel_clustered"]) == ((1, 1) if env == "1" else (0, 0))
+                sf.sifar_chain_destroy(ch)
+                results.append(_rows(ring, stride, steps, n, dtype))
+        assert results[0][-1].any() and np.array_equal(results[0].view(np.uint8), results[1].view(np.uint8))
