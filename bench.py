@@ -771,7 +771,8 @@ def run_gpu(args) -> None:
                "h2d_bytes_per_step": ARS_PER_STEP * P * n * 2, "d2h_bytes_per_step": ARS_PER_STEP * n * 2,
                "what": "sifar_allreduce_host on pinned host buffers: one kernel reads the 8 partials straight from "
                        "host memory (H2D inside the kernel), sums them and writes the result to host memory, then "
-                       "a stream synchronisation; per call"}
+                       "a stream synchronisation; per call (nothing is packed, waited for or validated, so the mode "
+                       "makes no difference here)"}
         # -- 5. CPU oracle ---------------------------------------------------------------------------
         from oracle import oracle
         ar_us, reps_ar = oracle_allreduce_us(oracle, synth, n, 5.0)

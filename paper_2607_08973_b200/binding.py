@@ -190,6 +190,7 @@ def sifar_noalloc_max_elems() -> int:
 
 
 def sifar_noalloc_counters() -> dict:
+    """"cta_arrive" is reserved: no count of CTAs is kept between calls, so it is always 0."""
     buf = (ctypes.c_ulonglong * 3)()
     _check(lib().sifar_noalloc_counters(buf))
     return {"cta_arrive": int(buf[0]), "calls": int(buf[1]), "elements": int(buf[2])}

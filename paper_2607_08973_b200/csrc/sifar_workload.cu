@@ -235,10 +235,12 @@ __global__ void k_store_blocks(const void *src, void *dst, uint32_t *flags, unsi
 /*
  * (unit, rank) pairs up to which the result is handed over in tagged words (speculative, dual-buffered), and up to
  * which the speculative reader polls all stale ranks of its own slots (a sentinel slot per rank and warp above).
- * us per run of 64 steps, P = 8, speculative, flag / tagged with sentinel / tagged and wide: 98 KB per rank
- * 293 / 181 / 126, 128 KB 254 / 188 / 154, 195 KB (133 336 pairs) 309 / 215 / 212, 256 KB (174 768) 323 / 289 / 293,
- * 512 KB 547 / 544 / 561; dual-buffered, flag / tagged: 128 KB 250 / 227, 195 KB (100 000 pairs) 265 / 256, 256 KB
- * 335 / 318, 512 KB 529 / 567.
+ * us per run of 64 steps, spread over the machine.  Dual-buffered, flag / tagged: P = 8 bf16 128 KB per rank 254 / 229,
+ * 224 KB (114 688 pairs) 288 / 278, 256 KB (131 072) 298 / 296, 320 KB 353 / 358, 512 KB 465 / 528; P = 4 bf16 384 KB 268 /
+ * 252, 512 KB (131 072) 287 / 352: the line is where the forms cross.  Speculative, flag / tagged with sentinel / tagged
+ * and wide: P = 8 bf16 128 KB 252 / 191 / 155, 192 KB 301 / 214 / 211, 256 KB (174 768) 330 / 285 / 293, 512 KB 545 / 539 /
+ * 558; P = 8 fp32 256 KB 299 / 195 / 190, 512 KB 417 / 352 / 346; P = 4 bf16 512 KB 321 / 283 / 280: here the line lies
+ * too low, the tagged form stays ahead of the flag, and the sentinel's line would have to be parted from it.
  */
 constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE ? 170000 : 130000; }
 /*
