@@ -527,7 +527,11 @@ static int sym_setup(sifar_symchain *ch)
     ch->K = K; ch->C = (uint32_t)C; ch->grid = (int)(C * P);
     ch->clustered = false;
     if (clusters_allowed) {
-        /* one unit per thread and every chunk resident: the ranks of a chunk meet in the cluster's shared memory */
+        /* One unit per thread and every chunk resident: the ranks of a chunk meet in the cluster's shared memory.  As far
+           as that fits: us per run of 64 steps against chunks spread over the machine, bf16, both barriers / dual-buffered /
+           speculative, P = 8 64 KB per rank 152 / 106 / 124 against 302 / 230 / 151, 128 KB 205 / 161 / 192 against 371 /
+           269 / 218; P = 4 128 KB 120 / 86 / 100 against 263 / 197 / 132, 256 KB 153 / 131 / 151 against 304 / 240 / 183.
+           fp32 at P = 8 speculative is the exception at its upper end: 32 KB 85 against 103, 96 KB 144 against 135. */
         const size_t chunks = (units + kSymThreads - 1) / kSymThreads;
         const void *fn = sym_cluster_kernel(c->dtype, P, ch->mode);
         if (cluster_fits(fn, P, chunks)) {
