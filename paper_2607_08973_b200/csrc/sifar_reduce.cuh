@@ -74,6 +74,26 @@ __device__ __forceinline__ bool wait_flag_or_fail(const uint32_t *flag, uint32_t
 /* ------------------------------------------------------------------------ */
 /* rank-order accumulation                                                   */
 /* ------------------------------------------------------------------------ */
+/*
+ * acc + the low / high bf16 half of a word: the half is widened inside the add (one correctly rounded binary32 add, as
+ * with a separate widening).  A separate widening is a shift or a mask on the integer pipe, which issues every other
+ * cycle and bounds the large chains: 1.26 cycles per add and scheduler against 2.5 with a shift.  The chain of 8 KB steps,
+ * P = 8: 65.1 -> 62.9 us per 64; clusters with both barriers 115.1 -> 112.6 at 32 KB; bandwidth-bound reducers level.
+ */
+__device__ __forceinline__ float add_bf16lo(float acc, uint32_t w)
+{
+    float d;
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.bf16 %0, l, %2;\n\t}" : "=f"(d) : "r"(w), "f"(acc));
+    return d;
+}
+
+__device__ __forceinline__ float add_bf16hi(float acc, uint32_t w)
+{
+    float d;
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.bf16 %0, h, %2;\n\t}" : "=f"(d) : "r"(w), "f"(acc));
+    return d;
+}
+
 template <int DT, int P>
 __device__ __forceinline__ uint32_t sum_word(const uint32_t (&w)[P])
 {
@@ -81,8 +101,8 @@ __device__ __forceinline__ uint32_t sum_word(const uint32_t (&w)[P])
         float lo = bf16lo_to_f32(w[0]), hi = bf16hi_to_f32(w[0]);
 #pragma unroll
         for (int r = 1; r < P; ++r) {
-            lo = __fadd_rn(lo, bf16lo_to_f32(w[r]));
-            hi = __fadd_rn(hi, bf16hi_to_f32(w[r]));
+            lo = add_bf16lo(lo, w[r]);
+            hi = add_bf16hi(hi, w[r]);
         }
         return f32x2_to_bf16x2(lo, hi);
     } else {
