@@ -32,9 +32,10 @@
  *                           40000 with seven, where the cluster is there for placement only)
  *   SIFAR_CHAIN_HANDOFF_MAX persistent chain: up to this many (unit, rank) pairs a result reaches the next step's
  *                           producers in tagged 16-byte words that each thread polls for itself, above it through one
- *                           ready flag per chunk (170000 speculative, 130000 dual-buffered)
+ *                           ready flag per chunk (170000 speculative, 130000 dual-buffered; not set, speculative chains
+ *                           of more than one unit per thread go back to tagged words above 174768)
  *   SIFAR_CHAIN_WIDE_MAX    persistent speculative chain with tagged hand-over: re-poll all stale ranks per round up to
- *                           this many (slot, rank) pairs, wait on a sentinel slot above (170000)
+ *                           this many (slot, rank) pairs, wait on a sentinel slot above (320000)
  *   SIFAR_CHAIN_PDL         0 = stream / graph chains record the step events the plain way (by default the
  *                           all-reduce of a step fires its event as soon as all its CTAs have started, and the
  *                           next step's producers wait inside the kernel for its completion), and a run of a

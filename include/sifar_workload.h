@@ -139,7 +139,8 @@ int sifar_chain_chunks(sifar_chain *chain);
  * thread-block cluster (sifar.h, SIFAR_CHAIN_CLUSTER), [4] 1 = results reach the next step's producers unit by unit,
  * in tagged words or counted stores (0 = ready flag per chunk, or done flags with both barriers); from the kernel: [5] the role layout it used (1 = clustered), [6] CTAs
  * per cluster as the hardware reported them (1 without clusters), [7] the form of the hand-over it was built for.
- * Before the first run [5..7] are 0.
+ * Before the first run [5..7] are 0.  Speculative chains whose threads take several units in turn may have smaller
+ * chunks, of fewer units per thread, for the reducer than for the producers: [0] and [1] are the reducer's.
  */
 int sifar_chain_geometry(sifar_chain *chain, unsigned out[8]);
 

@@ -34,7 +34,7 @@ LIB_S8X2 = os.path.join(PKG, "libsifar_s8x2.so")
 
 # which translation units go into which library
 CORE_UNITS = ("sifar_core", "sifar_noalloc")
-BENCH_UNITS = ("sifar_workload", "sifar_symmetric", "sifar_chain_cluster")
+BENCH_UNITS = ("sifar_workload", "sifar_symmetric", "sifar_chain_cluster", "sifar_chain_pipe")
 
 NVCC_FLAGS = [
     "-std=c++17", "-O3", "-lineinfo",

@@ -47,6 +47,7 @@ struct PersistArgs {
     uint32_t steps;
     uint32_t C;                     /* chunks = reducer CTAs               */
     uint32_t K;                     /* units per thread and step           */
+    uint32_t prod_C, prod_K;        /* k_chain_pipe: the same for the producers (C, K: the readers) */
     uint32_t exit_base;
     uint32_t placed;                /* k_chain: one cluster per chunk, for placement only */
     PollShape poll;
@@ -185,6 +186,9 @@ __device__ __forceinline__ void book_sym_run(const SymArgs &a, bool marks)
    thread, kChainThreads threads per CTA.  sym_cluster_kernel() is NULL for modes that have no such form. */
 const void *chain_cluster_kernel(int dtype, int P, int mode, bool trace);
 const void *sym_cluster_kernel(int dtype, int P, int mode);
+/* The speculative chain whose threads take several units in turn (sifar_chain_pipe.cu), and how many at most. */
+constexpr uint32_t kPipeParked = 8;
+const void *chain_pipe_kernel(int dtype, int P, bool trace);
 /* Can the device hold `clusters` clusters of `cluster` CTAs of the kernel at once? */
 bool cluster_fits(const void *kernel, int cluster, size_t clusters);
 /* `dependent`: the kernel does a prologue of its own and then waits for what precedes it on the stream. */

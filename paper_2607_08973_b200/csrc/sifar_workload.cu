@@ -239,8 +239,8 @@ __global__ void k_store_blocks(const void *src, void *dst, uint32_t *flags, unsi
  * 224 KB (114 688 pairs) 288 / 278, 256 KB (131 072) 298 / 296, 320 KB 353 / 358, 512 KB 465 / 528; P = 4 bf16 384 KB 268 /
  * 252, 512 KB (131 072) 287 / 352: the line is where the forms cross.  Speculative, flag / tagged with sentinel / tagged
  * and wide: P = 8 bf16 128 KB 252 / 191 / 155, 192 KB 301 / 214 / 211, 256 KB (174 768) 330 / 285 / 293, 512 KB 545 / 539 /
- * 558; P = 8 fp32 256 KB 299 / 195 / 190, 512 KB 417 / 352 / 346; P = 4 bf16 512 KB 321 / 283 / 280: here the line lies
- * too low, the tagged form stays ahead of the flag, and the sentinel's line would have to be parted from it.
+ * 558; P = 8 fp32 256 KB 299 / 195 / 190, 512 KB 417 / 352 / 346; P = 4 bf16 512 KB 321 / 283 / 280: the tagged form stays
+ * ahead of the flag above this line too; what is above runs k_chain_pipe (kPipeMinPairs).
  */
 constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE ? 170000 : 130000; }
 /*
@@ -261,6 +261,21 @@ constexpr size_t cluster_max_pairs(int mode, int P)
     return mode != SIFAR_SPECULATIVE ? 50000 : P == 8 ? 25000 : P == 7 ? 40000 : 50000;
 }
 constexpr size_t kPlacedMaxPairs = 50000;
+/*
+ * Speculative grids whose threads take more than one unit run k_chain_pipe (sifar_chain_pipe.cu) with tagged words, up to
+ * the hand-over's line and again above this one; in between lies 256 KB per rank at P = 8 (174 768 pairs), which is
+ * documented and tested as the first payload by ready flag.  us per 64 steps, k_chain / k_chain_pipe: P = 8 bf16 160 KB per
+ * rank 206 / 176, 240 KB 255 / 207, 320 KB 378 / 302, 384 KB 418 / 366, 512 KB 544 / 425; P = 8 fp32 180 KB 150 / 138, 300 KB
+ * 305 / 161, 480 KB 407 / 280; P = 4 bf16 360 KB 216 / 177; P = 6 400 KB 364 / 286.  With one unit per thread k_chain is
+ * level or ahead (P = 8 80 KB 122 / 128, P = 4 300 KB 165 / 201).
+ */
+constexpr size_t kPipeMinPairs = 174768;
+/*
+ * Its readers (and k_chain's with tagged words) poll all stale ranks of their own slots up to this many pairs and wait on a
+ * sentinel slot per rank above.  Sentinel / wide: P = 8 bf16 240 KB 221 / 207, 384 KB (262 144 pairs) 371 / 366, 512 KB
+ * (349 528) 425 / 465; fp32 480 KB (320 008) 280 / 280.
+ */
+constexpr size_t kWideMaxPairs = 320000;
 constexpr int kPreUnits = 4;            /* units per producer thread, beyond its first, whose seeded half is computed before the wait */
 
 /*
@@ -672,7 +687,9 @@ struct sifar_chain {
     size_t handoff_stride;
     bool tagged;                    /* form of the hand-over (see handoff_store) */
     bool dense;                     /* the kernel compiled for more CTAs per SM (see chain_ctas) */
+    bool pipe;                      /* the units of a thread taken in turn (sifar_chain_pipe.cu) */
     uint32_t C, K;
+    uint32_t prod_C, prod_K;        /* of the producers, where they differ from the readers' (pipe) */
     int grid;
     const void *cluster_kernel;     /* not NULL: one thread-block cluster per chunk, whose ranks meet in its shared
                                        memory (sifar_chain_cluster.cu) */
@@ -872,6 +889,7 @@ static const void *chain_kernel_dt(int P, int mode, bool trace, bool tagged)
 static const void *chain_kernel(const sifar_chain *ch, bool trace = false)
 {
     const int P = ch->ctx->P;
+    if (ch->pipe) return chain_pipe_kernel(ch->ctx->dtype, P, trace);
     if (ch->ctx->dtype == SIFAR_BF16)
         return ch->dense ? chain_kernel_dt<SIFAR_BF16, true>(P, ch->mode, trace, ch->tagged)
                          : chain_kernel_dt<SIFAR_BF16, false>(P, ch->mode, trace, ch->tagged);
@@ -894,6 +912,27 @@ static int chain_spread(const sifar_chain *ch, size_t units, int roles, uint32_t
         chunks = (units + (size_t)kChainThreads * *K - 1) / ((size_t)kChainThreads * *K);
     }
     *C = (uint32_t)chunks;
+    return SIFAR_OK;
+}
+
+/* The layout of k_chain_pipe, for grids whose threads take more than one unit: the producers as chain_spread() lays them
+   out, the readers with as few units each as still fits beside them, but two at least (see sifar_chain_pipe.cu).  Left as
+   it is where the producers have more units than the kernel parks. */
+static int chain_take_in_turn(sifar_chain *ch, size_t units, int roles)
+{
+    const uint32_t K = ch->K, C = ch->C;
+    ch->pipe = true;
+    int rc = chain_spread(ch, units, roles, &ch->prod_K, &ch->prod_C), per_sm = 0;
+    if (rc) return rc;
+    if (ch->prod_K > kPipeParked) { ch->pipe = false; ch->K = K; ch->C = C; return SIFAR_OK; }
+    SIFAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chain_kernel(ch), kChainThreads, 0));
+    const size_t room = (size_t)per_sm * ch->ctx->sm_count - (size_t)ch->ctx->P * ch->prod_C;
+    ch->tagged = true;
+    ch->K = ch->prod_K; ch->C = ch->prod_C;
+    for (uint32_t k = 2; k < ch->prod_K; ++k) {
+        const size_t chunks = (units + (size_t)kChainThreads * k - 1) / ((size_t)kChainThreads * k);
+        if (chunks <= room) { ch->K = k; ch->C = (uint32_t)chunks; break; }
+    }
     return SIFAR_OK;
 }
 
@@ -926,7 +965,8 @@ static int chain_setup_persistent(sifar_chain *ch)
     /* how a result reaches the next step's producers: tagged words up to handoff_max_pairs() polling threads, the
        chunks' ready flags above (see handoff_store); with both barriers the done flags do it */
     size_t max_pairs = handoff_max_pairs(ch->mode);
-    if (const char *env = getenv("SIFAR_CHAIN_HANDOFF_MAX")) max_pairs = (size_t)strtoull(env, nullptr, 10);
+    const char *env_handoff = getenv("SIFAR_CHAIN_HANDOFF_MAX");
+    if (env_handoff) max_pairs = (size_t)strtoull(env_handoff, nullptr, 10);
     ch->tagged = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && units * (size_t)c->P <= max_pairs;
     /* One cluster per chunk, its ranks meeting in the cluster's shared memory, for grids up to cluster_max_pairs()
        (unit, rank) pairs that the device can hold at once with one unit per thread.  SIFAR_CHAIN_CLUSTER=0: never;
@@ -939,12 +979,14 @@ static int chain_setup_persistent(sifar_chain *ch)
         const void *fn = chain_cluster_kernel(c->dtype, c->P, ch->mode, false);
         if (cluster_fits(fn, roles, chunks)) ch->cluster_kernel = fn;
     }
-    ch->stamp_pipes = ch->cluster_kernel ? kChainThreads / 32 : 1;
     if (ch->cluster_kernel) {
         ch->K = 1; ch->C = (uint32_t)chunks;
     } else {
         int rc = chain_spread(ch, units, roles, &ch->K, &ch->C);
         if (rc) return rc;
+        if (ch->K > 1 && ch->mode == SIFAR_SPECULATIVE &&
+            (ch->tagged || (!env_handoff && units * (size_t)c->P > kPipeMinPairs)) && (rc = chain_take_in_turn(ch, units, roles)))
+            return rc;
         if (ch->K > 1 && (ch->mode == SIFAR_BARRIER_ONESHOT || ch->mode == SIFAR_DUALBUF)) {
             uint32_t K, C;
             ch->dense = true;
@@ -955,8 +997,9 @@ static int chain_setup_persistent(sifar_chain *ch)
         ch->placed = clusters_allowed && ch->mode == SIFAR_SPECULATIVE && ch->K == 1 &&
                      units * (size_t)c->P <= kPlacedMaxPairs && cluster_fits(chain_kernel(ch), roles, chunks);
     }
+    ch->stamp_pipes = (ch->cluster_kernel || ch->pipe) ? kChainThreads / 32 : 1;
     const size_t C = ch->C;
-    ch->grid = (int)(C * roles);
+    ch->grid = (int)(ch->pipe ? C + (size_t)c->P * ch->prod_C : C * roles);
     SIFAR_CUDA(cudaMalloc(&ch->d_cs, sizeof(ChainDev)));
     SIFAR_CUDA(cudaMalloc(&ch->d_chunks, sizeof(ChunkFlags) * C));
     SIFAR_CUDA(cudaMalloc(&ch->d_stamps, sizeof(unsigned long long) * (ch->steps + 1) * C * ch->stamp_pipes));
@@ -1078,13 +1121,12 @@ extern "C" int sifar_chain_run(sifar_chain *ch, void *stream)
         a.ring = ch->ring; a.ring_stride = ch->ring_stride; a.ring_len = (uint32_t)ch->ring_len;
         a.e0 = no_ar ? ch->base_epoch + ch->runs * (uint32_t)ch->steps : c->h_epoch;
         a.base_epoch = ch->base_epoch; a.steps = (uint32_t)ch->steps;
-        a.C = ch->C; a.K = ch->K;
+        a.C = ch->C; a.K = ch->K; a.prod_C = ch->prod_C; a.prod_K = ch->prod_K;
         a.poll = poll_shape_for(c, ch->n);
         if (ch->tagged && ch->mode == SIFAR_SPECULATIVE) {
             /* with the tagged hand-over the producers store sooner after the reducer's result, and the reducer does
-               best polling all stale ranks of its own slots up to a larger grid than the discrete reducer's (see
-               handoff_max_pairs) */
-            size_t wide_max = handoff_max_pairs(ch->mode);
+               best polling all stale ranks of its own slots up to a larger grid than the discrete reducer's */
+            size_t wide_max = kWideMaxPairs;
             if (const char *env = getenv("SIFAR_CHAIN_WIDE_MAX")) wide_max = (size_t)strtoull(env, nullptr, 10);
             const bool wide = slots_for(c->dtype, ch->n) * (size_t)c->P <= wide_max;
             a.poll.wide = wide ? 1u : 0u;
