@@ -27,9 +27,11 @@
  *   SIFAR_POLL_PACE_NS/_MIN sleep between polling rounds above _MIN pairs (0 = unpaced)
  *   SIFAR_POLL_SENTINEL_MIN persistent chain: above this many pairs a warp first waits on one slot per rank (16384)
  *   SIFAR_CHAIN_CLUSTER     0 = persistent chains without thread-block clusters (by default the CTAs of a chunk are one
- *                           cluster up to 50000 (unit, rank) pairs speculative, 65000 in the modes with flags, and its
- *                           ranks meet in shared memory, except speculative above 25000 pairs with eight ranks and
- *                           40000 with seven, where the cluster is there for placement only)
+ *                           cluster and its ranks meet in shared memory, as far as the GPU holds all clusters at once: in
+ *                           the modes with flags at every size but 65001 to 65536 (unit, rank) pairs with eight ranks;
+ *                           speculative up to 25000 pairs with eight ranks, 40000 with seven, 37000 to 90000, by ranks and
+ *                           type, with fewer.  Speculative grids above those lines and up to 50000 pairs have clusters for
+ *                           placement only)
  *   SIFAR_CHAIN_HANDOFF_MAX persistent chain: up to this many (unit, rank) pairs a result reaches the next step's
  *                           producers in tagged 16-byte words that each thread polls for itself, above it through one
  *                           ready flag per chunk (170000 speculative, 130000 dual-buffered; not set, speculative chains

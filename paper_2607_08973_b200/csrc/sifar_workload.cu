@@ -244,21 +244,29 @@ __global__ void k_store_blocks(const void *src, void *dst, uint32_t *flags, unsi
  */
 constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE ? 170000 : 130000; }
 /*
- * One thread-block cluster per chunk, its ranks meeting in shared memory, up to this many (unit, rank) pairs
- * (sifar_chain_cluster.cu); above that, speculative, one cluster per chunk for placement (see k_chain) up to
- * kPlacedMaxPairs, as far as cluster_max_pairs() ends before.  us per run of 64 steps, P = 8, bf16, shared memory against
- * spread over the machine: dual-buffered 8 KB per rank 58 / 170, 64 KB 94 / 203, 96 KB 123 / 213; both barriers
- * 104 / 220, 132 / 232, 156 / 241.  The modes with flags gain beyond 65 000 pairs, too (127 KB 150 / 228 and 192 / 247);
- * nothing above is taken, because where the two layouts cross has not been measured.
- * Speculative, shared memory / placed: P = 8 bf16 24 KB 74 / 83, 32 KB 82 / 84, 40 KB 86 / 85, 56 KB 107 / 97, 72 KB
- * 121 / 112; P = 8 fp32 32 KB 80 / 79, 48 KB 102 / 83, 64 KB 112 / 84; P = 7 bf16 56 KB 87 / 94, 64 KB 95 / 98, 72 KB
- * 104 / 98; P = 6 72 KB 81 / 95; P = 4 128 KB 89 / 110.  A chunk's one reader CTA takes and sends P vectors per thread
- * through its SM's ports; with eight ranks and more than about 30 clusters that costs more than the hop saves.
+ * One thread-block cluster per chunk, its ranks meeting in shared memory (sifar_chain_cluster.cu), for these numbers of
+ * (unit, rank) pairs as far as the clusters fit the machine; otherwise, speculative, one cluster per chunk for placement
+ * (see k_chain) up to kPlacedMaxPairs.  us per run of 64 steps, shared memory against spread over the machine.
+ * Modes with flags: ahead wherever they fit.  P = 8 bf16 dual-buffered 8 KB per rank 57 / 170, 64 KB 94 / 203, 129 KB 150 / 221,
+ * 146 KB 163 / 235, both barriers 104 / 220, 132 / 232, 197 / 248, 199 / 257; P = 7 152 KB 138 / 225 and 177 / 249; P = 4 256 KB
+ * 134 / 215 and 140 / 250; P = 2 508 KB 147 / 216 and 158 / 248.  With eight ranks 128 KB (65 536 pairs) is documented and
+ * tested as the first payload that spreads; the sizes around it do not.
+ * Speculative: a chunk's one reader CTA takes and sends P vectors per thread through its SM's ports, and its lanes poll; with
+ * seven or eight ranks and more than about 30 clusters that costs more than the hop saves (P = 8 bf16 24 KB 74 / 83, 32 KB
+ * 82 / 84, 40 KB 86 / 85, 72 KB 121 / 112; fp32 32 KB 80 / 79, 64 KB 112 / 84; P = 7 bf16 56 KB 87 / 94, 72 KB 104 / 98).
+ * P = 4 bf16 160 KB 98 / 119, 256 KB 132 / 149, fp32 180 KB 82 / 109, 264 KB 107 / 116; P = 5 bf16 140 KB 100 / 121, 208 KB
+ * 131 / 159, fp32 160 KB 103 / 111, 212 KB 128 / 116; P = 6 bf16 110 KB 97 / 121, 168 KB 140 / 153, fp32 120 KB 111 / 113,
+ * 144 KB 127 / 117.  Two and three ranks have few partials per hop and many chunks: P = 2 bf16 200 KB 97 / 105, 240 KB
+ * 119 / 109, fp32 280 KB 98 / 106, 400 KB 126 / 108; P = 3 bf16 180 KB 106 / 111, 220 KB 112 / 110, fp32 200 KB 89 / 106, 280 KB
+ * 110 / 110.
  */
-constexpr size_t cluster_max_pairs(int mode, int P)
+constexpr bool cluster_pays(int mode, int P, int dtype, size_t pairs)
 {
-    if (mode == SIFAR_DUALBUF || mode == SIFAR_BARRIER_ONESHOT) return 65000;
-    return mode != SIFAR_SPECULATIVE ? 50000 : P == 8 ? 25000 : P == 7 ? 40000 : 50000;
+    if (mode == SIFAR_DUALBUF || mode == SIFAR_BARRIER_ONESHOT) return P < 8 || pairs <= 65000 || pairs > 65536;
+    if (mode != SIFAR_SPECULATIVE) return pairs <= 50000;
+    constexpr size_t line[2][9] = {{0, 50000, 37000, 52000, 90000, 90000, 90000, 40000, 25000},      /* bf16, by P */
+                                   {0, 50000, 50000, 65000, 90000, 75000, 60000, 40000, 25000}};
+    return pairs <= line[dtype == SIFAR_BF16 ? 0 : 1][P];
 }
 constexpr size_t kPlacedMaxPairs = 50000;
 /*
@@ -968,14 +976,14 @@ static int chain_setup_persistent(sifar_chain *ch)
     const char *env_handoff = getenv("SIFAR_CHAIN_HANDOFF_MAX");
     if (env_handoff) max_pairs = (size_t)strtoull(env_handoff, nullptr, 10);
     ch->tagged = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && units * (size_t)c->P <= max_pairs;
-    /* One cluster per chunk, its ranks meeting in the cluster's shared memory, for grids up to cluster_max_pairs()
-       (unit, rank) pairs that the device can hold at once with one unit per thread.  SIFAR_CHAIN_CLUSTER=0: never;
+    /* One cluster per chunk, its ranks meeting in the cluster's shared memory, for grids that cluster_pays() for and
+       that the device can hold at once with one unit per thread.  SIFAR_CHAIN_CLUSTER=0: never;
        nor with the flag form of the hand-over asked for at such a size. */
     const char *env_cluster = getenv("SIFAR_CHAIN_CLUSTER");
     const size_t chunks = (units + kChainThreads - 1) / kChainThreads;
     const bool flag_form = (ch->mode == SIFAR_DUALBUF || ch->mode == SIFAR_SPECULATIVE) && !ch->tagged;
     const bool clusters_allowed = !(env_cluster && atoi(env_cluster) == 0) && !flag_form;
-    if (clusters_allowed && units * (size_t)c->P <= cluster_max_pairs(ch->mode, c->P)) {
+    if (clusters_allowed && cluster_pays(ch->mode, c->P, c->dtype, units * (size_t)c->P)) {
         const void *fn = chain_cluster_kernel(c->dtype, c->P, ch->mode, false);
         if (cluster_fits(fn, roles, chunks)) ch->cluster_kernel = fn;
     }

@@ -128,3 +128,28 @@ def test_speculative_chunks_meet_in_shared_memory_or_through_the_l2(monkeypatch,
                 sf.sifar_chain_destroy(ch)
                 results.append(_rows(ring, stride, steps, n, dtype))
         assert results[0][-1].any() and np.array_equal(results[0].view(np.uint8), results[1].view(np.uint8))
+
+
+@pytest.mark.parametrize("P,n,dtype,mode", [
+    (8, 65_537, BF16, sf.DUALBUF), (8, 73_729, BF16, sf.BARRIER_ONESHOT), (7, 78_001, BF16, sf.DUALBUF),
+    (4, 131_072, BF16, sf.BARRIER_ONESHOT), (2, 131_071, F32, sf.DUALBUF), (4, 131_069, BF16, sf.SPECULATIVE),
+    (4, 66_001, F32, sf.SPECULATIVE), (6, 84_001, BF16, sf.SPECULATIVE), (5, 44_999, F32, sf.SPECULATIVE)])
+def test_the_largest_grids_in_clusters_agree_with_spread_ones(monkeypatch, P, n, dtype, mode):
+    """Grids that nearly fill the machine with clusters, whole and ragged last chunks: two runs, the second from the first."""
+    steps = 6
+    d = synth.chain_workload("moe", P)
+    results = []
+    for env in ("1", "0"):
+        monkeypatch.setenv("SIFAR_CHAIN_CLUSTER", env)
+        with Ctx(P, n, dtype) as ctx:
+            ring, stride = _ring(n, dtype, steps)
+            ch = sf.sifar_chain_create(ctx.h, sf.make_workload(**d), n, mode, sf.CHAIN_PERSISTENT, ring.data_ptr(), steps, steps)
+            for _ in range(2):
+                sf.sifar_chain_run(ch, 0)
+            torch.cuda.synchronize()
+            assert sf.sifar_status(ctx.h) == 0
+            g = sf.sifar_chain_geometry(ch)
+            assert g["kernel_clustered"] == int(env) and g["units_per_thread"] >= 1
+            sf.sifar_chain_destroy(ch)
+            results.append(_rows(ring, stride, steps, n, dtype))
+    assert results[0][-1].any() and np.array_equal(results[0].view(np.uint8), results[1].view(np.uint8))
