@@ -59,6 +59,10 @@ struct ProduceArgs {
     uint32_t base_epoch;       /* step t = call number - base_epoch                                 */
     uint32_t parity;
     uint32_t t_fixed;          /* no-all-reduce chains: the step, since no call number advances     */
+    uint4 *handoff;            /* k_produce_tagged: [parity][slot], results as their reducers hand them over       */
+    unsigned long long handoff_stride;
+    uint32_t *step_word;       /* ... by parity, the call number that the step's producers found                   */
+    uint32_t opening;          /* ... 1: first step of a run, the call number is the one published                 */
 };
 
 constexpr int kProdThreads = 128;
@@ -166,6 +170,67 @@ __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
         if (MODE != kModeNoAllreduce)
             signal_arrival(&st->pack_count[rank], gridDim.x, &st->arrive[e & 1u][rank], e);
     }
+}
+
+/*
+ * Producer kernel of the graph chain in tagged slots (sifar_chain::by_tags): nothing of it waits for a kernel.  A thread
+ * polls the previous result of its slots where the reducer hands it over slot by slot (call number in the word), as in the
+ * persistent kernels, and stores slots that carry their own tags.  What bounds a step is then these two hops and the two
+ * launches, not the ends of kernels: producers and reducers are two rows of programmatic launches that meet in the data
+ * alone, each kernel letting the next of its row in once it has what it waits for.  us per 64 steps, by events / by tags:
+ * P = 8 bf16 8 KB per rank 223 / 148, 32 KB 270 / 153, 140 KB 325 / 240; P = 2 60 KB 303 / 180; P = 4 fp32 240 KB 359 / 211.
+ * For the slot format up to kConcurrentTiles reducer CTAs (above that a step's reducer is ordered behind its producers).
+ */
+template <int DT>
+__global__ void __launch_bounds__(kProdThreads) k_produce_tagged(const ProduceArgs a)
+{
+    constexpr int NE = 3 * ((DT == SIFAR_BF16) ? 2 : 1);
+    DevState *st = a.st;
+    const uint32_t rank = a.rank + blockIdx.y;
+    uint4 *dst = reinterpret_cast<uint4 *>(a.dst + rank * a.dst_stride);
+    const size_t tid = (size_t)blockIdx.x * kProdThreads + threadIdx.x;
+    const size_t nthreads = (size_t)gridDim.x * kProdThreads;
+    const size_t n = (size_t)a.n, nslots = (n + NE - 1) / NE;
+    __shared__ uint32_t s_e;
+    /* The call number: the first step of a run finds it published; a later one is let in while the calls before it are
+       still on their way and takes it from the step before, which left it before it let this one in. */
+    if (threadIdx.x == 0) {
+        uint32_t e = a.opening ? ld_relaxed_u32(&st->epoch) + 1u : ld_relaxed_u32(a.step_word + (a.parity ^ 1u)) + 1u;
+        if (ld_relaxed_u32(&st->status) != 0u) e = 0u;
+        if (e && (e & 1u) != a.parity) { fail(st, a.host_status, SIFAR_ERR_EPOCH); e = 0u; }
+        if (e && blockIdx.x == 0 && rank == 0u) {
+            st_relaxed_u32(a.step_word + a.parity, e);
+            __threadfence();
+        }
+        s_e = e;
+    }
+    __syncthreads();
+    const uint32_t e = s_e, t = e - a.base_epoch;
+    if (e != 0u) {
+        const bool first = (t == 1u);
+        const uint4 *prev = a.handoff + (size_t)((e - 1u) & 1u) * a.handoff_stride;
+        Gen g = make_gen(a.w, rank, t);
+        float z[NE];
+        if (tid < nslots) {
+            unit_noise<DT, 3>(g, first, tid * NE, z);
+#pragma unroll
+            for (int k = 0; k < NE; ++k) asm volatile("" : "+f"(z[k]));
+        }
+        for (size_t s = tid; s < nslots; s += nthreads) {
+            uint32_t pw[3] = {0u, 0u, 0u}, w[3];
+            if (!first && !handoff_wait<3>(prev, s, e - 1u, pw, st, a.host_status, a.timeout_ns)) break;
+            if (s == tid) {
+                /* the next step's producers get ready beside this step's reducer, no further step's */
+                asm volatile("griddepcontrol.launch_dependents;");
+                if (a.w.delay_max_ns != 0u) spin_ns(gen_delay_ns(a.w, rank, t));
+            } else {
+                unit_noise<DT, 3>(g, first, s * NE, z);
+            }
+            unit_apply<DT, 3>(g, first, pw, s * NE, n, z, w);
+            store_slot(dst, s, w[0], w[1], w[2], e);
+        }
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");     /* nothing is left to do: the row of producers ends in order */
 }
 
 /* Generator probes: plain elements to dst, no protocol. */
@@ -693,6 +758,7 @@ struct sifar_chain {
     uint32_t *d_retry_steps;
     uint4 *d_handoff;
     size_t handoff_stride;
+    bool by_tags;                   /* graph chain, speculative and concurrent, whose kernels wait for tagged words only (k_produce_tagged) */
     bool tagged;                    /* form of the hand-over (see handoff_store) */
     bool dense;                     /* the kernel compiled for more CTAs per SM (see chain_ctas) */
     bool pipe;                      /* the units of a thread taken in turn (sifar_chain_pipe.cu) */
@@ -741,6 +807,7 @@ static cudaError_t preload_produce()
     if (e == cudaSuccess) e = preload(k_produce<DT, SIFAR_DUALBUF>);
     if (e == cudaSuccess) e = preload(k_produce<DT, SIFAR_SPECULATIVE>);
     if (e == cudaSuccess) e = preload(k_produce<DT, kModeNoAllreduce>);
+    if (e == cudaSuccess) e = preload(k_produce_tagged<DT>);
     return e;
 }
 
@@ -768,6 +835,18 @@ static cudaError_t launch_produce_dt(int mode, dim3 grid, cudaStream_t s, const 
     default:                    k_produce<DT, kModeNoAllreduce><<<grid, kProdThreads, 0, s>>>(a); break;
     }
     return cudaGetLastError();
+}
+
+template <int DT>
+static cudaError_t launch_produce_tagged(dim3 grid, bool dependent, cudaStream_t s, const ProduceArgs &a)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(kProdThreads); cfg.stream = s;
+    cfg.attrs = at; cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_produce_tagged<DT>, a);
 }
 
 /* Producer streams of a stream / graph chain (see enqueue_run). */
@@ -812,7 +891,7 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
         const uint32_t t = first_t + (uint32_t)s;
         const uint32_t e = ch->base_epoch + t;
         for (int r = 0; r < lanes; ++r) {
-            if (s > 0 && !no_ar) SIFAR_CUDA(cudaStreamWaitEvent(ch->prod[r], ch->ev_step[s - 1], 0));
+            if (s > 0 && !no_ar && !ch->by_tags) SIFAR_CUDA(cudaStreamWaitEvent(ch->prod[r], ch->ev_step[s - 1], 0));
             ProduceArgs a;
             memset(&a, 0, sizeof a);
             a.st = c->d_state; a.host_status = c->d_status_alias; a.timeout_ns = c->timeout_ns;
@@ -824,6 +903,15 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
             a.prev_stride = no_ar ? c->plain_stride : 0u;
             a.base_epoch = ch->base_epoch; a.parity = e & 1u;
             a.t_fixed = no_ar ? t : 0u;
+            if (ch->by_tags) {
+                a.handoff = ch->d_handoff; a.handoff_stride = ch->handoff_stride;
+                a.step_word = reinterpret_cast<uint32_t *>(ch->d_handoff + 2 * ch->handoff_stride);
+                a.opening = s == 0 ? 1u : 0u;
+                const dim3 grid((unsigned)pgrid, (unsigned)P);
+                SIFAR_CUDA(c->dtype == SIFAR_BF16 ? launch_produce_tagged<SIFAR_BF16>(grid, s > 0, ch->prod[r], a)
+                                                  : launch_produce_tagged<SIFAR_F32>(grid, s > 0, ch->prod[r], a));
+                continue;
+            }
             cudaError_t err = (c->dtype == SIFAR_BF16)
                 ? launch_produce_dt<SIFAR_BF16>(ch->mode, dim3((unsigned)pgrid, (unsigned)(P / lanes)), ch->prod[r], a)
                 : launch_produce_dt<SIFAR_F32>(ch->mode, dim3((unsigned)pgrid, (unsigned)(P / lanes)), ch->prod[r], a);
@@ -846,10 +934,15 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
                out of every step (CUDA-graph chain at 8 KB, P = 8: 7.5 -> 4.9 us per step).  SIFAR_CHAIN_PDL=0
                records the event the plain way. */
             static const bool early = !(getenv("SIFAR_CHAIN_PDL") && atoi(getenv("SIFAR_CHAIN_PDL")) == 0);
-            if (early) rl.programmatic_event = ch->ev_step[s];
+            if (ch->by_tags) {
+                rl.handoff = ch->d_handoff + (size_t)(e & 1u) * ch->handoff_stride;
+                rl.chained = rl.early = s > 0;
+            } else if (early) {
+                rl.programmatic_event = ch->ev_step[s];
+            }
             int rc = launch_reduce(c, rl, ch->red);
             if (rc) return rc;
-            if (!early) SIFAR_CUDA(cudaEventRecord(ch->ev_step[s], ch->red));
+            if (!early && !ch->by_tags) SIFAR_CUDA(cudaEventRecord(ch->ev_step[s], ch->red));
         }
     }
     for (int r = 0; r < lanes; ++r) {
@@ -1070,6 +1163,15 @@ extern "C" sifar_chain *sifar_chain_create(sifar_ctx *c, const sifar_workload *w
         for (int r = 0; r <= c->P; ++r) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_join[r], cudaEventDisableTiming));
         for (int r = 0; r < c->P; ++r) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_prod[r], cudaEventDisableTiming));
         ch->concurrent = reduce_tiles(c, n, mode == kModeNoAllreduce ? SIFAR_DUALBUF : mode) <= kConcurrentTiles;
+        const char *env_pdl = getenv("SIFAR_CHAIN_PDL");
+        ch->by_tags = impl == SIFAR_CHAIN_GRAPH && mode == SIFAR_SPECULATIVE && ch->concurrent && dependent_launches() &&
+                      !(env_pdl && atoi(env_pdl) == 0);
+        if (ch->by_tags) {
+            ch->handoff_stride = slots_for(c->dtype, n);
+            /* the words of both parities, then the step words; zero = call number 0 = never valid */
+            SIFAR_CUDA(cudaMalloc(&ch->d_handoff, (2 * ch->handoff_stride + 1) * sizeof(uint4)));
+            SIFAR_CUDA(cudaMemset(ch->d_handoff, 0, (2 * ch->handoff_stride + 1) * sizeof(uint4)));
+        }
         ch->ev_step.assign((size_t)ch->steps, nullptr);
         for (int s = 0; s < ch->steps; ++s) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_step[s], cudaEventDisableTiming));
         ch->launches_per_run = ch->steps * (producer_streams(ch) + (mode == kModeNoAllreduce ? 0 : 1));      /* one reducer kernel per all-reduce */
