@@ -562,11 +562,13 @@ static int sym_setup(sifar_symchain *ch)
     SIFAR_CUDA(cudaMalloc(&ch->d_stamps, sizeof(unsigned long long) * nstamps));
     SIFAR_CUDA(cudaMalloc(&ch->d_marks, sizeof(uint32_t) * P * ch->steps));
     SIFAR_CUDA(cudaMalloc(&ch->d_rank_retries, sizeof(unsigned long long) * kMaxRanks));
-    SIFAR_CUDA(cudaMemset(ch->d_cs, 0, sizeof(SymDev)));
-    SIFAR_CUDA(cudaMemset(ch->d_flags, 0, sizeof(SymFlags) * ch->C));
-    SIFAR_CUDA(cudaMemset(ch->d_stamps, 0, sizeof(unsigned long long) * nstamps));
-    SIFAR_CUDA(cudaMemset(ch->d_marks, 0, sizeof(uint32_t) * P * ch->steps));
-    SIFAR_CUDA(cudaMemset(ch->d_rank_retries, 0, sizeof(unsigned long long) * kMaxRanks));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_cs, 0, sizeof(SymDev), c->host_stream));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_flags, 0, sizeof(SymFlags) * ch->C, c->host_stream));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_stamps, 0, sizeof(unsigned long long) * nstamps, c->host_stream));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_marks, 0, sizeof(uint32_t) * P * ch->steps, c->host_stream));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_rank_retries, 0, sizeof(unsigned long long) * kMaxRanks, c->host_stream));
+    /* the chain's state is zero before its first run, which no stream orders behind the memsets */
+    SIFAR_CUDA(cudaStreamSynchronize(c->host_stream));
     return SIFAR_OK;
 }
 

@@ -1105,12 +1105,12 @@ static int chain_setup_persistent(sifar_chain *ch)
     SIFAR_CUDA(cudaMalloc(&ch->d_chunks, sizeof(ChunkFlags) * C));
     SIFAR_CUDA(cudaMalloc(&ch->d_stamps, sizeof(unsigned long long) * (ch->steps + 1) * C * ch->stamp_pipes));
     SIFAR_CUDA(cudaMalloc(&ch->d_trace, sizeof(unsigned long long) * ch->steps * kTraceSlots));
-    SIFAR_CUDA(cudaMemset(ch->d_trace, 0, sizeof(unsigned long long) * ch->steps * kTraceSlots));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_trace, 0, sizeof(unsigned long long) * ch->steps * kTraceSlots, c->host_stream));
     SIFAR_CUDA(cudaMalloc(&ch->d_retry_steps, sizeof(uint32_t) * ch->steps));
-    SIFAR_CUDA(cudaMemset(ch->d_cs, 0, sizeof(ChainDev)));
-    SIFAR_CUDA(cudaMemset(ch->d_chunks, 0, sizeof(ChunkFlags) * C));
-    SIFAR_CUDA(cudaMemset(ch->d_stamps, 0, sizeof(unsigned long long) * (ch->steps + 1) * C * ch->stamp_pipes));
-    SIFAR_CUDA(cudaMemset(ch->d_retry_steps, 0, sizeof(uint32_t) * ch->steps));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_cs, 0, sizeof(ChainDev), c->host_stream));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_chunks, 0, sizeof(ChunkFlags) * C, c->host_stream));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_stamps, 0, sizeof(unsigned long long) * (ch->steps + 1) * C * ch->stamp_pipes, c->host_stream));
+    SIFAR_CUDA(cudaMemsetAsync(ch->d_retry_steps, 0, sizeof(uint32_t) * ch->steps, c->host_stream));
     /* the hand-over buffer (see handoff_store): one 16-byte word per 12-byte unit, two per 16-byte vector, whole
        warps of units, both parities; zero = tag 0 = never valid.  Large grids use the chunks' ready flags instead. */
     if (ch->tagged || ch->mode == kModeNoAllreduce) {
@@ -1119,7 +1119,7 @@ static int chain_setup_persistent(sifar_chain *ch)
         const size_t sets = (ch->mode == kModeNoAllreduce) ? (size_t)c->P : 1;
         ch->handoff_stride = padded * (ch->mode == SIFAR_DUALBUF ? 2 : 1);
         SIFAR_CUDA(cudaMalloc(&ch->d_handoff, 2 * sets * ch->handoff_stride * sizeof(uint4)));
-        SIFAR_CUDA(cudaMemset(ch->d_handoff, 0, 2 * sets * ch->handoff_stride * sizeof(uint4)));
+        SIFAR_CUDA(cudaMemsetAsync(ch->d_handoff, 0, 2 * sets * ch->handoff_stride * sizeof(uint4), c->host_stream));
     }
     return SIFAR_OK;
 }
@@ -1170,7 +1170,7 @@ extern "C" sifar_chain *sifar_chain_create(sifar_ctx *c, const sifar_workload *w
             ch->handoff_stride = slots_for(c->dtype, n);
             /* the words of both parities, then the step words; zero = call number 0 = never valid */
             SIFAR_CUDA(cudaMalloc(&ch->d_handoff, (2 * ch->handoff_stride + 1) * sizeof(uint4)));
-            SIFAR_CUDA(cudaMemset(ch->d_handoff, 0, (2 * ch->handoff_stride + 1) * sizeof(uint4)));
+            SIFAR_CUDA(cudaMemsetAsync(ch->d_handoff, 0, (2 * ch->handoff_stride + 1) * sizeof(uint4), c->host_stream));
         }
         ch->ev_step.assign((size_t)ch->steps, nullptr);
         for (int s = 0; s < ch->steps; ++s) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_step[s], cudaEventDisableTiming));
@@ -1193,6 +1193,11 @@ extern "C" sifar_chain *sifar_chain_create(sifar_ctx *c, const sifar_workload *w
         return SIFAR_OK;
     };
     rc = setup();
+    /* the chain's state is zero before its first run, which no stream orders behind the memsets */
+    if (!rc) {
+        const cudaError_t e = cudaStreamSynchronize(c->host_stream);
+        if (e != cudaSuccess) rc = cuda_fail(e, "cudaStreamSynchronize");
+    }
     if (rc) { cudaGetLastError(); chain_free(ch); return nullptr; }
     return ch;
 }
