@@ -191,8 +191,10 @@ constexpr uint32_t kPipeParked = 8;
 const void *chain_pipe_kernel(int dtype, int P, bool trace);
 /* Can the device hold `clusters` clusters of `cluster` CTAs of the kernel at once? */
 bool cluster_fits(const void *kernel, int cluster, size_t clusters);
-/* `dependent`: the kernel does a prologue of its own and then waits for what precedes it on the stream. */
-cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params, bool dependent);
+/* `dependent`: the kernel does a prologue of its own and then waits for what precedes it on the stream.  `by_load`: the
+   CTAs go where the fewest are (cluster_by_load). */
+cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params, bool dependent,
+                            bool by_load);
 
 }  /* namespace sifar */
 #endif

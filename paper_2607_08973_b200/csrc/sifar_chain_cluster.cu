@@ -582,6 +582,8 @@ const void *sym_cluster_kernel(int dtype, int P, int mode)
     return dtype == SIFAR_BF16 ? sym_cluster_dt<SIFAR_BF16>(P, mode) : sym_cluster_dt<SIFAR_F32>(P, mode);
 }
 
+/* Asked for the default placement; by load the device holds as many clusters or more (reported on B200, default / by load:
+   nine CTAs 93 / 96, seven 142 / 148, five 168 / 174, three 284 / 296). */
 bool cluster_fits(const void *kernel, int cluster, size_t clusters)
 {
     if (!kernel) return false;
@@ -595,16 +597,16 @@ bool cluster_fits(const void *kernel, int cluster, size_t clusters)
     return (size_t)most >= clusters;
 }
 
-cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params, bool dependent)
+cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params, bool dependent,
+                            bool by_load)
 {
     static const bool early = !(getenv("SIFAR_CHAIN_PDL") && atoi(getenv("SIFAR_CHAIN_PDL")) == 0);
     cudaLaunchAttribute attr[3];
     cudaLaunchConfig_t cfg = cluster_config(attr, cluster, clusters, kChainThreads, stream);
-    /* where the CTAs of a cluster go: by load, not as the hardware likes them best.  us per 64 steps, default / by load:
-       P = 8 dual-buffered 60 KB 87 / 81, P = 2 450 KB 135 / 126, P = 4 speculative 256 KB 142 / 134; grids of at most one CTA
-       per SM level */
-    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterSchedulingPolicyPreference;
-    attr[cfg.numAttrs++].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
+    if (by_load) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterSchedulingPolicyPreference;
+        attr[cfg.numAttrs++].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
+    }
     if (dependent && early) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;

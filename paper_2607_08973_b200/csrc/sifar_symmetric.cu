@@ -635,7 +635,7 @@ extern "C" int sifar_symchain_run(sifar_symchain *ch, void *stream)
     const void *fn = sym_kernel(ch);
     cudaStream_t s = (cudaStream_t)stream;
     if (ch->cluster_kernel) {
-        SIFAR_CUDA(launch_clusters(ch->cluster_kernel, c->P, ch->C, s, params, true));
+        SIFAR_CUDA(launch_clusters(ch->cluster_kernel, c->P, ch->C, s, params, true, false));
     } else if (ch->clustered) {
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof cfg);

@@ -335,6 +335,21 @@ constexpr bool cluster_pays(int mode, int P, int dtype, size_t pairs)
 }
 constexpr size_t kPlacedMaxPairs = 50000;
 /*
+ * Where the CTAs of a cluster go: as the hardware likes them best, or by load (cudaClusterSchedulingPolicyLoadBalancing).  The
+ * busiest SM sets the pace of a step.  Left alone the hardware puts one CTA more than need be on some SMs where the last
+ * level of CTAs per SM is nearly full, and that is where placing by load pays; elsewhere it is level or, with its CTAs
+ * farther apart, slower.  us per 64 steps, default / by load, by CTAs per SM: P = 5 fp32 dual-buffered 2.9 86 / 73, P = 8 fp32
+ * both barriers 4.9 228 / 198, P = 7 bf16 both barriers 3.9 175 / 150, P = 2 bf16 both barriers 2.9 112 / 94; against
+ * it P = 2 bf16 dual-buffered 1.8 68 / 76, P = 3 bf16 both barriers 1.0 80 / 88, P = 6 fp32 dual-buffered 4.9 121 / 140 and 1.1
+ * 50 / 56, P = 4 fp32 dual-buffered 4.9 94 / 100.  Over 1161 chains of one reader the rule takes it for 146, 4.2 % faster on
+ * average and none more than 3 % slower; with P readers it is level at best (both barriers 1.3 % slower) and not taken.
+ */
+constexpr bool cluster_by_load(int mode, int P, int dtype, size_t ctas, size_t sms)
+{
+    if (ctas <= sms || P == 6 || (P == 4 && dtype == SIFAR_F32 && mode == SIFAR_DUALBUF)) return false;
+    return ctas % sms * 100 >= sms * (P >= 7 ? 50 : 82);
+}
+/*
  * Speculative grids whose threads take more than one unit run k_chain_pipe (sifar_chain_pipe.cu) with tagged words, up to
  * the hand-over's line and again above this one; in between lies 256 KB per rank at P = 8 (174 768 pairs), which is
  * documented and tested as the first payload by ready flag.  us per 64 steps, k_chain / k_chain_pipe: P = 8 bf16 160 KB per
@@ -768,6 +783,7 @@ struct sifar_chain {
     const void *cluster_kernel;     /* not NULL: one thread-block cluster per chunk, whose ranks meet in its shared
                                        memory (sifar_chain_cluster.cu) */
     bool placed;                    /* k_chain in one cluster per chunk, for placement */
+    bool by_load;                   /* ... placed by load (cluster_by_load) */
     uint32_t stamp_pipes;           /* rows of stamps per chunk (see PersistArgs::stamps) */
 };
 
@@ -1098,6 +1114,7 @@ static int chain_setup_persistent(sifar_chain *ch)
         ch->placed = clusters_allowed && ch->mode == SIFAR_SPECULATIVE && ch->K == 1 &&
                      units * (size_t)c->P <= kPlacedMaxPairs && cluster_fits(chain_kernel(ch), roles, chunks);
     }
+    ch->by_load = cluster_by_load(ch->mode, c->P, c->dtype, (size_t)ch->C * roles, (size_t)c->sm_count);
     ch->stamp_pipes = (ch->cluster_kernel || ch->pipe) ? kChainThreads / 32 : 1;
     const size_t C = ch->C;
     ch->grid = (int)(ch->pipe ? C + (size_t)c->P * ch->prod_C : C * roles);
@@ -1254,10 +1271,11 @@ extern "C" int sifar_chain_run(sifar_chain *ch, void *stream)
         void *params[] = {&a};
         if (ch->cluster_kernel) {
             const void *fn = ch->trace_on ? chain_cluster_kernel(c->dtype, c->P, ch->mode, true) : ch->cluster_kernel;
-            SIFAR_CUDA(launch_clusters(fn, no_ar ? c->P : c->P + 1, ch->C, s, params, true));
+            SIFAR_CUDA(launch_clusters(fn, no_ar ? c->P : c->P + 1, ch->C, s, params, true, ch->by_load));
         } else if (ch->placed) {
             a.placed = 1u;
-            SIFAR_CUDA(launch_clusters(chain_kernel(ch, ch->trace_on != 0), c->P + 1, ch->C, s, params, false));
+            SIFAR_CUDA(launch_clusters(chain_kernel(ch, ch->trace_on != 0), c->P + 1, ch->C, s, params, false,
+                                       ch->by_load));
         } else {
             SIFAR_CUDA(cudaLaunchCooperativeKernel(chain_kernel(ch, ch->trace_on != 0), dim3((unsigned)ch->grid),
                                                    dim3(kChainThreads), params, 0, s));

@@ -153,3 +153,25 @@ def test_the_largest_grids_in_clusters_agree_with_spread_ones(monkeypatch, P, n,
             sf.sifar_chain_destroy(ch)
             results.append(_rows(ring, stride, steps, n, dtype))
     assert results[0][-1].any() and np.array_equal(results[0].view(np.uint8), results[1].view(np.uint8))
+
+
+@pytest.mark.parametrize("P,n,dtype,mode", [
+    (8, 65_537, BF16, sf.DUALBUF), (8, 73_729, BF16, sf.BARRIER_ONESHOT), (4, 131_072, BF16, sf.BARRIER_ONESHOT),
+    (2, 131_071, F32, sf.DUALBUF), (6, 84_001, BF16, sf.SPECULATIVE), (5, 36_864, F32, sf.DUALBUF)])
+def test_all_clusters_of_a_grid_run_at_once(P, n, dtype, mode):
+    """Grids near the largest that go in clusters, placed by load and not: every chunk has started before any has ended."""
+    steps = 64
+    d = synth.chain_workload("llama", P)
+    with Ctx(P, n, dtype) as ctx:
+        ring, _ = _ring(n, dtype, steps)
+        ch = sf.sifar_chain_create(ctx.h, sf.make_workload(**d), n, mode, sf.CHAIN_PERSISTENT, ring.data_ptr(), steps, steps)
+        try:
+            for _ in range(2):
+                sf.sifar_chain_run(ch, 0)
+                torch.cuda.synchronize()
+            stamps = [sf.sifar_chain_chunk_stamps(ch, c, steps) for c in range(sf.sifar_chain_chunks(ch))]
+            assert sf.sifar_chain_geometry(ch)["kernel_clustered"] == 1
+        finally:
+            sf.sifar_chain_destroy(ch)
+        assert sf.sifar_status(ctx.h) == 0
+    assert len(stamps) > 1 and max(s[0] for s in stamps) < min(s[-1] for s in stamps)
