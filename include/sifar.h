@@ -40,9 +40,9 @@
  *                           this many (slot, rank) pairs, wait on a sentinel slot above (320000)
  *   SIFAR_CHAIN_PDL         0 = stream / graph chains record the step events the plain way (by default the
  *                           all-reduce of a step fires its event as soon as all its CTAs have started, and the
- *                           next step's producers wait inside the kernel for its completion; the kernels of a
- *                           speculative graph chain whose steps are left unordered wait for no kernel at all but for
- *                           words that carry the call number), and a run of a
+ *                           next step's producers wait inside the kernel for its completion, or, in a
+ *                           speculative graph chain whose steps are left unordered, for words that carry the call
+ *                           number), and a run of a
  *                           persistent chain in clusters starts when the kernel before it on its stream is over (by
  *                           default its prologue overlaps that kernel's end); read at the first such launch of the
  *                           process

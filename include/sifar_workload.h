@@ -166,6 +166,12 @@ int sifar_chain_geometry(sifar_chain *chain, unsigned out[8]);
  */
 int sifar_chain_trace(sifar_chain *chain, int enable, unsigned long long *phases);
 
+/*
+ * The graph of a GRAPH chain (else SIFAR_ERR_INVALID): out[0] kernel nodes, [1] those of them that are producers waiting
+ * for tagged words only, [2] edges behind the end of a node, [3] edges behind a kernel that lets its dependents in.
+ */
+int sifar_chain_graph_shape(sifar_chain *chain, unsigned out[4]);
+
 /* Kernels launched per run by this chain (graph replays count their kernel nodes). */
 int sifar_chain_launches_per_run(sifar_chain *chain);
 

@@ -90,7 +90,6 @@ struct ReduceArgs {
     uint32_t e_host;         /* the call number the host expects, or 0: take it from device memory   */
     uint32_t pdl;            /* host side only: launch with programmatic stream serialization         */
     uint4 *handoff;          /* slots only: NULL, or where each reduced slot goes once more, with the call number        */
-    uint32_t chained;        /* 1: the stream's kernel before this one is the reducer of the chain's call before     */
     uint32_t let_in;         /* 1: the stream's next kernel may become resident at once, 0: when this grid is done
                                 waiting for its producers (see let_dependents_in)                    */
     uint32_t sweeper;        /* 1: k_sweep follows on the stream: this grid keeps no count and no janitors */
@@ -721,12 +720,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_reduce_spec(const ReduceArgs a)
         }
     }
     __syncthreads();
-    if (a.chained && predecessor_unpublished(a, s_es)) {
-        /* that reducer let this one in when the call before it was published (see below), so it is one short at most */
-        __syncthreads();
-        if (threadIdx.x == 0) s_es.x += 1u;
-        __syncthreads();
-    } else if (!a.e_host && predecessor_unpublished(a, s_es)) {    /* uniform over the CTA */
+    if (!a.e_host && predecessor_unpublished(a, s_es)) {    /* uniform over the CTA */
         /* this context's previous reducer is still running ahead of us on the stream: wait for it and read
            the call number again (what was loaded above is then stale and is loaded again by the validation) */
         gdc_wait();
@@ -746,11 +740,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_reduce_spec(const ReduceArgs a)
             ok = validate_slot<P>(x[u], a.src, s, e, limit_ns, a.poll, reloads);
         }
     }
-    if (alive && ok && !a.chained) let_dependents_in<false>(a);
+    if (alive && ok) let_dependents_in<false>(a);
     if (a.early) gdc_wait();                                /* everything from here on writes */
-    /* in a chain the next reducer tells its call number from the parity of what is published, so the call before this
-       one has to be */
-    if (a.chained) gdc_launch_dependents();
     if (alive) {
         if (ok) {
 #pragma unroll
@@ -1228,7 +1219,6 @@ int launch_reduce(sifar_ctx *ctx, const ReduceLaunch &rl, cudaStream_t stream)
     /* Early reads need programmatic launch to mean anything, and the baseline keeps the plain stream order. */
     a.pdl = ((rl.early || rl.behind) && g_pdl && !rl.programmatic_event) ? 1u : 0u;
     a.handoff = rl.handoff;
-    a.chained = rl.chained ? 1u : 0u;
     a.early = (a.pdl && rl.early && (rl.mode != SIFAR_BARRIER_ONESHOT || g_barrier_early)) ? 1u : 0u;
     /* Are the producers done?  A large plain-format call whose producers run on other streams and have not all
        finished leaves what its grid queues to a sweep kernel of its own (see k_sweep) instead of the grid's janitors;

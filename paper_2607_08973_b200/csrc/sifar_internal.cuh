@@ -145,7 +145,6 @@ struct ReduceLaunch {
     const uint32_t *tile_flags;      /* SIFAR_FORMAT_TILES: the flag array of this call's parity                */
     bool behind;                     /* all producers were enqueued on the reducer's own stream                  */
     uint4 *handoff;                  /* NULL, or where every reduced slot goes once more, with the call number (graph chains) */
-    bool chained;                    /* the kernel before this one on the stream is the reducer of the chain's call before */
     bool early;                      /* the producers are known to run on other streams: reads need not wait for
                                         the kernel before this one on the stream (see the reducer kernels)       */
 };

@@ -173,12 +173,14 @@ __global__ void __launch_bounds__(kProdThreads) k_produce(const ProduceArgs a)
 }
 
 /*
- * Producer kernel of the graph chain in tagged slots (sifar_chain::by_tags): nothing of it waits for a kernel.  A thread
- * polls the previous result of its slots where the reducer hands it over slot by slot (call number in the word), as in the
- * persistent kernels, and stores slots that carry their own tags.  What bounds a step is then these two hops and the two
- * launches, not the ends of kernels: producers and reducers are two rows of programmatic launches that meet in the data
- * alone, each kernel letting the next of its row in once it has what it waits for.  us per 64 steps, by events / by tags:
- * P = 8 bf16 8 KB per rank 223 / 148, 32 KB 270 / 153, 140 KB 325 / 240; P = 2 60 KB 303 / 180; P = 4 fp32 240 KB 359 / 211.
+ * Producer kernel of the graph chain in tagged slots (sifar_chain::by_tags): no data of it waits for the end of a kernel.  A
+ * thread polls the previous result of its slots where the reducer hands it over slot by slot (call number in the word), as in
+ * the persistent kernels, and stores slots that carry their own tags.  A kernel becomes resident when all CTAs of the reducer
+ * that it polls for are (the step's event) and the producers before it have what they waited for, so nothing that polls holds
+ * the place of what it polls for, however many chains share the GPU.  What bounds a step is then the two hops and the end and
+ * the launch of the reducer, whose row is in plain order.  us per 64 steps, with the producers waiting for the reducer's end /
+ * by tags: P = 8 bf16 8 KB per rank 240 / 168, 32 KB 265 / 205, 140 KB 349 / 273; P = 2 60 KB 324 / 207; P = 4 fp32 240 KB
+ * 318 / 238.  Without the order between the rows (8 KB 149, 140 KB 246) the polling kernels of a few chains could fill the GPU.
  * For the slot format up to kConcurrentTiles reducer CTAs (above that a step's reducer is ordered behind its producers).
  */
 template <int DT>
@@ -192,8 +194,8 @@ __global__ void __launch_bounds__(kProdThreads) k_produce_tagged(const ProduceAr
     const size_t nthreads = (size_t)gridDim.x * kProdThreads;
     const size_t n = (size_t)a.n, nslots = (n + NE - 1) / NE;
     __shared__ uint32_t s_e;
-    /* The call number: the first step of a run finds it published; a later one is let in while the calls before it are
-       still on their way and takes it from the step before, which left it before it let this one in. */
+    /* The call number: the first step of a run finds it published; a later one becomes resident while the call before it is
+       still on its way and takes it from the step before, which left it before it let this one in. */
     if (threadIdx.x == 0) {
         uint32_t e = a.opening ? ld_relaxed_u32(&st->epoch) + 1u : ld_relaxed_u32(a.step_word + (a.parity ^ 1u)) + 1u;
         if (ld_relaxed_u32(&st->status) != 0u) e = 0u;
@@ -907,7 +909,7 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
         const uint32_t t = first_t + (uint32_t)s;
         const uint32_t e = ch->base_epoch + t;
         for (int r = 0; r < lanes; ++r) {
-            if (s > 0 && !no_ar && !ch->by_tags) SIFAR_CUDA(cudaStreamWaitEvent(ch->prod[r], ch->ev_step[s - 1], 0));
+            if (s > 0 && !no_ar) SIFAR_CUDA(cudaStreamWaitEvent(ch->prod[r], ch->ev_step[s - 1], 0));
             ProduceArgs a;
             memset(&a, 0, sizeof a);
             a.st = c->d_state; a.host_status = c->d_status_alias; a.timeout_ns = c->timeout_ns;
@@ -950,12 +952,8 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
                out of every step (CUDA-graph chain at 8 KB, P = 8: 7.5 -> 4.9 us per step).  SIFAR_CHAIN_PDL=0
                records the event the plain way. */
             static const bool early = !(getenv("SIFAR_CHAIN_PDL") && atoi(getenv("SIFAR_CHAIN_PDL")) == 0);
-            if (ch->by_tags) {
-                rl.handoff = ch->d_handoff + (size_t)(e & 1u) * ch->handoff_stride;
-                rl.chained = rl.early = s > 0;
-            } else if (early) {
-                rl.programmatic_event = ch->ev_step[s];
-            }
+            if (ch->by_tags) rl.handoff = ch->d_handoff + (size_t)(e & 1u) * ch->handoff_stride;
+            if (early || ch->by_tags) rl.programmatic_event = ch->ev_step[s];
             int rc = launch_reduce(c, rl, ch->red);
             if (rc) return rc;
             if (!early && !ch->by_tags) SIFAR_CUDA(cudaEventRecord(ch->ev_step[s], ch->red));
@@ -1368,6 +1366,32 @@ extern "C" int sifar_chain_trace(sifar_chain *ch, int enable, unsigned long long
         SIFAR_CUDA(cudaMemcpy(phases, ch->d_trace, sizeof(unsigned long long) * ch->steps * kTraceSlots,
                               cudaMemcpyDeviceToHost));
     }
+    return SIFAR_OK;
+}
+
+extern "C" int sifar_chain_graph_shape(sifar_chain *ch, unsigned out[4])
+{
+    if (!ch || !out || ch->impl != SIFAR_CHAIN_GRAPH) { set_error("sifar_chain_graph_shape: not a graph chain"); return SIFAR_ERR_INVALID; }
+    for (int i = 0; i < 4; ++i) out[i] = 0u;
+    size_t nodes = 0, edges = 0;
+    SIFAR_CUDA(cudaGraphGetNodes(ch->graph, nullptr, &nodes));
+    SIFAR_CUDA(cudaGraphGetEdges_v2(ch->graph, nullptr, nullptr, nullptr, &edges));
+    std::vector<cudaGraphNode_t> node(nodes), from(edges), to(edges);
+    std::vector<cudaGraphEdgeData> data(edges);
+    SIFAR_CUDA(cudaGraphGetNodes(ch->graph, node.data(), &nodes));
+    if (edges) SIFAR_CUDA(cudaGraphGetEdges_v2(ch->graph, from.data(), to.data(), data.data(), &edges));
+    for (size_t i = 0; i < nodes; ++i) {
+        cudaGraphNodeType type;
+        SIFAR_CUDA(cudaGraphNodeGetType(node[i], &type));
+        if (type != cudaGraphNodeTypeKernel) continue;
+        ++out[0];
+        cudaKernelNodeParams kp;
+        const cudaError_t known = cudaGraphKernelNodeGetParams(node[i], &kp);
+        if (known == cudaErrorInvalidDeviceFunction) { cudaGetLastError(); continue; }       /* a reducer, of the other library */
+        SIFAR_CUDA(known);
+        if (kp.func == (void *)k_produce_tagged<SIFAR_BF16> || kp.func == (void *)k_produce_tagged<SIFAR_F32>) ++out[1];
+    }
+    for (size_t i = 0; i < edges; ++i) ++out[data[i].from_port == cudaGraphKernelNodePortDefault ? 2 : 3];
     return SIFAR_OK;
 }
 
