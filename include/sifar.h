@@ -35,7 +35,8 @@
  *   SIFAR_CHAIN_HANDOFF_MAX persistent chain: up to this many (unit, rank) pairs a result reaches the next step's
  *                           producers in tagged 16-byte words that each thread polls for itself, above it through one
  *                           ready flag per chunk (170000 speculative, 130000 dual-buffered; not set, speculative chains
- *                           of more than one unit per thread go back to tagged words above 174768)
+ *                           of more than one unit per thread go back to tagged words above 174768, with two ranks in
+ *                           bf16 alone and above 250000, with one rank not at all)
  *   SIFAR_CHAIN_WIDE_MAX    persistent speculative chain with tagged hand-over: re-poll all stale ranks per round up to
  *                           this many (slot, rank) pairs, wait on a sentinel slot above (320000)
  *   SIFAR_CHAIN_PDL         0 = stream / graph chains record the step events the plain way (by default the

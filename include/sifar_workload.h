@@ -144,6 +144,10 @@ int sifar_chain_chunks(sifar_chain *chain);
  */
 int sifar_chain_geometry(sifar_chain *chain, unsigned out[8]);
 
+/* 1 = the kernel of a PERSISTENT chain's last run took the units of a thread in turn, 0 = not, or no run yet (synchronizes
+   the device); a negative status otherwise. */
+int sifar_chain_in_turn(sifar_chain *chain);
+
 /*
  * Phase timeline of the persistent chain (the latency breakdown that stands in for
  * a bandwidth figure at decode payloads).  enable != 0 makes later runs record,

@@ -237,6 +237,7 @@ def _wl() -> ctypes.CDLL:
             "sifar_chain_chunk_stamps": (ci, [vp, ci, ullp]),
             "sifar_chain_chunks": (ci, [vp]),
             "sifar_chain_geometry": (ci, [vp, ctypes.POINTER(ctypes.c_uint)]),
+            "sifar_chain_in_turn": (ci, [vp]),
             "sifar_chain_graph_shape": (ci, [vp, ctypes.POINTER(ctypes.c_uint)]),
             "sifar_chain_launches_per_run": (ci, [vp]),
             "sifar_chain_trace": (ci, [vp, ci, ullp]),
@@ -306,6 +307,13 @@ def sifar_chain_geometry(chain: int) -> dict:
     keys = ("chunks", "units_per_thread", "ctas", "clustered", "tagged", "kernel_clustered", "kernel_cluster_ctas",
             "kernel_tagged")
     return dict(zip(keys, (int(x) for x in out)))
+
+
+def sifar_chain_in_turn(chain: int) -> bool:
+    rc = _wl().sifar_chain_in_turn(chain)
+    if rc < 0:
+        _check(rc)
+    return bool(rc)
 
 
 def sifar_chain_graph_shape(chain: int) -> dict:

@@ -24,9 +24,10 @@ struct __align__(128) ChunkFlags {
 
 struct __align__(128) ChainDev {
     uint32_t exit_count;            /* CTAs that left the kernel (monotonic)                        */
-    uint32_t seen[3];               /* written by CTA 0 of the last run: role layout (1 = clustered), CTAs per
-                                       cluster as the hardware reports them, form of the hand-over (1 = tagged) */
-    uint32_t pad0[28];
+    uint32_t seen[4];               /* written by CTA 0 of the last run: role layout (1 = clustered), CTAs per
+                                       cluster as the hardware reports them, form of the hand-over (1 = tagged),
+                                       [3] by k_chain_pipe alone (1 = units in turn) */
+    uint32_t pad0[27];
 };
 
 struct PersistArgs {

@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kChainThreads, 6) k_chain_pipe(const PersistAr
     /* the seeded halves of the next step, by unit */
     __shared__ float s_z[kPipeParked][NE][kChainThreads];
     __shared__ int s_last;
-    if (blockIdx.x == 0 && threadIdx.x == 0) { a.cs->seen[0] = 0u; a.cs->seen[1] = 1u; a.cs->seen[2] = 1u; }
+    if (blockIdx.x == 0 && threadIdx.x == 0) { a.cs->seen[0] = 0u; a.cs->seen[1] = 1u; a.cs->seen[2] = 1u; a.cs->seen[3] = 1u; }
     unsigned reloads = 0;
     unsigned long long *my_stamps = a.stamps + ((size_t)chunk * kPipeWarps + warp) * (a.steps + 1u);
     const bool stamper = is_reader && lane == 0u;

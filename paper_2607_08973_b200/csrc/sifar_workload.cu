@@ -361,6 +361,21 @@ constexpr bool cluster_by_load(int mode, int P, int dtype, size_t ctas, size_t s
  */
 constexpr size_t kPipeMinPairs = 174768;
 /*
+ * ... where taking turns pays: a thread has to have enough to do between two looks.  With one or two ranks, and in fp32, whose
+ * units have half the arithmetic, with three and five near the first size of two units per thread, it polls instead, and the
+ * polls get in the way of the stores.  us per 64 steps, k_chain / k_chain_pipe: P = 1 bf16 700 KB 192 / 269, 1.6 MB 304 / 404, fp32
+ * 1 MB 157 / 264; P = 2 bf16 447 KB 168 / 228, 512 KB 196 / 276, 1.3 MB (221 866 pairs) 381 / 435, 1.6 MB (273 066) 499 / 389, fp32
+ * 620 KB 151 / 259, 1.6 MB 333 / 434, 2 MB 381 / 400; P = 3 fp32 395 KB 151 / 223, 512 KB 159 / 200, 620 KB 186 / 229, 700 KB (179 196)
+ * 289 / 232; P = 5 fp32 226 KB 146 / 171, 252 KB (107 515) 146 / 180, 265 KB (113 060) 146 / 132.
+ */
+constexpr bool pipe_pays(int P, int dtype, size_t pairs)
+{
+    constexpr size_t never = SIZE_MAX;
+    constexpr size_t line[2][9] = {{0, never, 250000, 0, 0, 0, 0, 0, 0},                            /* bf16, by P */
+                                   {0, never, never, 170000, 0, 110000, 0, 0, 0}};
+    return line[dtype == SIFAR_BF16 ? 0 : 1][P] != never && pairs > line[dtype == SIFAR_BF16 ? 0 : 1][P];
+}
+/*
  * Its readers (and k_chain's with tagged words) poll all stale ranks of their own slots up to this many pairs and wait on a
  * sentinel slot per rank above.  Sentinel / wide: P = 8 bf16 240 KB 221 / 207, 384 KB (262 144 pairs) 371 / 366, 512 KB
  * (349 528) 425 / 465; fp32 480 KB (320 008) 280 / 280.
@@ -1100,7 +1115,8 @@ static int chain_setup_persistent(sifar_chain *ch)
         int rc = chain_spread(ch, units, roles, &ch->K, &ch->C);
         if (rc) return rc;
         if (ch->K > 1 && ch->mode == SIFAR_SPECULATIVE &&
-            (ch->tagged || (!env_handoff && units * (size_t)c->P > kPipeMinPairs)) && (rc = chain_take_in_turn(ch, units, roles)))
+            (ch->tagged || (!env_handoff && units * (size_t)c->P > kPipeMinPairs)) &&
+            pipe_pays(c->P, c->dtype, units * (size_t)c->P) && (rc = chain_take_in_turn(ch, units, roles)))
             return rc;
         if (ch->K > 1 && (ch->mode == SIFAR_BARRIER_ONESHOT || ch->mode == SIFAR_DUALBUF)) {
             uint32_t K, C;
@@ -1342,6 +1358,15 @@ extern "C" int sifar_chain_geometry(sifar_chain *ch, unsigned out[8])
     out[3] = (ch->cluster_kernel || ch->placed) ? 1u : 0u; out[4] = ch->tagged ? 1u : 0u;
     out[5] = h.seen[0]; out[6] = h.seen[1]; out[7] = h.seen[2];
     return SIFAR_OK;
+}
+
+extern "C" int sifar_chain_in_turn(sifar_chain *ch)
+{
+    if (!ch || ch->impl != SIFAR_CHAIN_PERSISTENT) { set_error("sifar_chain_in_turn: needs a persistent chain"); return SIFAR_ERR_INVALID; }
+    ChainDev h;
+    SIFAR_CUDA(cudaDeviceSynchronize());
+    SIFAR_CUDA(cudaMemcpy(&h, ch->d_cs, sizeof h, cudaMemcpyDeviceToHost));
+    return h.seen[3] ? 1 : 0;
 }
 
 extern "C" int sifar_chain_trace(sifar_chain *ch, int enable, unsigned long long *phases)
