@@ -45,8 +45,8 @@
  *                           speculative graph chain whose steps are left unordered, for words that carry the call
  *                           number), and a run of a
  *                           persistent chain in clusters starts when the kernel before it on its stream is over (by
- *                           default its prologue overlaps that kernel's end); read at the first such launch of the
- *                           process
+ *                           default its prologue overlaps that kernel's end); read once, when the process creates its
+ *                           first graph chain or first launches one of the others
  *   SIFAR_PDL               0 = every kernel of libsifar.so is launched without programmatic dependent launch (read
  *                           when the library is loaded).  By default a kernel of one of these kinds may become
  *                           resident while the kernel before it on its stream drains: a reducer with more CTAs than

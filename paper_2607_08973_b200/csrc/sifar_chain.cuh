@@ -190,6 +190,8 @@ const void *sym_cluster_kernel(int dtype, int P, int mode);
 /* The speculative chain whose threads take several units in turn (sifar_chain_pipe.cu), and how many at most. */
 constexpr uint32_t kPipeParked = 8;
 const void *chain_pipe_kernel(int dtype, int P, bool trace);
+/* false: SIFAR_CHAIN_PDL=0 when this was first asked for */
+bool chain_dependent_launches();
 /* Can the device hold `clusters` clusters of `cluster` CTAs of the kernel at once? */
 bool cluster_fits(const void *kernel, int cluster, size_t clusters);
 /* `dependent`: the kernel does a prologue of its own and then waits for what precedes it on the stream.  `by_load`: the

@@ -597,17 +597,22 @@ bool cluster_fits(const void *kernel, int cluster, size_t clusters)
     return (size_t)most >= clusters;
 }
 
+bool chain_dependent_launches()
+{
+    static const bool on = !(getenv("SIFAR_CHAIN_PDL") && atoi(getenv("SIFAR_CHAIN_PDL")) == 0);
+    return on;
+}
+
 cudaError_t launch_clusters(const void *kernel, int cluster, size_t clusters, cudaStream_t stream, void **params, bool dependent,
                             bool by_load)
 {
-    static const bool early = !(getenv("SIFAR_CHAIN_PDL") && atoi(getenv("SIFAR_CHAIN_PDL")) == 0);
     cudaLaunchAttribute attr[3];
     cudaLaunchConfig_t cfg = cluster_config(attr, cluster, clusters, kChainThreads, stream);
     if (by_load) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeClusterSchedulingPolicyPreference;
         attr[cfg.numAttrs++].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
     }
-    if (dependent && early) {
+    if (dependent && chain_dependent_launches()) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }

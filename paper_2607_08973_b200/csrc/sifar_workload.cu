@@ -966,12 +966,12 @@ static int enqueue_run(sifar_chain *ch, cudaStream_t origin, uint32_t first_t)
                for its completion before they read anything.  This takes the launch latency of the producers
                out of every step (CUDA-graph chain at 8 KB, P = 8: 7.5 -> 4.9 us per step).  SIFAR_CHAIN_PDL=0
                records the event the plain way. */
-            static const bool early = !(getenv("SIFAR_CHAIN_PDL") && atoi(getenv("SIFAR_CHAIN_PDL")) == 0);
+            const bool early = chain_dependent_launches();
             if (ch->by_tags) rl.handoff = ch->d_handoff + (size_t)(e & 1u) * ch->handoff_stride;
-            if (early || ch->by_tags) rl.programmatic_event = ch->ev_step[s];
+            if (early) rl.programmatic_event = ch->ev_step[s];
             int rc = launch_reduce(c, rl, ch->red);
             if (rc) return rc;
-            if (!early && !ch->by_tags) SIFAR_CUDA(cudaEventRecord(ch->ev_step[s], ch->red));
+            if (!early) SIFAR_CUDA(cudaEventRecord(ch->ev_step[s], ch->red));
         }
     }
     for (int r = 0; r < lanes; ++r) {
@@ -1194,9 +1194,8 @@ extern "C" sifar_chain *sifar_chain_create(sifar_ctx *c, const sifar_workload *w
         for (int r = 0; r <= c->P; ++r) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_join[r], cudaEventDisableTiming));
         for (int r = 0; r < c->P; ++r) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_prod[r], cudaEventDisableTiming));
         ch->concurrent = reduce_tiles(c, n, mode == kModeNoAllreduce ? SIFAR_DUALBUF : mode) <= kConcurrentTiles;
-        const char *env_pdl = getenv("SIFAR_CHAIN_PDL");
         ch->by_tags = impl == SIFAR_CHAIN_GRAPH && mode == SIFAR_SPECULATIVE && ch->concurrent && dependent_launches() &&
-                      !(env_pdl && atoi(env_pdl) == 0);
+                      chain_dependent_launches();
         if (ch->by_tags) {
             ch->handoff_stride = slots_for(c->dtype, n);
             /* the words of both parities, then the step words; zero = call number 0 = never valid */

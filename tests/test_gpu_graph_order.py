@@ -55,3 +55,17 @@ def test_several_chains_at_once(oracle, chains, P, n, dtype):
         want = oracle.chain(_oracle_w(oracle, d), P, n, dtype, steps * runs)
         for t in range(steps):
             assert_bits_equal(got[i][t], want[(runs - 1) * steps + t], dtype, f"chain {i} step {(runs - 1) * steps + t + 1}")
+
+
+def test_the_environment_is_read_once(monkeypatch):
+    """SIFAR_CHAIN_PDL, set after the first chain, changes neither the form nor the order of a later one."""
+    P, n, steps = 8, 4096, 6
+    shapes = []
+    with Ctx(P, n, BF16) as ctx:
+        for env in (None, "0"):
+            if env is not None:
+                monkeypatch.setenv("SIFAR_CHAIN_PDL", env)
+            ch, _, _ = _create(ctx, synth.chain_workload("llama", P), n, BF16, steps)
+            shapes.append(sf.sifar_chain_graph_shape(ch))
+            sf.sifar_chain_destroy(ch)
+    assert shapes[0] == shapes[1] and shapes[0]["tagged_producers"] == steps
