@@ -1194,8 +1194,10 @@ extern "C" sifar_chain *sifar_chain_create(sifar_ctx *c, const sifar_workload *w
         for (int r = 0; r <= c->P; ++r) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_join[r], cudaEventDisableTiming));
         for (int r = 0; r < c->P; ++r) SIFAR_CUDA(cudaEventCreateWithFlags(&ch->ev_prod[r], cudaEventDisableTiming));
         ch->concurrent = reduce_tiles(c, n, mode == kModeNoAllreduce ? SIFAR_DUALBUF : mode) <= kConcurrentTiles;
+        /* By tags only where no reducer CTA can leave its tile to another: what a janitor sums is not handed over in words.
+           (launch_reduce defers above one CTA per SM, which takes a GPU of fewer than kConcurrentTiles SMs.) */
         ch->by_tags = impl == SIFAR_CHAIN_GRAPH && mode == SIFAR_SPECULATIVE && ch->concurrent && dependent_launches() &&
-                      chain_dependent_launches();
+                      chain_dependent_launches() && reduce_tiles(c, n, mode) <= (size_t)c->sm_count;
         if (ch->by_tags) {
             ch->handoff_stride = slots_for(c->dtype, n);
             /* the words of both parities, then the step words; zero = call number 0 = never valid */
