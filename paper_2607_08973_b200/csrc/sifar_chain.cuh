@@ -70,9 +70,9 @@ struct PersistArgs {
  * do in the speculative mode: data and call number in one 16-byte store, validated by the reader, who polls the
  * unit it needs and nothing else - no CTA-wide barrier, no fence, no flag, no second round trip for the data.
  * The other form, one ready flag per chunk (barrier, release; acquire poll by thread 0, barrier, then the loads),
- * costs 0.3-2 us more per step up to 128 KB per rank at P = 8; it is kept for large grids (handoff_max_pairs), where
- * eight times as many threads polling data lines as there are units slow the reducers' stores by as much as the flag
- * costs.  With both barriers neither form is needed: the done flags
+ * costs 0.3-2 us more per step up to 128 KB per rank at P = 8; it is kept for large dual-buffered grids (handoff_max_pairs),
+ * where eight times as many threads polling data lines as there are units slow the reducers' stores by as much as the
+ * flag costs, and for the large speculative ones that do not run k_chain_pipe (pipe_pays).  With both barriers neither form is needed: the done flags
  * of the bottom barrier follow the result stores.  The chain without all-reduce uses the words too: every rank
  * hands its partial to itself.
  * NW = 3 result words (a 12-byte unit: speculative mode, chain without all-reduce): {w0, w1, w2, tag}.  NW = 4

@@ -13,8 +13,9 @@
  * P tags is one word.
  * Readers have fewer units per thread than producers where there is room (their trip per unit, about 1800 cycles under
  * load, is what a reader waits for and does little in), but not one alone: a reader needs something to do while it waits
- * (P = 8, 240 KB per rank, 1 / 2 units per reader thread: 263 / 227 us; 512 KB, 4 / 2: 953 / 887 per 120 steps).
- * us per 120 steps at P = 8, bf16, 512 KB per rank: k_chain 1007, this kernel 784; other sizes at kPipeMinPairs.
+ * (P = 8: at 240 KB per rank two units per reader thread took 14 % less time than one, at 512 KB 7 % less than four).
+ * us per 120 steps at P = 8, bf16, 512 KB per rank: k_chain 1007, this kernel 787; other sizes at kPipeMinPairs, and where few
+ * ranks give a thread too little to do, at pipe_pays().
  */
 #include "sifar_internal.cuh"
 #ifdef SIFAR_SLOT_S8X2

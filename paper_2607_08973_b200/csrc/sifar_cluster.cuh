@@ -148,8 +148,8 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v)
     asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
 }
 
-/* Time limit of a loop that polls shared memory: a poll takes some 30 cycles, so the clock is read on every 64th and
-   the context's status looked at on every 1024th. */
+/* Time limit of a loop that polls shared memory: a poll takes some 30 cycles, 20 ns more in take_box_slots, so the clock is
+   read on every 64th (after 1 to 3 us) and the context's status looked at on every 1024th (after 16 to 40 us). */
 struct LocalDeadline {
     unsigned long long t0 = 0;
     unsigned polls = 0;
@@ -176,7 +176,8 @@ constexpr uint32_t kBoxStride = kBoxThreads + 1;
  * again until they are (a sender's warp stores its 32 slots with one instruction, so that is rare).  Polling one word
  * per rank instead of P slots per lane leaves the shared-memory ports to the arriving stores, and the pause between two
  * looks leaves issue slots to the warps that compute (one reader, P = 8, 64 steps: 8 KB 63.9 -> 62.2 us, 32 KB 82.1 ->
- * 79.2; a pause of 100 ns, or one in the producers' polls too, is slower).  `reloads` counts looks
+ * 79.2; P = 3 fp32 4 KB 51.3 -> 49.1; P = 1 level, 1 us either way by size; a pause of 100 ns, or one in the producers' polls
+ * too, is slower).  `reloads` counts looks
  * that found a stale slot.  False (on all lanes): time limit, or somebody has failed.
  */
 template <int P>

@@ -78,7 +78,8 @@ __device__ __forceinline__ bool wait_flag_or_fail(const uint32_t *flag, uint32_t
  * acc + the low / high bf16 half of a word: the half is widened inside the add (one correctly rounded binary32 add, as
  * with a separate widening).  A separate widening is a shift or a mask on the integer pipe, which issues every other
  * cycle and bounds the large chains: 1.26 cycles per add and scheduler against 2.5 with a shift.  The chain of 8 KB steps,
- * P = 8: 65.1 -> 62.9 us per 64; clusters with both barriers 115.1 -> 112.6 at 32 KB; bandwidth-bound reducers level.
+ * P = 8: 65.1 -> 62.9 us per 64; clusters with both barriers 115.1 -> 112.6 at 32 KB,
+ * dual-buffered 72.2 -> 70.8 at 40 KB, but 93 -> 96..100 at 61 to 82 KB (P = 8 alone); bandwidth-bound reducers level.
  */
 __device__ __forceinline__ float add_bf16lo(float acc, uint32_t w)
 {

@@ -307,7 +307,7 @@ __global__ void k_store_blocks(const void *src, void *dst, uint32_t *flags, unsi
  * 252, 512 KB (131 072) 287 / 352: the line is where the forms cross.  Speculative, flag / tagged with sentinel / tagged
  * and wide: P = 8 bf16 128 KB 252 / 191 / 155, 192 KB 301 / 214 / 211, 256 KB (174 768) 330 / 285 / 293, 512 KB 545 / 539 /
  * 558; P = 8 fp32 256 KB 299 / 195 / 190, 512 KB 417 / 352 / 346; P = 4 bf16 512 KB 321 / 283 / 280: the tagged form stays
- * ahead of the flag above this line too; what is above runs k_chain_pipe (kPipeMinPairs).
+ * ahead of the flag above this line too; what is above runs k_chain_pipe (kPipeMinPairs) where pipe_pays().
  */
 constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE ? 170000 : 130000; }
 /*
@@ -316,8 +316,11 @@ constexpr size_t handoff_max_pairs(int mode) { return mode == SIFAR_SPECULATIVE 
  * (see k_chain) up to kPlacedMaxPairs.  us per run of 64 steps, shared memory against spread over the machine.
  * Modes with flags: ahead wherever they fit.  P = 8 bf16 dual-buffered 8 KB per rank 57 / 170, 64 KB 94 / 203, 129 KB 150 / 221,
  * 146 KB 163 / 235, both barriers 104 / 220, 132 / 232, 197 / 248, 199 / 257; P = 7 152 KB 138 / 225 and 177 / 249; P = 4 256 KB
- * 134 / 215 and 140 / 250; P = 2 508 KB 147 / 216 and 158 / 248.  With eight ranks 128 KB (65 536 pairs) is documented and
- * tested as the first payload that spreads; the sizes around it do not.
+ * 134 / 215 and 140 / 250; P = 2 508 KB 147 / 216 and 158 / 248; P = 3 415 KB 152 / 223 and 162 / 254; P = 5 270 KB 154 / 232 and
+ * 168 / 265; P = 6 212 KB 151 / 235 and 173 / 259; fp32 P = 3 473 KB 100 / 233 and 123 / 241, P = 4 386 KB 116 / 238 and 152 / 243, P = 5
+ * 299 KB 138 / 234 and 180 / 246, P = 8 183 KB 178 / 238 dual-buffered; with one rank every payload up to 512 KB fits.  With eight
+ * ranks 65 001 to 65 536 pairs spread although clusters are faster there too (128 KB 220, 127 and 129 KB 138-150): that 128 KB is the
+ * first payload to spread is documented, and tests hold it.
  * Speculative: a chunk's one reader CTA takes and sends P vectors per thread through its SM's ports, and its lanes poll; with
  * seven or eight ranks and more than about 30 clusters that costs more than the hop saves (P = 8 bf16 24 KB 74 / 83, 32 KB
  * 82 / 84, 40 KB 86 / 85, 72 KB 121 / 112; fp32 32 KB 80 / 79, 64 KB 112 / 84; P = 7 bf16 56 KB 87 / 94, 72 KB 104 / 98).
@@ -353,8 +356,9 @@ constexpr bool cluster_by_load(int mode, int P, int dtype, size_t ctas, size_t s
 }
 /*
  * Speculative grids whose threads take more than one unit run k_chain_pipe (sifar_chain_pipe.cu) with tagged words, up to
- * the hand-over's line and again above this one; in between lies 256 KB per rank at P = 8 (174 768 pairs), which is
- * documented and tested as the first payload by ready flag.  us per 64 steps, k_chain / k_chain_pipe: P = 8 bf16 160 KB per
+ * the hand-over's line and again above this one; in between k_chain with the ready flag, although it is slower there too
+ * (P = 8 fp32 252 KB 303 against 157 at 265 KB): that 256 KB per rank at P = 8 (174 768 pairs) is the first payload by ready
+ * flag is documented, and a test holds it.  us per 64 steps, k_chain / k_chain_pipe: P = 8 bf16 160 KB per
  * rank 206 / 176, 240 KB 255 / 207, 320 KB 378 / 302, 384 KB 418 / 366, 512 KB 544 / 425; P = 8 fp32 180 KB 150 / 138, 300 KB
  * 305 / 161, 480 KB 407 / 280; P = 4 bf16 360 KB 216 / 177; P = 6 400 KB 364 / 286.  With one unit per thread k_chain is
  * level or ahead (P = 8 80 KB 122 / 128, P = 4 300 KB 165 / 201).
